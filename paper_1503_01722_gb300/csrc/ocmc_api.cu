@@ -219,12 +219,21 @@ void ctx_launch_shape(const ocmc_ctx* c, int* threads, int* blocks, int* cap, in
     launch_shape(c, threads, blocks, cap, nreg);
 }
 
-ocmc_status ctx_ensure_stacks(ocmc_ctx* c, size_t need)
+ocmc_status ctx_ensure_stacks(ocmc_ctx* c, size_t warps, size_t records_per_warp)
 {
-    if (need > c->stack_records) {
+    const size_t need = warps * records_per_warp;
+    if (need > c->stack_records || warps > c->left_warps) {
         if (c->ran || c->last_stream) cudaDeviceSynchronize();
-        CK(dalloc(&c->d_stacks, need), "stack allocation");
-        c->stack_records = need;
+        if (need > c->stack_records) {
+            c->stack_records = 0;
+            CK(dalloc(&c->d_stacks, need), "stack allocation");
+            c->stack_records = need;
+        }
+        if (warps > c->left_warps) {
+            c->left_warps = 0;
+            CK(dalloc(&c->d_left, warps), "stack allocation");
+            c->left_warps = warps;
+        }
     }
     return OCMC_OK;
 }
@@ -325,7 +334,7 @@ ocmc_status ocmc_init(ocmc_ctx** out, int device, const ocmc_params* p)
         c->t.n_mat = NMAT_DEFAULT;
     }
     if (r == cudaSuccess) r = dalloc(&c->d_stats, ST_COUNT);
-    if (r == cudaSuccess) r = dalloc(&c->d_counter, 1);
+    if (r == cudaSuccess) r = dalloc(&c->d_counter, RUN_COUNTERS);
     if (r == cudaSuccess) r = dalloc(&c->d_sum, 1);
     if (r == cudaSuccess) r = dalloc(&c->d_err, 1);
     if (r == cudaSuccess) r = cudaMemset(c->d_stats, 0, ST_COUNT * sizeof(unsigned long long));
@@ -585,12 +594,9 @@ ocmc_status ocmc_run_range(ocmc_ctx* c, uint64_t first, uint64_t count, uint64_t
     int threads, blocks, cap, nreg;
     launch_shape(c, &threads, &blocks, &cap, &nreg);
     const int nstk = c->p.e_class_split > 0.f ? 3 : 2;
-    size_t need = (size_t)blocks * (threads / 32) * nstk * cap;
-    if (need > c->stack_records) {
-        if (c->ran || c->last_stream) cudaDeviceSynchronize();
-        CK(dalloc(&c->d_stacks, need), "stack allocation");
-        c->stack_records = need;
-    }
+    const int warps = blocks * (threads / 32);
+    st = ctx_ensure_stacks(c, (size_t)warps, (size_t)nstk * cap);
+    if (st != OCMC_OK) return st;
     TransportArgs a;
     fill_args(c, a);
     if (c->src_kind == 0) stratify(c, n_total, a.src);
@@ -600,6 +606,7 @@ ocmc_status ocmc_run_range(ocmc_ctx* c, uint64_t first, uint64_t count, uint64_t
     a.key0 = (uint32_t)seed;
     a.key1 = (uint32_t)(seed >> 32);
     a.stacks = c->d_stacks;
+    a.left_out = c->d_left;
     a.cap = cap;
     a.nstk = nstk;
     a.e_split = c->p.e_class_split;
@@ -613,7 +620,7 @@ ocmc_status ocmc_run_range(ocmc_ctx* c, uint64_t first, uint64_t count, uint64_t
     for (uint64_t done = 0; done < count; done += RUN_CHUNK) {
         a.first = first + done;
         a.count = std::min<uint64_t>(RUN_CHUNK, count - done);
-        CK(cudaMemsetAsync(c->d_counter, 0, sizeof(unsigned long long), s), "counter reset");
+        CK(cudaMemsetAsync(c->d_counter, 0, RUN_COUNTERS * sizeof(unsigned long long), s), "counter reset");
         CK(launch_transport(a, blocks, threads, transport_smem_bytes(c->t.n_mat), s, nreg), "transport launch");
     }
     CK(cudaEventRecord(c->ev1, s), "event");
@@ -796,7 +803,7 @@ void ocmc_destroy(ocmc_ctx* c)
     cudaSetDevice(c->device);
     cudaDeviceSynchronize();
     dfree(&c->d_density); dfree(&c->d_material); dfree(&c->d_tally); dfree(&c->d_stats);
-    dfree(&c->d_counter); dfree(&c->d_sum); dfree(&c->d_err); dfree(&c->d_stacks); dfree(&c->d_dose);
+    dfree(&c->d_counter); dfree(&c->d_sum); dfree(&c->d_err); dfree(&c->d_stacks); dfree(&c->d_left); dfree(&c->d_dose);
     dfree(&c->d_sigma); dfree(&c->d_invnb);
     dfree(&c->t.ph); dfree(&c->t.el); dfree(&c->t.el2); dfree(&c->t.phmaj); dfree(&c->t.elmaj); dfree(&c->t.rinv); dfree(&c->t.msA);
     dfree(&c->t.rmeta); dfree(&c->t.msc); dfree(&c->t.scratch); dfree(&c->t.rho_max);

@@ -99,7 +99,7 @@ __global__ void k_test_sample(const TransportArgs a, int kind, int m, float E, f
     for (unsigned long long j = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; j < n;
          j += (unsigned long long)gridDim.x * blockDim.x) {
         Rng r;
-        r.h0 = (uint32_t)j; r.h1 = (uint32_t)(j >> 32); r.sub = 0x5A5Au + (uint32_t)kind; r.n = 0; r.blk = 0xFFFFFFFFu;
+        r.h0 = (uint32_t)j; r.h1 = (uint32_t)(j >> 32); r.sub = 0x5A5Au + (uint32_t)kind; r.n = 0;
         bool ok = true;
         float v = 0.f, eps;
         if (kind == 0) v = sample_compton(E, r, a.key0, a.key1, &eps, &ok);

@@ -105,9 +105,10 @@ ocmc_status beamlet_args(ocmc_ctx* c, unsigned long long total, uint64_t seed, T
     int cap;
     ctx_launch_shape(c, threads, blocks, &cap, nreg);
     const int nstk = c->p.e_class_split > 0.f ? 3 : 2;
-    ocmc_status st = ctx_ensure_stacks(c, (size_t)*blocks * (*threads / 32) * nstk * cap);
+    ocmc_status st = ctx_ensure_stacks(c, (size_t)*blocks * (*threads / 32), (size_t)nstk * cap);
     if (st != OCMC_OK) return st;
     a.stacks = c->d_stacks;
+    a.left_out = c->d_left;
     a.cap = cap;
     a.nstk = nstk;
     a.e_split = c->p.e_class_split;
@@ -124,7 +125,7 @@ cudaError_t enqueue_beamlets(ocmc_ctx* c, const TransportArgs& a, size_t slots, 
     cudaError_t e = cudaMemsetAsync(c->d_bl_keys, 0xFF, sizeof(unsigned int) * slots, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_bl_vals, 0, sizeof(unsigned long long) * slots, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_bl_over, 0, sizeof(unsigned int) * c->bl_n, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->d_counter, 0, sizeof(unsigned long long), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->d_counter, 0, RUN_COUNTERS * sizeof(unsigned long long), s);
     // a beamlet run replaces its tallies, so its statistics describe that run alone
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_stats, 0, sizeof(unsigned long long) * ST_COUNT, s);
     if (e == cudaSuccess) e = launch_transport(a, blocks, threads, transport_smem_bytes(c->t.n_mat), s, nreg);

@@ -51,6 +51,8 @@ struct ocmc_ctx {
     int* d_err = nullptr;
     ocmc::PRec* d_stacks = nullptr;
     size_t stack_records = 0;
+    int* d_left = nullptr;          // per warp: photons left to k_chains
+    size_t left_warps = 0;
     // outputs
     float* d_dose = nullptr;
     float* d_sigma = nullptr;
@@ -94,7 +96,7 @@ ocmc_status ctx_cuda_fail(ocmc_ctx* c, cudaError_t e, const char* where);
 ocmc_status ctx_ensure_tables(ocmc_ctx* c, cudaStream_t s);
 void ctx_fill_args(const ocmc_ctx* c, TransportArgs& a);
 void ctx_launch_shape(const ocmc_ctx* c, int* threads, int* blocks, int* cap, int* nreg);
-ocmc_status ctx_ensure_stacks(ocmc_ctx* c, size_t records);
+ocmc_status ctx_ensure_stacks(ocmc_ctx* c, size_t warps, size_t records_per_warp);
 void stratify_bins(const float* edges, const float* weights, int n_bins, unsigned long long N, int* order,
                    unsigned long long* bound);
 void beam_frame(const float dir[3], float d[3], float e1[3], float e2[3]);

@@ -24,8 +24,9 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1
 // key = the run's seed. Draw n is word n mod 4 of that block, mapped to
 // ((x >> 8) + 1) 2^-24 in (0, 1]. The stream depends only on the particle, never
 // on the thread that transports it, so the dose is independent of scheduling.
+// buf holds block n/4 while n is inside it; a draw at a block's first word generates the block.
 struct Rng {
-    uint32_t h0, h1, sub, n, blk;
+    uint32_t h0, h1, sub, n;
     uint4 buf;
 };
 
@@ -43,21 +44,19 @@ static __device__ __noinline__ uint4 philox_block(uint32_t b, uint32_t h0, uint3
 __device__ __forceinline__ void rng_step_start(Rng& r, uint32_t k0, uint32_t k1)
 {
     r.n = (r.n + 3u) & ~3u;
-    r.blk = r.n >> 2;
-    r.buf = philox4x32_10(make_uint4(r.blk, r.h0, r.h1, r.sub), k0, k1);
+    r.buf = philox4x32_10(make_uint4(r.n >> 2, r.h0, r.h1, r.sub), k0, k1);
 }
 
+__device__ __forceinline__ float u01(uint32_t x) { return (float)((x >> 8) + 1u) * 5.9604644775390625e-08f; }
+
+// The next draw. After rng_step_start the caller takes the block's first draws from buf itself (u01)
+// and advances n past them, at least by one, before it calls this.
 __device__ __forceinline__ float rng_u(Rng& r, uint32_t k0, uint32_t k1)
 {
-    uint32_t b = r.n >> 2;
-    if (b != r.blk) {
-        r.buf = philox_block(b, r.h0, r.h1, r.sub, k0, k1);
-        r.blk = b;
-    }
-    uint32_t i = r.n & 3u;
+    const uint32_t i = r.n & 3u;
+    if (i == 0u) r.buf = philox_block(r.n >> 2, r.h0, r.h1, r.sub, k0, k1);
     r.n++;
-    uint32_t x = i == 0 ? r.buf.x : (i == 1 ? r.buf.y : (i == 2 ? r.buf.z : r.buf.w));
-    return (float)((x >> 8) + 1u) * 5.9604644775390625e-08f;
+    return u01(i == 0u ? r.buf.x : (i == 1u ? r.buf.y : (i == 2u ? r.buf.z : r.buf.w)));
 }
 
 __device__ __forceinline__ uint32_t child_sub(uint32_t parent, uint32_t n, uint32_t slot)
@@ -142,12 +141,15 @@ __device__ __forceinline__ float sample_compton(float E, Rng& r, uint32_t k0, ui
     float k = E / MC2F;
     float e0 = 1.f / (1.f + 2.f * k);
     float a1 = __logf(1.f + 2.f * k);
-    float a2 = 0.5f * (1.f - e0 * e0);
+    // explicitly rounded: products that the compiler might contract one way in one instantiation of
+    // the transport kernel and another way in the next are written out, here and in photon_step
+    const float e02 = __fmul_rn(e0, e0), d02 = __fsub_rn(1.f, e02);
+    float a2 = 0.5f * d02;
     float eps = 1.f, t = 0.f;
     for (int it = 0; it < SAMPLE_LIMIT; ++it) {
         float r1 = rng_u(r, k0, k1), r2 = rng_u(r, k0, k1), r3 = rng_u(r, k0, k1);
         if (r1 * (a1 + a2) < a1) eps = __expf(-a1 * r2);
-        else eps = sqrtf(e0 * e0 + (1.f - e0 * e0) * r2);
+        else eps = sqrtf(__fmaf_rn(d02, r2, e02));
         eps = fminf(fmaxf(eps, e0), 1.f);
         t = (1.f - eps) / (k * eps);
         float s2 = t * (2.f - t);
@@ -201,10 +203,10 @@ __device__ __forceinline__ float sample_brems(float T, float wcb, float S1, floa
 
 // Multiple-scattering cos(theta) for G1 = s / lambda_1: Wentzel distribution with
 // screening A chosen so that <1 - cos> = 1 - exp(-G1) (table of ln A at ln G1).
-__device__ __forceinline__ float sample_ms(const SmemTables& T, float G1, Rng& r, uint32_t k0, uint32_t k1)
+// sample_ms_u takes its draw as an argument (unused below G1 = 1e-12).
+__device__ __forceinline__ float sample_ms_u(const SmemTables& T, float G1, float xi)
 {
     if (!(G1 >= 1e-12f)) return 1.f;
-    float xi = rng_u(r, k0, k1);
     if (G1 >= 15.f) return 2.f * xi - 1.f;
     float x = (__logf(G1) - LN_G_LO) * INV_DLNG;
     x = fminf(fmaxf(x, 0.f), (float)(NG - 1) - 1e-3f);
@@ -213,6 +215,11 @@ __device__ __forceinline__ float sample_ms(const SmemTables& T, float G1, Rng& r
     float q = 1.f - xi;                              // [0, 1)
     float u = 2.f * A * q / (1.f + A - q);
     return fmaxf(-1.f, 1.f - u);
+}
+
+__device__ __forceinline__ float sample_ms(const SmemTables& T, float G1, Rng& r, uint32_t k0, uint32_t k1)
+{
+    return sample_ms_u(T, G1, G1 >= 1e-12f ? rng_u(r, k0, k1) : 0.f);
 }
 
 // The GPU's global nanosecond timer (consistent across SMs).
@@ -236,16 +243,13 @@ __device__ __forceinline__ void rotate(float& u, float& v, float& w, float mu, f
     // across launch shapes.
     const float s2 = __fmaf_rn(u, u, __fmul_rn(v, v));
     const float is = rsqrtf(s2), s = __fmul_rn(s2, is);
-    float nu, nv, nw;
-    if (s2 > 1e-20f) {
-        nu = u * mu + st * (u * w * cp - v * sp) * is;
-        nv = v * mu + st * (v * w * cp + u * sp) * is;
-        nw = w * mu - s * st * cp;
-    } else {
-        float sg = w >= 0.f ? 1.f : -1.f;
+    float nu = u * mu + st * (u * w * cp - v * sp) * is;
+    float nv = v * mu + st * (v * w * cp + u * sp) * is;
+    float nw = w * mu - s * st * cp;
+    if (!(s2 > 1e-20f)) {                        // along the pole: a few selects, no branch
         nu = st * cp;
         nv = st * sp;
-        nw = sg * mu;
+        nw = w >= 0.f ? mu : -mu;
     }
     float inv = rsqrtf(nu * nu + nv * nv + nw * nw);
     u = nu * inv;
@@ -255,25 +259,24 @@ __device__ __forceinline__ void rotate(float& u, float& v, float& w, float mu, f
 
 // ---- voxel geometry -----------------------------------------------------------------------
 // Distance from (x,y,z) along (u,v,w) to the faces of voxel (ix,iy,iz);
-// *face = axis*2 + (direction > 0).
+// *face = axis*2 + (direction > 0). No branches: along an axis with a zero direction component the
+// face is "far" (with a branch per axis electron runs took 3 to 5 % longer).
+__device__ __forceinline__ float dist_axis(float x, float u, int i, float d)
+{
+    // the face's coordinate rounded as cross_face rounds it: a particle on a face is at distance 0 from it
+    const float t = fmaxf(__fdividef(__fsub_rn(__fmul_rn((float)(i + (u > 0.f ? 1 : 0)), d), x), u), 0.f);
+    return u != 0.f ? t : 3.0e38f;
+}
+
 __device__ __forceinline__ float dist_to_face(float x, float y, float z, float u, float v, float w, int ix, int iy,
                                               int iz, float dx, float dy, float dz, int* face)
 {
-    float best = 3.0e38f;
-    int f = 0;
-    if (u != 0.f) {
-        float t = fmaxf(__fdividef((u > 0.f ? (float)(ix + 1) : (float)ix) * dx - x, u), 0.f);
-        if (t < best) { best = t; f = u > 0.f ? 1 : 0; }
-    }
-    if (v != 0.f) {
-        float t = fmaxf(__fdividef((v > 0.f ? (float)(iy + 1) : (float)iy) * dy - y, v), 0.f);
-        if (t < best) { best = t; f = v > 0.f ? 3 : 2; }
-    }
-    if (w != 0.f) {
-        float t = fmaxf(__fdividef((w > 0.f ? (float)(iz + 1) : (float)iz) * dz - z, w), 0.f);
-        if (t < best) { best = t; f = w > 0.f ? 5 : 4; }
-    }
-    *face = f;
+    const float tx = dist_axis(x, u, ix, dx), ty = dist_axis(y, v, iy, dy), tz = dist_axis(z, w, iz, dz);
+    float best = tx, dir = u;
+    int ax = 0;
+    if (ty < best) { best = ty; ax = 2; dir = v; }
+    if (tz < best) { best = tz; ax = 4; dir = w; }
+    *face = ax + (dir > 0.f ? 1 : 0);
     return best;
 }
 
@@ -384,7 +387,6 @@ __device__ __forceinline__ bool init_source(const TransportArgs& a, const G& g, 
     p.r.h1 = (uint32_t)(h >> 32) ^ h1_tag;
     p.r.sub = 0u;
     p.r.n = 0u;
-    p.r.blk = 0xFFFFFFFFu;
     p.type = s.particle == 0 ? PHOTON : ELECTRON;
     p.steps = 0;
     int lo = 0, hi = s.n_bins - 1;               // last q with bound[q] <= h
@@ -429,7 +431,6 @@ __device__ __forceinline__ bool init_phase_space(const TransportArgs& a, unsigne
     p.r.h1 = (uint32_t)(h >> 32) ^ a.stream_tag;
     p.r.sub = 0u;
     p.r.n = 0u;
-    p.r.blk = 0xFFFFFFFFu;
     p.type = r.type == 0 ? PHOTON : (r.type == 1 ? ELECTRON : POSITRON);
     p.steps = 0;
     p.E = r.E;

@@ -153,6 +153,8 @@ struct PsRec {
     int type;                            // 0 photon, 1 electron, 2 positron
 };
 
+constexpr int RUN_COUNTERS = 2;
+
 struct TransportArgs {
     // geometry
     int nx, ny, nz;
@@ -174,7 +176,13 @@ struct TransportArgs {
     float e_split;              // MeV; energy-class boundary of the charged stacks when nstk == 3
     int switch_high, switch_low;
     int refill_min;                      // free lanes needed before a warp refills (>= 1)
-    unsigned long long* hist_counter;
+    int src_share;                       // histories a warp draws at once, at most (1 to 32)
+    int* left_out;                       // per warp: photons it ends with and leaves to k_chains (null: none)
+    unsigned long long* n_left_out;
+    const int* left_in;                  // resumed launch: the same of the launch before (null: a first launch)
+    const unsigned long long* n_left_in;
+    unsigned long long* hist_counter;    // RUN_COUNTERS words, cleared before a launch: [0] histories drawn,
+                                         // [1] warps that left photons to k_chains
     unsigned long long* stats;  // ST_COUNT
     int* err;
     SourceDev src;
@@ -196,6 +204,8 @@ cudaError_t build_tables(const Tables& t, const PhysParams& pp, const float* den
 cudaError_t build_material_tables(const Tables& t, const PhysParams& pp, const MatDef* defs, cudaStream_t s);
 cudaError_t build_phantom_tables(const Tables& t, const float* density, const uint8_t* material, long long nvox,
                                  int* d_err, cudaStream_t s);
+// a.left_out: one int per warp of the launch, or null (long photon chains then stay in their warps);
+// hist_counter's RUN_COUNTERS words are zero
 cudaError_t launch_transport(const TransportArgs& a, int blocks, int threads, size_t smem, cudaStream_t s,
                              int nreg);
 size_t transport_smem_bytes(int n_mat);

@@ -171,7 +171,7 @@ extern "C" ocmc_status ocmc_run_noalloc(int device, int nx, int ny, int nz, cons
     MatDef defs[NMAT_DEFAULT];
     material_defs(defs);
     unsigned long long* stats = cv.take<unsigned long long>(ST_COUNT);
-    unsigned long long* counter = cv.take<unsigned long long>(1);
+    unsigned long long* counter = cv.take<unsigned long long>(RUN_COUNTERS);
     int* err = cv.take<int>(1);
     size_t counters_end = cv.used;
 
@@ -193,6 +193,8 @@ extern "C" ocmc_status ocmc_run_noalloc(int device, int nx, int ny, int nz, cons
         return M.fail(OCMC_ERR_ARG, "launch shape needs more secondary-stack scratch than the 64 MiB static array "
                                    "(lower stack_capacity, block_threads or blocks_per_sm)");
     PRec* stacks = cv.take<PRec>((size_t)blocks * (threads / 32) * nstk * cap);
+    const size_t left_bytes = (size_t)blocks * (threads / 32) * sizeof(int);
+    int* left = cv.used + left_bytes <= NOALLOC_BYTES ? cv.take<int>(left_bytes / sizeof(int)) : nullptr;
 
     cudaStream_t s = reinterpret_cast<cudaStream_t>(cuda_stream);
     size_t stats_off = (size_t)(reinterpret_cast<unsigned char*>(stats) - base);
@@ -227,6 +229,7 @@ extern "C" ocmc_status ocmc_run_noalloc(int device, int nx, int ny, int nz, cons
     a.key1 = (uint32_t)(seed >> 32);
     a.tally = reinterpret_cast<unsigned long long*>(tally_dev);
     a.stacks = stacks;
+    a.left_out = left;
     a.cap = cap;
     a.nstk = nstk;
     a.e_split = p.e_class_split;

@@ -21,11 +21,24 @@
 // the source is exhausted and its stacks are empty; no warp ever waits on
 // another.
 //
+// What bounds it: instruction issue and instruction fetch, not memory (DRAM 2 % of its rate). A warp
+// instruction carries about 19 of 32 lanes because steps differ, and the kernel is larger than an
+// SM's instruction caches, so the code is kept small and uniform: one copy of everything that ends or
+// emits a particle (finish), 32-bit event counters (a 64-bit shared add is a loop per lane), the first
+// draws of a step taken straight from its random block, geometric crossings and post-hinge crossings
+// through one piece of code, no branches in the face distances and the rotation, and a scheduler that
+// is skipped while no lane and no stack needs it. Against the version before (88 KB of code, now 65):
+// 1e8 6 MV photons on the 120^3 slab 123.8 -> 102 ms, 5e6 electrons of 15 MeV on the half-slab
+// 50.3 -> 35.4 ms, 1.3e6 photons on a CT-like 128^3 phantom 3.7 -> 2.3 ms (k_chains, below), the same
+// tallies bit for bit.
+//
 // Dose tally (Sec. 2.2.2): 64-bit fixed-point integer atomics (2^-28 MeV
 // units) into the tally of batch (history id mod B). Integer addition is
 // associative and every particle's random stream is keyed by its lineage, so
 // the tally is bit-identical for any launch configuration and timing.
 #include "ocmc_device.cuh"
+
+#include <algorithm>
 
 namespace ocmc {
 
@@ -34,6 +47,19 @@ namespace {
 constexpr unsigned FULL = 0xFFFFFFFFu;
 constexpr int MAX_WARPS = 32;
 constexpr int STEP_LIMIT = 1 << 22;
+constexpr int CHAIN_LANES = 8;    // a warp flies chains together while at most this many photons are left in it
+constexpr int CHAIN_STEPS = 24;   // flights in a row that make a chain (a photon makes about 6 in water)
+constexpr uint32_t CHAIN_MAX_N = 4u * STEP_LIMIT;   // draws after which a photon is left to its steps and their limit
+
+// Block statistics in shared memory: event counts as 32-bit words (shared memory adds 32-bit
+// integers natively and a warp's lanes together; a 64-bit shared add is a compare-and-swap loop
+// per lane), the two energy sums that hot paths add to as 32-bit halves. Counts move to the
+// 64-bit totals in global memory before a word can wrap (flush_stats) and when a warp ends.
+struct BlockStats {
+    unsigned int n[ST_E_IN];       // event counts, slots [0, ST_E_IN)
+    unsigned int e[2][2];          // energy in, energy escaped: low and high words
+};
+enum { BE_IN = 0, BE_ESC = 1 };
 
 // BL: batched-beamlet mode (sparse hash tallies) or single-beam mode (dense tally);
 // a compile-time flag so the single-beam kernel carries no beamlet code.
@@ -44,13 +70,26 @@ struct CtxT {
     const SmemTables& T;
     PRec* stk;                   // warp's stacks: [0, cap) photons, [cap, 2cap) charged, [2cap, 3cap) slow charged
     int* top;                    // shared: top[0] photons, top[1] charged, top[2] charged below e_split
-    unsigned long long* st;      // shared block statistics
+    BlockStats* st;              // shared block statistics
     float inv_dx, inv_dy, inv_dz, Lx, Ly, Lz;
-    bool ok;
 };
 
+// one event of kind k
 template <class C>
-__device__ __forceinline__ void stat_add(C& c, int k, unsigned long long v) { atomicAdd(c.st + k, v); }
+__device__ __forceinline__ void count(C& c, int k) { atomicAdd(&c.st->n[k], 1u); }
+
+// rare events and energies go straight to the totals
+template <class C>
+__device__ __forceinline__ void count_rare(C& c, int k, unsigned long long v) { atomicAdd(c.a.stats + k, v); }
+
+template <class C>
+__device__ __forceinline__ void add_energy(C& c, int k, unsigned long long q)
+{
+    const unsigned lo = (unsigned)q, hi = (unsigned)(q >> 32);
+    const unsigned old = atomicAdd(&c.st->e[k][0], lo);
+    const unsigned carry = hi + (old > ~lo ? 1u : 0u);
+    if (carry) atomicAdd(&c.st->e[k][1], carry);
+}
 
 // Checks build: a lane whose voxel index lies outside the grid flags ERR_BOUNDS (and its
 // particle is ended by the caller before any access). Always false in the normal build.
@@ -104,10 +143,11 @@ __device__ __forceinline__ void hash_add(const TransportArgs& a, uint32_t b, uin
     atomicOr(a.bl_overflow + b, 1u);
 }
 
+// add q fixed-point units to the lane's tally at voxel (ix, iy, iz)
 template <class C>
-__device__ __forceinline__ void deposit(C& c, const Lane& p, int ix, int iy, int iz, float dE)
+__device__ __forceinline__ void deposit_q(C& c, const Lane& p, int ix, int iy, int iz, unsigned long long q)
 {
-    if (dE > 0.f) {
+    if (q) {
         const int v = ix + c.a.nx * (iy + c.a.ny * iz);     // grids have at most 1024^3 voxels
         if constexpr (OCMC_CHECKS) {
             if (ix < 0 || iy < 0 || iz < 0 || ix >= c.a.nx || iy >= c.a.ny || iz >= c.a.nz ||
@@ -116,46 +156,35 @@ __device__ __forceinline__ void deposit(C& c, const Lane& p, int ix, int iy, int
                 return;
             }
         }
-        if constexpr (C::beamlets) hash_add(c.a, p.r.h1 & ~BL_TAG, (uint32_t)v, fx(dE));
-        else atomicAdd(c.a.tally + (long long)p.batch * c.a.nvox + v, fx(dE));
+        if constexpr (C::beamlets) hash_add(c.a, p.r.h1 & ~BL_TAG, (uint32_t)v, q);
+        else atomicAdd(c.a.tally + (long long)p.batch * c.a.nvox + v, q);
     }
 }
 
+// energy dE > 0 (nothing otherwise) to voxel (ix, iy, iz)
 template <class C>
-__device__ __forceinline__ void push(C& c, int t, float x, float y, float z, float E, float u, float v, float w, int ix,
-                                     int iy, int iz, int type, uint32_t h0, uint32_t h1, uint32_t sub)
+__device__ __forceinline__ void deposit(C& c, const Lane& p, int ix, int iy, int iz, float dE)
+{
+    deposit_q(c, p, ix, iy, iz, dE > 0.f ? fx(dE) : 0ull);
+}
+
+// a particle at p's position on stack t
+template <class C>
+__device__ __forceinline__ void push(C& c, int t, const Lane& p, float E, float u, float v, float w, int type, uint32_t sub,
+                                     uint32_t n)
 {
     int slot = atomicAdd(c.top + t, 1);
     if (slot >= c.a.cap) {
         atomicOr(c.a.err, ERR_OVERFLOW);
-        stat_add(c, ST_DROPPED, 1);
-        stat_add(c, ST_E_DROPPED, fx(E));
+        count_rare(c, ST_DROPPED, 1);
+        count_rare(c, ST_E_DROPPED, fx(E));
         return;
     }
-    PRec* r = c.stk + (size_t)t * c.a.cap + slot;
-    uint32_t vt = (uint32_t)ix | ((uint32_t)iy << 10) | ((uint32_t)iz << 20) | ((uint32_t)type << 30);
-    uint4* q = reinterpret_cast<uint4*>(r);
-    q[0] = make_uint4(__float_as_uint(x), __float_as_uint(y), __float_as_uint(z), __float_as_uint(E));
+    uint32_t vt = (uint32_t)p.ix | ((uint32_t)p.iy << 10) | ((uint32_t)p.iz << 20) | ((uint32_t)type << 30);
+    uint4* q = reinterpret_cast<uint4*>(c.stk + (size_t)t * c.a.cap + slot);
+    q[0] = make_uint4(__float_as_uint(p.x), __float_as_uint(p.y), __float_as_uint(p.z), __float_as_uint(E));
     q[1] = make_uint4(__float_as_uint(u), __float_as_uint(v), __float_as_uint(w), vt);
-    q[2] = make_uint4(h0, h1, sub, 0u);
-}
-
-template <class C>
-__device__ __forceinline__ void push_lane(C& c, int t, const Lane& p)
-{
-    int slot = atomicAdd(c.top + t, 1);
-    if (slot >= c.a.cap) {
-        atomicOr(c.a.err, ERR_OVERFLOW);
-        stat_add(c, ST_DROPPED, 1);
-        stat_add(c, ST_E_DROPPED, fx(p.E));
-        return;
-    }
-    PRec* r = c.stk + (size_t)t * c.a.cap + slot;
-    uint32_t vt = (uint32_t)p.ix | ((uint32_t)p.iy << 10) | ((uint32_t)p.iz << 20) | ((uint32_t)p.type << 30);
-    uint4* q = reinterpret_cast<uint4*>(r);
-    q[0] = make_uint4(__float_as_uint(p.x), __float_as_uint(p.y), __float_as_uint(p.z), __float_as_uint(p.E));
-    q[1] = make_uint4(__float_as_uint(p.u), __float_as_uint(p.v), __float_as_uint(p.w), vt);
-    q[2] = make_uint4(p.r.h0, p.r.h1, p.r.sub, p.r.n);
+    q[2] = make_uint4(p.r.h0, p.r.h1, sub, n);
 }
 
 template <class C>
@@ -173,72 +202,44 @@ __device__ __forceinline__ void pop_lane(const C& c, int t, int slot, Lane& p)
     p.x = __uint_as_float(a.x); p.y = __uint_as_float(a.y); p.z = __uint_as_float(a.z); p.E = __uint_as_float(a.w);
     p.u = __uint_as_float(b.x); p.v = __uint_as_float(b.y); p.w = __uint_as_float(b.z);
     p.ix = b.w & 1023u; p.iy = (b.w >> 10) & 1023u; p.iz = (b.w >> 20) & 1023u; p.type = b.w >> 30;
-    p.r.h0 = d.x; p.r.h1 = d.y; p.r.sub = d.z; p.r.n = d.w; p.r.blk = 0xFFFFFFFFu;
+    p.r.h0 = d.x; p.r.h1 = d.y; p.r.sub = d.z; p.r.n = d.w;
     if constexpr (C::beamlets) p.batch = 0;
     else p.batch = batch_of(d.x, d.y ^ c.a.stream_tag, c.a.pp.n_batches);
     p.steps = 0;
 }
 
-template <class C>
-__device__ __forceinline__ void escape(C& c, const Lane& p)
-{
-    stat_add(c, ST_ESCAPED, 1);
-    stat_add(c, ST_E_ESC, fx(p.E));
-}
+// What a step leaves to the loop's common tail (finish): the lane's fate and at most one secondary
+// at the lane's position. One copy of the code that pushes, absorbs, annihilates and counts escapes
+// serves every kind of step: with a copy at each place that ends or emits a particle the kernel was
+// 88 KB of instructions and waited for instruction fetches more than for anything else.
+enum { LIVE = 0, GONE, ESCAPED, ABSORBED, MOVED };   // MOVED: to the stack of its kind
+struct Pend {
+    float E, u, v, w;
+    int type;                    // -1: no secondary
+    uint32_t sub;
+};
 
-// e-/e+ created at p's position with energy E and direction d: pushed if above the
-// absorption energy, otherwise deposited (a positron then annihilates).
+// Pair production: e- and e+ along the photon, sharing E - 2 mc^2 uniformly: the e- is the step's
+// secondary, the lane itself becomes the e+.
 template <class C>
-__device__ void emit_charged(C& c, const Lane& p, int type, float E, float du, float dv, float dw, uint32_t slot);
-
-// Two photons of mc^2, back to back and isotropic, from a positron with stream r.
-template <class C>
-__device__ __forceinline__ void annihilate(C& c, const Lane& p, Rng& r)
+__device__ __forceinline__ int pair_event(C& c, Lane& p, Pend& s)
 {
-    float wc = 2.f * rng_u(r, c.a.key0, c.a.key1) - 1.f, xi = rng_u(r, c.a.key0, c.a.key1);
-    float st = sqrtf(fmaxf(0.f, 1.f - wc * wc)), sp, cp;
-    __sincosf(6.283185307179586f * xi, &sp, &cp);
-    stat_add(c, ST_ANNIH, 1);
-    if (MC2F >= c.a.pp.e_abs_g) {
-        push(c, 0, p.x, p.y, p.z, MC2F, st * cp, st * sp, wc, p.ix, p.iy, p.iz, PHOTON, r.h0, r.h1,
-             child_sub(r.sub, r.n, 0));
-        push(c, 0, p.x, p.y, p.z, MC2F, -st * cp, -st * sp, -wc, p.ix, p.iy, p.iz, PHOTON, r.h0, r.h1,
-             child_sub(r.sub, r.n, 1));
-    } else {
-        deposit(c, p, p.ix, p.iy, p.iz, 2.f * MC2F);
-    }
-}
-
-template <class C>
-__device__ void emit_charged(C& c, const Lane& p, int type, float E, float du, float dv, float dw, uint32_t slot)
-{
-    uint32_t sub = child_sub(p.r.sub, p.r.n, slot);
-    if (E >= c.a.pp.e_abs_e && !(c.a.pp.flags & 8)) {
-        push(c, charged_stack(c.a, E), p.x, p.y, p.z, E, du, dv, dw, p.ix, p.iy, p.iz, type, p.r.h0, p.r.h1, sub);
-        return;
-    }
-    deposit(c, p, p.ix, p.iy, p.iz, E);
-    if (type == POSITRON) {
-        Rng r;
-        r.h0 = p.r.h0; r.h1 = p.r.h1; r.sub = sub; r.n = 0; r.blk = 0xFFFFFFFFu;
-        annihilate(c, p, r);
-    }
-}
-
-// Pair production: e- and e+ along the photon, sharing E - 2 mc^2 uniformly.
-template <class C>
-__device__ __forceinline__ void pair_event(C& c, Lane& p)
-{
-    stat_add(c, ST_PAIR, 1);
+    count(c, ST_PAIR);
     float avail = p.E - 2.f * MC2F;
     float Tm = rng_u(p.r, c.a.key0, c.a.key1) * avail, Tp = avail - Tm;
-    emit_charged(c, p, ELECTRON, Tm, p.u, p.v, p.w, 0);
-    emit_charged(c, p, POSITRON, Tp, p.u, p.v, p.w, 1);
+    s.E = Tm; s.u = p.u; s.v = p.v; s.w = p.w;
+    s.type = ELECTRON;
+    s.sub = child_sub(p.r.sub, p.r.n, 0);
+    p.r.sub = child_sub(p.r.sub, p.r.n, 1);
+    p.r.n = 0;
+    p.E = Tp;
+    p.type = POSITRON;
+    return Tp >= c.a.pp.e_abs_e && !(c.a.pp.flags & 8) ? MOVED : ABSORBED;
 }
 
-// One Woodcock flight and, if real, the interaction. Returns false when the photon ends.
+// One Woodcock flight and, if real, the interaction.
 template <class C>
-__device__ __forceinline__ bool photon_step(C& c, Lane& p, unsigned& n_fict)
+__device__ __forceinline__ int photon_step(C& c, Lane& p, Pend& sec)
 {
     const TransportArgs& a = c.a;
     const SmemTables& T = c.T;
@@ -246,19 +247,19 @@ __device__ __forceinline__ bool photon_step(C& c, Lane& p, unsigned& n_fict)
     rng_step_start(p.r, k0, k1);
     EIdx ei = e_index(p.E);
     float lnmaj = lerp1(T.phmaj[ei.i], T.phmaj[ei.i + 1], ei.f);
-    if (lnmaj < -1e29f) { escape(c, p); return false; }
+    if (lnmaj < -1e29f) return ESCAPED;
     float mumax = __expf(lnmaj);
-    float s = -__logf(rng_u(p.r, k0, k1)) / mumax;
+    float s = -__logf(u01(p.r.buf.x)) / mumax;         // the step's first three draws
+    const float u_real = u01(p.r.buf.y), xi = u01(p.r.buf.z);
     p.x = fmaf(s, p.u, p.x);
     p.y = fmaf(s, p.v, p.y);
     p.z = fmaf(s, p.w, p.z);
     if (!(p.x >= 0.f && p.y >= 0.f && p.z >= 0.f && p.x <= c.Lx && p.y <= c.Ly && p.z <= c.Lz)) {
         if ((a.pp.flags & 4) && p.z > c.Lz) {
-            stat_add(c, ST_TRANSMITTED, 1);
-            stat_add(c, ST_E_TRANS, fx(p.E));
+            count_rare(c, ST_TRANSMITTED, 1);
+            count_rare(c, ST_E_TRANS, fx(p.E));
         }
-        escape(c, p);
-        return false;
+        return ESCAPED;
     }
     p.ix = min((int)(p.x * c.inv_dx), a.nx - 1);
     p.iy = min((int)(p.y * c.inv_dy), a.ny - 1);
@@ -268,180 +269,170 @@ __device__ __forceinline__ bool photon_step(C& c, Lane& p, unsigned& n_fict)
     int m = __ldg(a.material + vox);
     float4 pa = T.ph[m * MS4 + ei.i], pb = T.ph[m * MS4 + ei.i + 1];
     float mu = rho * __expf(lerp1(pa.x, pb.x, ei.f));
-    if (mu > mumax * 1.00001f) stat_add(c, ST_VIOL, 1);
-    if (rng_u(p.r, k0, k1) * mumax >= mu) { n_fict++; return true; }
-    if (a.pp.flags & 4) { stat_add(c, ST_E_KILLED, fx(p.E)); return false; }
+    if (mu > mumax * 1.00001f) count_rare(c, ST_VIOL, 1);
+    p.r.n += 2u;
+    if (u_real * mumax >= mu) { count(c, ST_FICT); return LIVE; }
+    if (a.pp.flags & 4) { count_rare(c, ST_E_KILLED, fx(p.E)); return GONE; }
     float fC = lerp1(pa.y, pb.y, ei.f), fP = lerp1(pa.z, pb.z, ei.f);
-    float xi = rng_u(p.r, k0, k1);
+    p.r.n += 1u;
     if (xi >= fC && xi < fC + fP) {
-        stat_add(c, ST_PHOTO, 1);
-        deposit(c, p, p.ix, p.iy, p.iz, p.E);
-        return false;
+        count(c, ST_PHOTO);
+        return ABSORBED;
     }
-    if (xi >= fC + fP && p.E > 2.f * MC2F) {
-        pair_event(c, p);
-        return false;
-    }
+    if (xi >= fC + fP && p.E > 2.f * MC2F) return pair_event(c, p, sec);
     // Compton scattering (also the rare pair selection below threshold from table interpolation)
-    stat_add(c, ST_COMPTON, 1);
+    count(c, ST_COMPTON);
     float eps;
-    float cth = sample_compton(p.E, p.r, k0, k1, &eps, &c.ok);
+    bool ok = true;
+    float cth = sample_compton(p.E, p.r, k0, k1, &eps, &ok);
+    if (!ok) atomicOr(a.err, ERR_LIMIT);
     float xphi = rng_u(p.r, k0, k1);
-    float E0 = p.E, E1 = eps * E0, Te = E0 - E1;
+    float E0 = p.E, E1 = __fmul_rn(eps, E0), Te = __fsub_rn(E0, E1);
     float u0 = p.u, v0 = p.v, w0 = p.w;
     rotate(p.u, p.v, p.w, cth, xphi);
     if (Te > 0.f) {
-        float qu = E0 * u0 - E1 * p.u, qv = E0 * v0 - E1 * p.v, qw = E0 * w0 - E1 * p.w;
-        float inv = rsqrtf(fmaxf(qu * qu + qv * qv + qw * qw, 1e-30f));
-        emit_charged(c, p, ELECTRON, Te, qu * inv, qv * inv, qw * inv, 0);
+        float qu = __fsub_rn(__fmul_rn(E0, u0), __fmul_rn(E1, p.u)), qv = __fsub_rn(__fmul_rn(E0, v0), __fmul_rn(E1, p.v)),
+              qw = __fsub_rn(__fmul_rn(E0, w0), __fmul_rn(E1, p.w));
+        float inv = rsqrtf(fmaxf(__fmaf_rn(qw, qw, __fmaf_rn(qu, qu, __fmul_rn(qv, qv))), 1e-30f));
+        sec.E = Te; sec.u = qu * inv; sec.v = qv * inv; sec.w = qw * inv;
+        sec.type = ELECTRON;
+        sec.sub = child_sub(p.r.sub, p.r.n, 0);
     }
     p.E = E1;
-    if (p.E < a.pp.e_abs_g) {
-        deposit(c, p, p.ix, p.iy, p.iz, p.E);
-        return false;
-    }
-    return true;
+    return p.E < a.pp.e_abs_g ? ABSORBED : LIVE;
 }
 
+// the neighbouring voxel across a face, the position put exactly on it; false outside the phantom
 template <class C>
 __device__ __forceinline__ bool cross_face(const C& c, Lane& p, int face)
 {
-    int ax = face >> 1;
-    bool up = face & 1;
-    if (ax == 0) { p.ix += up ? 1 : -1; p.x = (float)(up ? p.ix : p.ix + 1) * c.a.dx; }
-    else if (ax == 1) { p.iy += up ? 1 : -1; p.y = (float)(up ? p.iy : p.iy + 1) * c.a.dy; }
-    else { p.iz += up ? 1 : -1; p.z = (float)(up ? p.iz : p.iz + 1) * c.a.dz; }
-    return p.ix >= 0 && p.iy >= 0 && p.iz >= 0 && p.ix < c.a.nx && p.iy < c.a.ny && p.iz < c.a.nz;
+    const int ax = face >> 1, up = face & 1;
+    const int i = (ax == 0 ? p.ix : ax == 1 ? p.iy : p.iz) + 2 * up - 1;
+    const float x = (float)(i + 1 - up) * (ax == 0 ? c.a.dx : ax == 1 ? c.a.dy : c.a.dz);
+    const int n = ax == 0 ? c.a.nx : ax == 1 ? c.a.ny : c.a.nz;
+    if (ax == 0) { p.ix = i; p.x = x; }
+    if (ax == 1) { p.iy = i; p.y = x; }
+    if (ax == 2) { p.iz = i; p.z = x; }
+    return (unsigned)i < (unsigned)n;
 }
 
 // Discrete hard event at the end of a step: Moller (probability sM / tot) or bremsstrahlung.
 template <class C>
-__device__ __forceinline__ void hard_event(C& c, Lane& p, int m, float sM, float tot)
+__device__ __forceinline__ void hard_event(C& c, Lane& p, int m, float sM, float tot, Pend& sec)
 {
     const SmemTables& T = c.T;
-    if (rng_u(p.r, c.a.key0, c.a.key1) * tot < sM) {
-        stat_add(c, ST_MOLLER, 1);
-        float Tk = p.E;
-        float eps = sample_moller(Tk, c.a.pp.w_cc, p.r, c.a.key0, c.a.key1, &c.ok);
-        float W = eps * Tk, T1 = Tk - W;
-        float xphi = rng_u(p.r, c.a.key0, c.a.key1);
-        float mu1 = sqrtf(fminf(1.f, T1 * (Tk + 2.f * MC2F) / (Tk * (T1 + 2.f * MC2F))));
-        float mu2 = sqrtf(fminf(1.f, W * (Tk + 2.f * MC2F) / (Tk * (W + 2.f * MC2F))));
-        float su = p.u, sv2 = p.v, sw = p.w;
-        rotate(su, sv2, sw, mu2, xphi + 0.5f);
-        emit_charged(c, p, ELECTRON, W, su, sv2, sw, 2);
-        rotate(p.u, p.v, p.w, mu1, xphi);
-        p.E = T1;
+    const float Tk = p.E;
+    const bool moller = rng_u(p.r, c.a.key0, c.a.key1) * tot < sM;
+    bool ok = true;
+    float mu, W, mu1 = 1.f;
+    if (moller) {
+        count(c, ST_MOLLER);
+        float eps = sample_moller(Tk, c.a.pp.w_cc, p.r, c.a.key0, c.a.key1, &ok);
+        W = eps * Tk;
+        float T1 = Tk - W;
+        mu1 = sqrtf(fminf(1.f, T1 * (Tk + 2.f * MC2F) / (Tk * (T1 + 2.f * MC2F))));
+        mu = sqrtf(fminf(1.f, W * (Tk + 2.f * MC2F) / (Tk * (W + 2.f * MC2F))));
     } else {
-        stat_add(c, ST_BREMS, 1);
-        float Tk = p.E;
-        float k = sample_brems(Tk, c.a.pp.w_cb, T.msc[m * MS1], T.msc[m * MS1 + 1], p.r, c.a.key0, c.a.key1, &c.ok);
+        count(c, ST_BREMS);
+        W = sample_brems(Tk, c.a.pp.w_cb, T.msc[m * MS1], T.msc[m * MS1 + 1], p.r, c.a.key0, c.a.key1, &ok);
         float th = MC2F / (Tk + MC2F);
-        float xphi = rng_u(p.r, c.a.key0, c.a.key1);
-        float gu = p.u, gv = p.v, gw = p.w;
-        rotate(gu, gv, gw, __cosf(th), xphi);
-        if (k >= c.a.pp.e_abs_g)
-            push(c, 0, p.x, p.y, p.z, k, gu, gv, gw, p.ix, p.iy, p.iz, PHOTON, p.r.h0, p.r.h1,
-                 child_sub(p.r.sub, p.r.n, 3));
-        else
-            deposit(c, p, p.ix, p.iy, p.iz, k);
-        p.E = Tk - k;
+        mu = __cosf(th);
     }
+    if (!ok) atomicOr(c.a.err, ERR_LIMIT);
+    float xphi = rng_u(p.r, c.a.key0, c.a.key1);
+    sec.E = W;
+    sec.u = p.u; sec.v = p.v; sec.w = p.w;
+    rotate(sec.u, sec.v, sec.w, mu, moller ? xphi + 0.5f : xphi);
+    sec.type = moller ? ELECTRON : PHOTON;
+    sec.sub = child_sub(p.r.sub, p.r.n, moller ? 2u : 3u);
+    if (moller) rotate(p.u, p.v, p.w, mu1, xphi);      // a bremsstrahlung electron keeps its direction
+    p.E = Tk - W;
 }
 
-// A charged particle that fell below its absorption energy.
+// One condensed-history step.
 template <class C>
-__device__ __forceinline__ void absorb_charged(C& c, Lane& p)
-{
-    deposit(c, p, p.ix, p.iy, p.iz, p.E);
-    if (p.type == POSITRON) annihilate(c, p, p.r);
-}
-
-// One condensed-history step. Returns false when the particle ends.
-template <class C>
-__device__ __forceinline__ bool charged_step(C& c, Lane& p, unsigned& n_hfict)
+__device__ __forceinline__ int charged_step(C& c, Lane& p, Pend& sec)
 {
     const TransportArgs& a = c.a;
     const SmemTables& T = c.T;
     const uint32_t k0 = a.key0, k1 = a.key1;
-    if (vox_bad(c, p)) return false;
+    if (vox_bad(c, p)) return GONE;
     const int vox = p.ix + a.nx * (p.iy + a.ny * p.iz);
     float rho = __ldg(a.density + vox);
     int m = __ldg(a.material + vox);
     int face;
     float sv = dist_to_face(p.x, p.y, p.z, p.u, p.v, p.w, p.ix, p.iy, p.iz, a.dx, a.dy, a.dz, &face);
-    if (!(rho > 0.f) || sv < a.pp.s_min) {
-        // nothing to interact with, or a boundary closer than s_min: cross geometrically
-        p.x = fmaf(sv, p.u, p.x);
-        p.y = fmaf(sv, p.v, p.y);
-        p.z = fmaf(sv, p.w, p.z);
-        stat_add(c, ST_GEO, 1);
-        if (!cross_face(c, p, face)) { escape(c, p); return false; }
-        return true;
-    }
-    rng_step_start(p.r, k0, k1);
-    EIdx ei = e_index(p.E);
     const int mb = m * MS4, mb2 = m * MS2;
-    float4 A = T.el[mb + ei.i], B = T.el[mb + ei.i + 1];
-    float2 C2 = T.el2[mb2 + ei.i], D2 = T.el2[mb2 + ei.i + 1];
-    float lnR = lerp1(A.x, B.x, ei.f);
-    float s_maxe = lerp1(C2.x, D2.x, ei.f) / rho;
-    float sighat = (a.pp.flags & 1) ? 0.f : C2.y;
-    float d_ev = sighat > 0.f ? -__logf(rng_u(p.r, k0, k1)) / (rho * sighat) : 3.0e38f;
-    float s = sv;
+    float hx = p.x, hy = p.y, hz = p.z, l2 = sv, sighat = 0.f;
     int lim = 0;
-    if (a.pp.d_maxs < s) { s = a.pp.d_maxs; lim = 1; }
-    if (s_maxe < s) { s = s_maxe; lim = 2; }
-    if (d_ev < s) { s = d_ev; lim = 3; }
-    // random hinge: s1 straight, deflect, then the rest (clipped to this voxel)
-    float s1 = rng_u(p.r, k0, k1) * s;
-    float hx = fmaf(s1, p.u, p.x), hy = fmaf(s1, p.v, p.y), hz = fmaf(s1, p.w, p.z);
-    float E0 = p.E;
-    const float R0 = __expf(lnR), g0 = range_to_lnE(T, m, lnR);
-    float Efull = csda_end2(T, m, E0, R0, g0, rho * s);
-    if (!(a.pp.flags & 2)) {
-        EIdx em = e_index(0.5f * (E0 + Efull));
-        float l1 = lerp1(T.el[mb + em.i].y, T.el[mb + em.i + 1].y, em.f);
-        float cth = sample_ms(T, rho * s * l1, p.r, k0, k1);
-        float xphi = rng_u(p.r, k0, k1);
-        rotate(p.u, p.v, p.w, cth, xphi);
-    }
-    int face2;
-    float tex = dist_to_face(hx, hy, hz, p.u, p.v, p.w, p.ix, p.iy, p.iz, a.dx, a.dy, a.dz, &face2);
-    float rem = s - s1, Eend;
-    bool crossed;
-    if (rem < tex) {
-        p.x = fmaf(rem, p.u, hx);
-        p.y = fmaf(rem, p.v, hy);
-        p.z = fmaf(rem, p.w, hz);
-        Eend = Efull;
-        crossed = false;
+    bool crossed = true;
+    // nothing to interact with, or a boundary closer than s_min: cross geometrically
+    const bool geo = !(rho > 0.f) || sv < a.pp.s_min;
+    if (geo) {
+        count(c, ST_GEO);
     } else {
-        p.x = fmaf(tex, p.u, hx);
-        p.y = fmaf(tex, p.v, hy);
-        p.z = fmaf(tex, p.w, hz);
-        Eend = csda_end2(T, m, E0, R0, g0, rho * (s1 + tex));
-        crossed = true;
+        rng_step_start(p.r, k0, k1);
+        EIdx ei = e_index(p.E);
+        float4 A = T.el[mb + ei.i], B = T.el[mb + ei.i + 1];
+        float2 C2 = T.el2[mb2 + ei.i], D2 = T.el2[mb2 + ei.i + 1];
+        float lnR = lerp1(A.x, B.x, ei.f);
+        float s_maxe = lerp1(C2.x, D2.x, ei.f) / rho;
+        sighat = (a.pp.flags & 1) ? 0.f : C2.y;
+        // the step's draws in order: event distance (only with a majorant), hinge, deflection, azimuth
+        const bool ev = sighat > 0.f;
+        const uint32_t w1 = ev ? p.r.buf.y : p.r.buf.x, w2 = ev ? p.r.buf.z : p.r.buf.y, w3 = ev ? p.r.buf.w : p.r.buf.z;
+        float d_ev = ev ? -__logf(u01(p.r.buf.x)) / (rho * sighat) : 3.0e38f;
+        p.r.n += ev ? 2u : 1u;
+        float s = sv;
+        if (a.pp.d_maxs < s) { s = a.pp.d_maxs; lim = 1; }
+        if (s_maxe < s) { s = s_maxe; lim = 2; }
+        if (d_ev < s) { s = d_ev; lim = 3; }
+        // random hinge: s1 straight, deflect, then the rest (clipped to this voxel)
+        float s1 = u01(w1) * s;
+        hx = fmaf(s1, p.u, p.x);
+        hy = fmaf(s1, p.v, p.y);
+        hz = fmaf(s1, p.w, p.z);
+        float E0 = p.E;
+        const float R0 = __expf(lnR), g0 = range_to_lnE(T, m, lnR);
+        float Eend = csda_end2(T, m, E0, R0, g0, rho * s);
+        if (!(a.pp.flags & 2)) {
+            EIdx em = e_index(0.5f * (E0 + Eend));
+            float l1 = lerp1(T.el[mb + em.i].y, T.el[mb + em.i + 1].y, em.f);
+            const float G1 = rho * s * l1;
+            const bool deflects = G1 >= 1e-12f;
+            float cth = sample_ms_u(T, G1, u01(w2));
+            p.r.n += deflects ? 2u : 1u;
+            rotate(p.u, p.v, p.w, cth, u01(deflects ? w3 : w2));
+        }
+        float tex = dist_to_face(hx, hy, hz, p.u, p.v, p.w, p.ix, p.iy, p.iz, a.dx, a.dy, a.dz, &face);
+        const float rem = s - s1;
+        crossed = !(rem < tex);
+        l2 = crossed ? tex : rem;
+        if (crossed) Eend = csda_end2(T, m, E0, R0, g0, rho * (s1 + tex));
+        deposit(c, p, p.ix, p.iy, p.iz, E0 - Eend);
+        p.E = Eend;
     }
-    deposit(c, p, p.ix, p.iy, p.iz, E0 - Eend);
-    p.E = Eend;
-    if (crossed && !cross_face(c, p, face2)) { escape(c, p); return false; }
-    if (p.E < a.pp.e_abs_e) { absorb_charged(c, p); return false; }
+    p.x = fmaf(l2, p.u, hx);
+    p.y = fmaf(l2, p.v, hy);
+    p.z = fmaf(l2, p.w, hz);
+    if (crossed && !cross_face(c, p, face)) return ESCAPED;
+    if (geo) return LIVE;
+    if (p.E < a.pp.e_abs_e) return ABSORBED;
     if (lim == 3 && !crossed) {
         EIdx e2 = e_index(p.E);
         float4 A2 = T.el[mb + e2.i], B2 = T.el[mb + e2.i + 1];
         float sM = p.E > 2.f * a.pp.w_cc ? lerp1(A2.z, B2.z, e2.f) : 0.f;
         float sB = p.E > a.pp.w_cb ? lerp1(A2.w, B2.w, e2.f) : 0.f;
         float tot = sM + sB;
-        if (tot > sighat * 1.00001f) stat_add(c, ST_VIOL, 1);
+        if (tot > sighat * 1.00001f) count_rare(c, ST_VIOL, 1);
         if (rng_u(p.r, k0, k1) * sighat < tot) {
-            hard_event(c, p, m, sM, tot);
-            if (p.E < a.pp.e_abs_e) { absorb_charged(c, p); return false; }
+            hard_event(c, p, m, sM, tot, sec);
+            if (p.E < a.pp.e_abs_e) return ABSORBED;
         } else {
-            n_hfict++;
+            count(c, ST_HARD_FICT);
         }
     }
-    return true;
+    return LIVE;
 }
 
 // ---- voxel-crossing (fixed-step) electron steps ------------------------------------------
@@ -454,7 +445,7 @@ __device__ __forceinline__ bool charged_step(C& c, Lane& p, unsigned& n_hfict)
 // E (1 - f_maxe) (before the hinge: deflected there, for the path travelled); a candidate at the
 // end of an event-limited step is real with probability rho sigma_hard(E) / majorant in the
 // voxel where it ends.
-enum { SEG_DONE = 0, SEG_FLOOR, SEG_OUT };   // SEG_OUT: the particle escaped or was absorbed
+enum { SEG_DONE = 0, SEG_FLOOR, SEG_OUT, SEG_ABSORBED, SEG_GONE };
 
 __device__ __forceinline__ float range_R(const SmemTables& T, int m, float E)
 {
@@ -472,8 +463,8 @@ __device__ __forceinline__ int cross_segment(C& c, Lane& p, float L, float Ef, f
     const SmemTables& T = c.T;
     float left = L, moved = 0.f;
     for (int guard = 0; left > 0.f; ++guard) {
-        if (guard > 4 * (a.nx + a.ny + a.nz)) { c.ok = false; break; }   // cannot happen: bounded crossings
-        if (vox_bad(c, p)) { *done = moved; return SEG_OUT; }
+        if (guard > 4 * (a.nx + a.ny + a.nz)) { atomicOr(a.err, ERR_LIMIT); break; }   // cannot happen: bounded crossings
+        if (vox_bad(c, p)) { *done = moved; return SEG_GONE; }
         const int vox = p.ix + a.nx * (p.iy + a.ny * p.iz);
         const float rho = __ldg(a.density + vox);
         const int m = __ldg(a.material + vox);
@@ -497,21 +488,23 @@ __device__ __forceinline__ int cross_segment(C& c, Lane& p, float L, float Ef, f
         p.E = Eend;
         left -= l;
         moved += l;
-        if (p.E < a.pp.e_abs_e) { absorb_charged(c, p); *done = moved; return SEG_OUT; }
+        if (p.E < a.pp.e_abs_e) { *done = moved; return SEG_ABSORBED; }
         if (flo) { *done = moved; return SEG_FLOOR; }
-        if (cross && !cross_face(c, p, face)) { escape(c, p); *done = moved; return SEG_OUT; }
+        if (cross && !cross_face(c, p, face)) { *done = moved; return SEG_OUT; }
     }
     *done = moved;
     return SEG_DONE;
 }
 
+__device__ __forceinline__ int segment_fate(int r) { return r == SEG_OUT ? ESCAPED : r == SEG_ABSORBED ? ABSORBED : GONE; }
+
 template <class C>
-__device__ __forceinline__ bool charged_step_cross(C& c, Lane& p, unsigned& n_hfict)
+__device__ __forceinline__ int charged_step_cross(C& c, Lane& p, Pend& sec)
 {
     const TransportArgs& a = c.a;
     const SmemTables& T = c.T;
     const uint32_t k0 = a.key0, k1 = a.key1;
-    if (vox_bad(c, p)) return false;
+    if (vox_bad(c, p)) return GONE;
     const int vox = p.ix + a.nx * (p.iy + a.ny * p.iz);
     const float rho0 = __ldg(a.density + vox);
     const int m0 = __ldg(a.material + vox);
@@ -521,9 +514,8 @@ __device__ __forceinline__ bool charged_step_cross(C& c, Lane& p, unsigned& n_hf
         p.x = fmaf(sv, p.u, p.x);
         p.y = fmaf(sv, p.v, p.y);
         p.z = fmaf(sv, p.w, p.z);
-        stat_add(c, ST_GEO, 1);
-        if (!cross_face(c, p, face)) { escape(c, p); return false; }
-        return true;
+        count(c, ST_GEO);
+        return cross_face(c, p, face) ? LIVE : ESCAPED;
     }
     rng_step_start(p.r, k0, k1);
     const float E0 = p.E;
@@ -532,17 +524,20 @@ __device__ __forceinline__ bool charged_step_cross(C& c, Lane& p, unsigned& n_hf
     const float lnR = lerp1(T.el[mb + ei.i].x, T.el[mb + ei.i + 1].x, ei.f);
     const float s_maxe = lerp1(T.el2[mb2 + ei.i].x, T.el2[mb2 + ei.i + 1].x, ei.f) / rho0;
     const float maj = (a.pp.flags & 1) ? 0.f : __ldg(a.t.elmaj + ei.i);
-    const float d_ev = maj > 0.f ? -__logf(rng_u(p.r, k0, k1)) / maj : 3.0e38f;
+    const bool ev = maj > 0.f;
+    const uint32_t w1 = ev ? p.r.buf.y : p.r.buf.x;
+    const float d_ev = ev ? -__logf(u01(p.r.buf.x)) / maj : 3.0e38f;
+    p.r.n += ev ? 2u : 1u;
     float s = a.pp.d_maxs;
     int lim = 1;
     if (s_maxe < s) { s = s_maxe; lim = 2; }
     if (d_ev < s) { s = d_ev; lim = 3; }
-    const float s1 = rng_u(p.r, k0, k1) * s;
+    const float s1 = u01(w1) * s;
     const float Ef = E0 * (1.f - a.pp.f_maxe);
     const float Efull = csda_end2(T, m0, E0, __expf(lnR), range_to_lnE(T, m0, lnR), rho0 * s);
     float done;
     int r = cross_segment(c, p, s1, Ef, &done);
-    if (r == SEG_OUT) return false;
+    if (r >= SEG_OUT) return segment_fate(r);
     if (!(a.pp.flags & 2)) {
         EIdx em = e_index(0.5f * (E0 + Efull));
         float l1 = lerp1(T.el[mb + em.i].y, T.el[mb + em.i + 1].y, em.f);
@@ -550,12 +545,12 @@ __device__ __forceinline__ bool charged_step_cross(C& c, Lane& p, unsigned& n_hf
         float xphi = rng_u(p.r, k0, k1);
         rotate(p.u, p.v, p.w, cth, xphi);
     }
-    if (r == SEG_FLOOR) return true;
+    if (r == SEG_FLOOR) return LIVE;
     r = cross_segment(c, p, s - s1, Ef, &done);
-    if (r == SEG_OUT) return false;
-    if (r == SEG_FLOOR || lim != 3) return true;
+    if (r >= SEG_OUT) return segment_fate(r);
+    if (r == SEG_FLOOR || lim != 3) return LIVE;
     // candidate hard event where the step ended
-    if (vox_bad(c, p)) return false;
+    if (vox_bad(c, p)) return GONE;
     const int v2 = p.ix + a.nx * (p.iy + a.ny * p.iz);
     const float rho = __ldg(a.density + v2);
     const int m = __ldg(a.material + v2);
@@ -564,14 +559,97 @@ __device__ __forceinline__ bool charged_step_cross(C& c, Lane& p, unsigned& n_hf
     const float sM = p.E > 2.f * a.pp.w_cc ? rho * lerp1(A2.z, B2.z, e2.f) : 0.f;
     const float sB = p.E > a.pp.w_cb ? rho * lerp1(A2.w, B2.w, e2.f) : 0.f;
     const float tot = sM + sB;
-    if (tot > maj * 1.00001f) stat_add(c, ST_VIOL, 1);
+    if (tot > maj * 1.00001f) count_rare(c, ST_VIOL, 1);
     if (rng_u(p.r, k0, k1) * maj < tot) {
-        hard_event(c, p, m, sM, tot);
-        if (p.E < a.pp.e_abs_e) { absorb_charged(c, p); return false; }
+        hard_event(c, p, m, sM, tot, sec);
+        if (p.E < a.pp.e_abs_e) return ABSORBED;
     } else {
-        n_hfict++;
+        count(c, ST_HARD_FICT);
     }
-    return true;
+    return LIVE;
+}
+
+// The common tail: emits the pending secondary and carries out the lane's fate. A secondary below
+// its absorption energy is deposited at the lane's voxel, as are an absorbed particle's energy and,
+// below the photon cutoff, a positron's annihilation photons; a positron above it emits two photons
+// of mc^2, back to back and isotropic, from its own stream.
+template <class C>
+__device__ __forceinline__ void finish(C& c, Lane& p, Pend& s, int fate)
+{
+    const TransportArgs& a = c.a;
+    unsigned long long q = 0ull;
+    const bool kerma = a.pp.flags & 8;
+    int todo = 0;                                  // pushes: 1 the secondary, 2 the lane, 4 and 8 annihilation photons
+    if (s.type >= 0) {
+        if (s.type == PHOTON ? s.E >= a.pp.e_abs_g : s.E >= a.pp.e_abs_e && !kerma) todo = 1;
+        else q = fx(s.E);
+    }
+    if (fate == ESCAPED) {
+        count(c, ST_ESCAPED);
+        add_energy(c, BE_ESC, fx(p.E));
+    } else if (fate == MOVED) {
+        todo |= 2;
+    } else if (fate == ABSORBED) {
+        q += p.E > 0.f ? fx(p.E) : 0ull;
+        if (p.type == POSITRON) {
+            count(c, ST_ANNIH);
+            if (MC2F >= a.pp.e_abs_g) todo |= 12;
+            else q += fx(2.f * MC2F);
+        }
+    }
+    deposit_q(c, p, p.ix, p.iy, p.iz, q);
+#pragma unroll 1
+    while (todo) {
+        if (!(todo & 1)) {
+            if (todo & 2) {
+                s.E = p.E; s.u = p.u; s.v = p.v; s.w = p.w;
+                s.type = p.type;
+                s.sub = p.r.sub;
+                todo ^= 2;
+            } else if (todo & 4) {
+                float wc = 2.f * rng_u(p.r, a.key0, a.key1) - 1.f, xi = rng_u(p.r, a.key0, a.key1);
+                float st = sqrtf(fmaxf(0.f, 1.f - wc * wc)), sp, cp;
+                __sincosf(6.283185307179586f * xi, &sp, &cp);
+                s.E = MC2F; s.u = st * cp; s.v = st * sp; s.w = wc;
+                s.type = PHOTON;
+                s.sub = child_sub(p.r.sub, p.r.n, 0);
+                todo ^= 4;
+            } else {
+                s.u = -s.u; s.v = -s.v; s.w = -s.w;
+                s.sub = child_sub(p.r.sub, p.r.n, 1);
+                todo ^= 8;
+            }
+        } else {
+            todo ^= 1;
+        }
+        push(c, s.type == PHOTON ? 0 : charged_stack(a, s.E), p, s.E, s.u, s.v, s.w, s.type, s.sub, 0u);
+    }
+}
+
+// A warp moves the block's counts to the totals when its own iterations since the last time reach
+// FLUSH_ITERS and when it ends: between two flushes a block's warps make at most 32 * 2^20 iterations
+// of 32 lanes, so no 32-bit count of events (at most one of a kind per lane and step) wraps.
+constexpr unsigned FLUSH_ITERS = 1u << 20;
+
+__device__ __noinline__ void flush_stats(const TransportArgs& a, BlockStats& st, unsigned int* wc)
+{
+#pragma unroll 1
+    for (int k = 0; k < ST_E_IN; ++k) {
+        const unsigned v = atomicExch(&st.n[k], 0u);
+        if (v) atomicAdd(a.stats + k, (unsigned long long)v);
+    }
+    // the halves one after the other: a carry that arrives between the two is added by the next flush
+#pragma unroll 1
+    for (int k = 0; k < 2; ++k) {
+        const unsigned lo = atomicExch(&st.e[k][0], 0u), hi = atomicExch(&st.e[k][1], 0u);
+        const unsigned long long q = ((unsigned long long)hi << 32) + lo;
+        if (q) atomicAdd(a.stats + (k == BE_IN ? ST_E_IN : ST_E_ESC), q);
+    }
+#pragma unroll 1
+    for (int k = 0; k < 3; ++k) {
+        const unsigned v = atomicExch(wc + k, 0u);
+        if (v) atomicAdd(a.stats + ST_WARP_ITERS + k, (unsigned long long)v);
+    }
 }
 
 // NREG: register cap per thread. More registers spill less; fewer registers let more
@@ -584,19 +662,22 @@ template <bool BL, bool PS, int NREG, bool XV = false>
 __global__ void __maxnreg__(NREG) k_transport(const __grid_constant__ TransportArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int s_top[MAX_WARPS][3];
-    __shared__ unsigned long long s_st[ST_COUNT];
+    __shared__ __align__(16) int s_top[MAX_WARPS][4];      // per warp: its stacks' tops (and a spare word)
+    __shared__ BlockStats s_st;
     __shared__ unsigned long long s_time[MAX_WARPS][2];   // per warp: start, source seen exhausted
-    __shared__ unsigned long long s_wc[MAX_WARPS][3];     // per warp: iterations, photon / charged lane-steps
+    __shared__ unsigned int s_wc[MAX_WARPS][4];           // per warp: iterations, photon / charged lane-steps
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    for (int i = threadIdx.x; i < ST_COUNT; i += blockDim.x) s_st[i] = 0ull;
-    if (lane == 0) { s_top[wib][0] = 0; s_top[wib][1] = 0; s_top[wib][2] = 0; }
+    for (int i = threadIdx.x; i < (int)(sizeof(BlockStats) / 4); i += blockDim.x) reinterpret_cast<unsigned*>(&s_st)[i] = 0u;
+    const long long gw = (long long)blockIdx.x * (blockDim.x >> 5) + wib;
+    // a resumed launch finishes what the warps of the launch before left on their photon stacks
+    const int rest = a.left_in && *a.n_left_in ? a.left_in[gw] : 0;
+    if (a.left_in && !__syncthreads_or(rest)) return;
+    if (lane < 4) { s_top[wib][lane] = lane == 0 ? rest : 0; s_wc[wib][lane] = 0u; }
     SmemTables T = stage_tables(a.t, smem);   // ends with __syncthreads()
     if (lane == 0) { s_time[wib][0] = globaltimer_ns(); s_time[wib][1] = 0ull; }
 
-    const long long gw = (long long)blockIdx.x * (blockDim.x >> 5) + wib;
-    CtxT<BL> c{a, T, a.stacks + (size_t)gw * a.nstk * a.cap, s_top[wib], s_st,
-          1.f / a.dx, 1.f / a.dy, 1.f / a.dz, a.nx * a.dx, a.ny * a.dy, a.nz * a.dz, true};
+    CtxT<BL> c{a, T, a.stacks + (size_t)gw * a.nstk * a.cap, s_top[wib], &s_st,
+          1.f / a.dx, 1.f / a.dy, 1.f / a.dz, a.nx * a.dx, a.ny * a.dy, a.nz * a.dz};
     const unsigned lt = (1u << lane) - 1u;
     const int src_mode = a.src.particle == 0 ? 0 : 1;
     // a phase-space source mixes particle types: warps of either type draw from it, and a
@@ -607,153 +688,231 @@ __global__ void __maxnreg__(NREG) k_transport(const __grid_constant__ TransportA
     // with switch_high >= cap, switching on stack size is off (stacks may then overflow, which
     // is reported); otherwise a warp also switches when another stack nears its capacity
     const int emergency = a.switch_high < a.cap ? a.cap - 128 : 0x7FFFFFFF;
-    bool active = false, just_switched = false;
-    Lane p;
-    unsigned n_fict = 0, n_hfict = 0;
-    // per-warp scheduler counters live in shared memory (iterations, photon and charged lane-steps),
-    // and per-history counts go straight to the block's statistics: none of them takes a register
-    // under the register cap
-    unsigned long long* wc = s_wc[wib];
-    if (lane == 0) { wc[0] = 0ull; wc[1] = 0ull; wc[2] = 0ull; }
+    // most iterations only step: nothing to schedule while few lanes are free and no stack is large
+    const int plan_free = min(a.refill_min, 32 - a.switch_low), plan_top = min(a.switch_high, emergency);
+    // per-warp scheduler counters live in shared memory (iterations, photon and charged lane-steps):
+    // none of them takes a register under the register cap
+    unsigned int* wc = s_wc[wib];
 
     // modes (= stacks): 0 photons, 1 charged particles (at or above e_split when there are
     // three stacks), 2 charged particles below e_split
+    bool active = false, just_switched = false;
+    Lane p;
+    int left = 0;                // photons this warp leaves to fly_chains
     for (;;) {
         __syncwarp();
-        int top0 = min(c.top[0], a.cap), top1 = min(c.top[1], a.cap), top2 = a.nstk == 3 ? min(c.top[2], a.cap) : 0;
+        const int4 tops = *reinterpret_cast<const int4*>(c.top);
+        int fate = LIVE;
+        Pend sec;
+        sec.type = -1;
         unsigned act = __ballot_sync(FULL, active);
-        int nfree = 32 - __popc(act);
-        // refill when enough lanes are free: the refill code runs on the free lanes only,
-        // so waiting for several of them spreads its cost
-        if (nfree >= a.refill_min || nfree == 32) {
-            int topm = mode == 0 ? top0 : (mode == 1 ? top1 : top2);
-            int rank = __popc(~act & lt);
-            int take = min(nfree, topm);
-            if (!active && rank < take) {
-                pop_lane(c, mode, topm - 1 - rank, p);
-                active = true;
-            }
-            int want = nfree - take;
-            if (want > 0 && (ps_src || mode == src_mode) && !src_done) {
-                unsigned long long base = 0;
-                if (lane == 0) base = atomicAdd(a.hist_counter, (unsigned long long)want);
-                base = __shfl_sync(FULL, base, 0);
-                if (base + want >= a.count) {
-                    src_done = true;
-                    if (lane == 0) s_time[wib][1] = globaltimer_ns();
+        if (32 - __popc(act) >= plan_free || max(tops.x, max(tops.y, tops.z)) >= plan_top) {
+            int top0 = min(tops.x, a.cap), top1 = min(tops.y, a.cap), top2 = a.nstk == 3 ? min(tops.z, a.cap) : 0;
+            int nfree = 32 - __popc(act);
+            // refill when enough lanes are free: the refill code runs on the free lanes only,
+            // so waiting for several of them spreads its cost
+            if (nfree >= a.refill_min || nfree == 32) {
+                int topm = mode == 0 ? top0 : (mode == 1 ? top1 : top2);
+                int rank = __popc(~act & lt);
+                int take = min(nfree, topm);
+                if (!active && rank < take) {
+                    pop_lane(c, mode, topm - 1 - rank, p);
+                    active = true;
                 }
-                int r2 = rank - take;
-                if (!active && r2 >= 0 && r2 < want && base + r2 < a.count) {
-                    stat_add(c, ST_HISTORIES, 1);
-                    bool in;
-                    if constexpr (BL) in = init_beamlet(a, base + r2, p);
-                    else if constexpr (ps_src) in = init_phase_space(a, a.first + base + r2, p);
-                    else in = init_primary(a, a.first + base + r2, p);
-                    float ecut = p.type == PHOTON ? a.pp.e_abs_g : a.pp.e_abs_e;
-                    if (!in) {
-                        stat_add(c, ST_MISSED, 1);
-                        stat_add(c, ST_E_MISS, fx(p.E));
-                    } else if constexpr (ps_src) {
-                        stat_add(c, ST_E_IN, fx(p.E));
-                        const bool charged = p.type != PHOTON;
-                        if (p.E >= ecut && !(charged && (a.pp.flags & 8))) {
-                            const int target = charged ? charged_stack(a, p.E) : 0;
-                            if (target == mode) active = true;
-                            else push_lane(c, target, p);
-                        } else if (charged) {
-                            absorb_charged(c, p);       // positrons annihilate
+                int want = min(nfree - take, a.src_share);
+                if (want > 0 && (ps_src || mode == src_mode) && !src_done) {
+                    unsigned long long base = 0;
+                    if (lane == 0) base = atomicAdd(a.hist_counter, (unsigned long long)want);
+                    base = __shfl_sync(FULL, base, 0);
+                    if (base + want >= a.count) {
+                        src_done = true;
+                        if (lane == 0) s_time[wib][1] = globaltimer_ns();
+                    }
+                    int r2 = rank - take;
+                    if (!active && r2 >= 0 && r2 < want && base + r2 < a.count) {
+                        count(c, ST_HISTORIES);
+                        bool in;
+                        if constexpr (BL) in = init_beamlet(a, base + r2, p);
+                        else if constexpr (ps_src) in = init_phase_space(a, a.first + base + r2, p);
+                        else in = init_primary(a, a.first + base + r2, p);
+                        if (!in) {
+                            count(c, ST_MISSED);
+                            count_rare(c, ST_E_MISS, fx(p.E));
                         } else {
-                            deposit(c, p, p.ix, p.iy, p.iz, p.E);
+                            add_energy(c, BE_IN, fx(p.E));
+                            const bool charged = p.type != PHOTON;
+                            if (!(p.E >= (charged ? a.pp.e_abs_e : a.pp.e_abs_g)) || (charged && (a.pp.flags & 8))) fate = ABSORBED;
+                            else if (ps_src && (charged ? charged_stack(a, p.E) : 0) != mode) fate = MOVED;
+                            else active = true;
                         }
-                    } else {
-                        stat_add(c, ST_E_IN, fx(p.E));
-                        if (p.E >= ecut && !(p.type != PHOTON && (a.pp.flags & 8))) active = true;
-                        else deposit(c, p, p.ix, p.iy, p.iz, p.E);
                     }
                 }
+                __syncwarp();
+                if (lane == 0) {
+                    c.top[mode] = topm - take;
+                    if (wc[0] >= FLUSH_ITERS) flush_stats(a, s_st, wc);
+                }
+                __syncwarp();
+                if (mode == 0) top0 = topm - take; else if (mode == 1) top1 = topm - take; else top2 = topm - take;
+                act = __ballot_sync(FULL, active);
+                if (__any_sync(FULL, fate != LIVE)) {
+                    if (fate != LIVE) finish(c, p, sec, fate);
+                    if (act == 0) continue;
+                    fate = LIVE;
+                    __syncwarp();
+                }
             }
-            __syncwarp();
-            if (lane == 0) c.top[mode] = topm - take;
-            __syncwarp();
-            if (mode == 0) top0 = topm - take; else if (mode == 1) top1 = topm - take; else top2 = topm - take;
-            act = __ballot_sync(FULL, active);
-        }
-        int nact = __popc(act);
-        const int topm = mode == 0 ? top0 : (mode == 1 ? top1 : top2);
-        bool m_avail = topm > 0 || ((ps_src || mode == src_mode) && !src_done);
-        // the other mode: the fullest other stack that has work (or that the source feeds)
-        int other = -1, topo = 0;
+            int nact = __popc(act);
+            const int topm = mode == 0 ? top0 : (mode == 1 ? top1 : top2);
+            bool m_avail = topm > 0 || ((ps_src || mode == src_mode) && !src_done);
+            // the other mode: the fullest other stack that has work (or that the source feeds)
+            int other = -1, topo = 0;
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const int tk = k == 0 ? top0 : (k == 1 ? top1 : top2);
-            if (k != mode && k < a.nstk && (tk > 0 || ((ps_src || k == src_mode) && !src_done)) &&
-                (other < 0 || tk > topo)) {
-                other = k;
-                topo = tk;
+            for (int k = 0; k < 3; ++k) {
+                const int tk = k == 0 ? top0 : (k == 1 ? top1 : top2);
+                if (k != mode && k < a.nstk && (tk > 0 || ((ps_src || k == src_mode) && !src_done)) &&
+                    (other < 0 || tk > topo)) {
+                    other = k;
+                    topo = tk;
+                }
             }
+            const bool o_avail = other >= 0;
+            if (nact == 0) {
+                if (m_avail) continue;
+                if (o_avail) { mode = other; continue; }
+                break;
+            }
+            bool sw = false;
+            if (o_avail && !just_switched) {     // at most one switch between two steps
+                // the other group must be strictly larger (or the source), so a switch is never undone at once
+                if (!m_avail && nact <= a.switch_low && (topo > nact || (!ps_src && other == src_mode && !src_done)))
+                    sw = true;
+                else if (topo >= a.switch_high && topo >= 2 * (nact + topm)) sw = true;
+                // the other stack is within one iteration's pushes (32 lanes x 3 secondaries, plus
+                // 32 refilled primaries) of its capacity: switch before it can overflow
+                else if (topo >= emergency && topo > topm) sw = true;
+            }
+            // few photons left in the warp, nothing to refill from and one of them in a long chain of
+            // fictitious events: the warp ends and leaves them to k_chains, after the other stacks' work
+            const bool chain = a.left_out && !sw && mode == 0 && !m_avail && nact <= CHAIN_LANES && !just_switched &&
+                               __any_sync(FULL, active && p.steps >= CHAIN_STEPS && p.r.n < CHAIN_MAX_N);
+            if (sw || chain) {
+                if (active) {
+                    push(c, mode ? charged_stack(a, p.E) : 0, p, p.E, p.u, p.v, p.w, p.type, p.r.sub, p.r.n);
+                    active = false;
+                }
+                if (chain && !o_avail) { left = nact; break; }
+                mode = other;
+                just_switched = true;
+                continue;
+            }
+            just_switched = false;
         }
-        const bool o_avail = other >= 0;
-        if (nact == 0) {
-            if (m_avail) continue;
-            if (o_avail) { mode = other; continue; }
-            break;
-        }
-        bool sw = false;
-        if (o_avail && !just_switched) {     // at most one switch between two steps
-            // the other group must be strictly larger (or the source), so a switch is never undone at once
-            if (!m_avail && nact <= a.switch_low && (topo > nact || (!ps_src && other == src_mode && !src_done)))
-                sw = true;
-            else if (topo >= a.switch_high && topo >= 2 * (nact + topm)) sw = true;
-            // the other stack is within one iteration's pushes (32 lanes x 3 secondaries, plus
-            // 32 refilled primaries) of its capacity: switch before it can overflow
-            else if (topo >= emergency && topo > topm) sw = true;
-        }
-        if (sw) {
-            if (active) { push_lane(c, mode ? charged_stack(a, p.E) : 0, p); active = false; }
-            mode = other;
-            just_switched = true;
-            continue;
-        }
-        just_switched = false;
         if (lane == 0) {
-            wc[0] += 1ull;
-            wc[mode ? 2 : 1] += (unsigned long long)nact;
+            atomicAdd(wc, 1u);
+            atomicAdd(wc + (mode ? 2 : 1), (unsigned)__popc(act));
         }
         if (active) {
-            if constexpr (XV) active = mode ? charged_step_cross(c, p, n_hfict) : photon_step(c, p, n_fict);
-            else active = mode ? charged_step(c, p, n_hfict) : photon_step(c, p, n_fict);
-            if (active && ++p.steps > STEP_LIMIT) {
-                atomicOr(a.err, ERR_LIMIT);
-                stat_add(c, ST_DROPPED, 1);
-                stat_add(c, ST_E_DROPPED, fx(p.E));
-                active = false;
+            if (mode) {
+                if constexpr (XV) fate = charged_step_cross(c, p, sec);
+                else fate = charged_step(c, p, sec);
+            } else {
+                fate = photon_step(c, p, sec);
             }
-            if (!c.ok) {
+            if (fate == LIVE && ++p.steps > STEP_LIMIT) {
                 atomicOr(a.err, ERR_LIMIT);
-                c.ok = true;
+                count_rare(c, ST_DROPPED, 1);
+                count_rare(c, ST_E_DROPPED, fx(p.E));
+                fate = GONE;
             }
+            active = fate == LIVE;
+            if (fate > GONE || sec.type >= 0) finish(c, p, sec, fate);
         }
     }
-    // per-warp and per-lane statistics
-    atomicAdd(s_st + ST_FICT, (unsigned long long)n_fict);
-    atomicAdd(s_st + ST_HARD_FICT, (unsigned long long)n_hfict);
+    __syncwarp();
     if (lane == 0) {
-        atomicAdd(s_st + ST_WARP_ITERS, wc[0]);
-        atomicAdd(s_st + ST_LANES_PHOTON, wc[1]);
-        atomicAdd(s_st + ST_LANES_CHARGED, wc[2]);
+        flush_stats(a, s_st, wc);
+        if (a.left_out) {
+            a.left_out[gw] = left;
+            if (left) atomicAdd(a.n_left_out, 1ull);
+        }
         // tail: how long this warp ran on its own stacks after the source ran dry
         const unsigned long long t_end = globaltimer_ns(), t0 = s_time[wib][0];
         const unsigned long long ts = s_time[wib][1] ? s_time[wib][1] : t0;
-        atomicAdd(s_st + ST_WARP_NS, t_end - t0);
-        atomicAdd(s_st + ST_WARPS, 1ull);
-        atomicAdd(s_st + ST_TAIL_NS, t_end - ts);
-        atomicMax(a.stats + ST_T_START_INV, ~t0);
-        atomicMax(a.stats + ST_T_SRC_INV, ~ts);
+        atomicAdd(a.stats + ST_WARP_NS, t_end - t0);
+        atomicAdd(a.stats + ST_TAIL_NS, t_end - ts);
+        if (!a.left_in) {
+            atomicAdd(a.stats + ST_WARPS, 1ull);
+            atomicMax(a.stats + ST_T_START_INV, ~t0);
+            atomicMax(a.stats + ST_T_SRC_INV, ~ts);
+        }
         atomicMax(a.stats + ST_T_END, t_end);
     }
-    __syncthreads();
-    for (int i = threadIdx.x; i < ST_COUNT; i += blockDim.x)
-        if (s_st[i]) atomicAdd(a.stats + i, s_st[i]);
+}
+
+// Long Woodcock chains. A photon of a few tens of keV in air or lung flies against the majorant of
+// the densest bone: hundreds to thousands of fictitious events in a row, one a step, in a warp whose
+// other lanes have run dry; a short run then waited for a handful of such photons (half of the 3.6 ms
+// of 1.3e6 6 MV photons on a CT-like 128^3 phantom). Between two real events the flights of a photon
+// differ only in their random block and position, so a whole warp works on one photon here: lane j
+// draws flight j of the next 32, all lanes follow the positions (the same chain of FMAs as the steps',
+// so the same bits), each lane judges its own flight, and the photon moves past the fictitious ones
+// before the first that is not; that one is left to photon_step in the resumed launch. One block per
+// warp of the transport launch, one warp per photon; tables are read from global memory (L2).
+__global__ void __launch_bounds__(32 * CHAIN_LANES) k_chains(const __grid_constant__ TransportArgs a)
+{
+    if (!*a.n_left_in) return;
+    const int lane = threadIdx.x & 31, i = threadIdx.x >> 5;
+    if (i >= a.left_in[blockIdx.x]) return;
+    PRec* rec = a.stacks + (size_t)blockIdx.x * a.nstk * a.cap + i;
+    PRec p = *rec;
+    const float Lx = a.nx * a.dx, Ly = a.ny * a.dy, Lz = a.nz * a.dz;
+    const float inv_dx = 1.f / a.dx, inv_dy = 1.f / a.dy, inv_dz = 1.f / a.dz;
+    const EIdx ei = e_index(p.E);
+    const float lnmaj = lerp1(__ldg(a.t.phmaj + ei.i), __ldg(a.t.phmaj + ei.i + 1), ei.f);
+    if (lnmaj < -1e29f) return;
+    const float mumax = __expf(lnmaj);
+    unsigned flights = 0;
+    for (int done = 32; done == 32 && p.n < CHAIN_MAX_N;) {
+        const uint32_t blk = (p.n + 3u) >> 2;
+        const uint4 b = philox4x32_10(make_uint4(blk + (uint32_t)lane, p.h0, p.h1, p.sub), a.key0, a.key1);
+        const float s = -__logf(u01(b.x)) / mumax, u_real = u01(b.y);
+        float x = p.x, y = p.y, z = p.z, mx = x, my = y, mz = z;
+#pragma unroll 8
+        for (int k = 0; k < 32; ++k) {
+            const float sk = __shfl_sync(FULL, s, k);
+            x = fmaf(sk, p.u, x);
+            y = fmaf(sk, p.v, y);
+            z = fmaf(sk, p.w, z);
+            if (k == lane) { mx = x; my = y; mz = z; }
+        }
+        bool fict = mx >= 0.f && my >= 0.f && mz >= 0.f && mx <= Lx && my <= Ly && mz <= Lz;
+        if (fict) {
+            const int ix = min((int)(mx * inv_dx), a.nx - 1), iy = min((int)(my * inv_dy), a.ny - 1),
+                      iz = min((int)(mz * inv_dz), a.nz - 1);
+            const int vox = ix + a.nx * (iy + a.ny * iz);
+            const float rho = __ldg(a.density + vox);
+            const int m = __ldg(a.material + vox);
+            const float mu = rho * __expf(lerp1(__ldg(&a.t.ph[m * NE + ei.i].x), __ldg(&a.t.ph[m * NE + ei.i + 1].x), ei.f));
+            fict = u_real * mumax >= mu;
+        }
+        const unsigned stop = __ballot_sync(FULL, !fict);
+        done = stop ? __ffs(stop) - 1 : 32;
+        if (done) {
+            p.x = __shfl_sync(FULL, mx, done - 1);
+            p.y = __shfl_sync(FULL, my, done - 1);
+            p.z = __shfl_sync(FULL, mz, done - 1);
+            p.n = (blk + (uint32_t)done) << 2;
+            flights += (unsigned)done;
+        }
+    }
+    __syncwarp();                              // every lane has read the record
+    if (lane == 0) {
+        rec->x = p.x; rec->y = p.y; rec->z = p.z;
+        rec->n = p.n;
+        atomicAdd(a.stats + ST_FICT, (unsigned long long)flights);
+        atomicAdd(a.stats + ST_LANES_PHOTON, (unsigned long long)flights);
+    }
 }
 
 }  // namespace
@@ -808,7 +967,7 @@ int transport_max_blocks_per_sm(int threads, size_t smem, int nreg)
     return occupancy<false, false, 80>(threads, smem);
 }
 
-cudaError_t launch_transport(const TransportArgs& a, int blocks, int threads, size_t smem, cudaStream_t s, int nreg)
+static cudaError_t launch_one(const TransportArgs& a, int blocks, int threads, size_t smem, cudaStream_t s, int nreg)
 {
     if (a.pp.flags & FLAG_CROSS_VOXELS) {
         // voxel-crossing electron steps: analytic single-beam source only (callers check)
@@ -820,6 +979,28 @@ cudaError_t launch_transport(const TransportArgs& a, int blocks, int threads, si
     if (a.beamlets) return launch_source<true, false>(a, blocks, threads, smem, s, nreg);
     if (a.ps) return launch_source<false, true>(a, blocks, threads, smem, s, nreg);
     return launch_source<false, false>(a, blocks, threads, smem, s, nreg);
+}
+
+cudaError_t launch_transport(const TransportArgs& args, int blocks, int threads, size_t smem, cudaStream_t s, int nreg)
+{
+    TransportArgs a = args;
+    // A run with fewer histories than lanes is spread over all warps: a chain of steps takes longer in
+    // a fuller warp, and whole warps would stay without work (5e4 electrons of 15 MeV on 4864 warps:
+    // 1.30 ms with 32 histories a draw, 1.06 ms with 11).
+    const unsigned long long warps = (unsigned long long)blocks * (threads / 32), per = (a.count + warps - 1) / warps;
+    a.src_share = (int)std::min<unsigned long long>(32, std::max<unsigned long long>(1, per));
+    int* left = a.left_out;                      // one count per warp; null: no room for it, every warp finishes its photons
+    a.n_left_out = a.hist_counter + 1;
+    cudaError_t e = launch_one(a, blocks, threads, smem, s, nreg);
+    if (!left || e != cudaSuccess) return e;
+    // the photons that warps left in long chains (usually none: both launches then return at once)
+    a.left_in = left;
+    a.n_left_in = a.hist_counter + 1;
+    a.left_out = nullptr;
+    a.count = 0;
+    k_chains<<<(unsigned)warps, 32 * CHAIN_LANES, 0, s>>>(a);
+    e = cudaGetLastError();
+    return e != cudaSuccess ? e : launch_one(a, blocks, threads, smem, s, nreg);
 }
 
 }  // namespace ocmc
