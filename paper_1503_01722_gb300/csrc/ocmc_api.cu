@@ -325,6 +325,8 @@ ocmc_status ocmc_init(ocmc_ctx** out, int device, const ocmc_params* p)
     if (r == cudaSuccess) r = dalloc(&c->t.scratch, MAX_STAGED * NE);
     if (r == cudaSuccess) r = dalloc(&c->t.rho_max, MAX_STAGED);
     if (r == cudaSuccess) r = dalloc(&c->t.mats, MAX_STAGED);
+    if (r == cudaSuccess) r = dalloc(&c->t.mc, MAX_STAGED);
+    if (r == cudaSuccess) r = dalloc(&c->t.elem, MAX_STAGED * MAX_ELEM);
     {
         MatDef d[NMAT_DEFAULT];
         material_defs(d);
@@ -806,7 +808,7 @@ void ocmc_destroy(ocmc_ctx* c)
     dfree(&c->d_counter); dfree(&c->d_sum); dfree(&c->d_err); dfree(&c->d_stacks); dfree(&c->d_left); dfree(&c->d_dose);
     dfree(&c->d_sigma); dfree(&c->d_invnb);
     dfree(&c->t.ph); dfree(&c->t.el); dfree(&c->t.el2); dfree(&c->t.phmaj); dfree(&c->t.elmaj); dfree(&c->t.rinv); dfree(&c->t.msA);
-    dfree(&c->t.rmeta); dfree(&c->t.msc); dfree(&c->t.scratch); dfree(&c->t.rho_max);
+    dfree(&c->t.rmeta); dfree(&c->t.msc); dfree(&c->t.scratch); dfree(&c->t.rho_max); dfree(&c->t.mc); dfree(&c->t.elem); dfree(&c->t.mats);
     dfree(&c->d_bl); dfree(&c->d_bl_prefix); dfree(&c->d_bl_offs); dfree(&c->d_bl_caps); dfree(&c->d_bl_nnz);
     dfree(&c->d_bl_over); dfree(&c->d_bl_keys); dfree(&c->d_bl_vals); dfree(&c->d_dense); dfree(&c->d_chunks);
     dfree(&c->d_oidx); dfree(&c->d_odose); dfree(&c->d_oraw); dfree(&c->d_ps);

@@ -64,6 +64,9 @@ enum Stat {
 
 // Tables in global memory, one row per staged material m < n_mat (capacity MAX_STAGED).
 struct MatDef;
+struct MatConst {
+    double ne, photo, pairZ, S1, S2, I, dC, dX0, dX1, dA;
+};
 struct Tables {
     int n_mat;      // staged materials (table rows)
     MatDef* mats;   // their definitions (device, MAX_STAGED)
@@ -77,6 +80,8 @@ struct Tables {
     float* rmeta;   // n_mat*2: lnR0, 1/dlnR
     float* msc;     // n_mat*2: bremsstrahlung screening sums S1, S2 (per gram)
     double* scratch;        // n_mat*NE interval ranges
+    MatConst* mc;           // n_mat: per-gram constants of the compositions
+    double2* elem;          // n_mat*MAX_ELEM: per element, atoms per gram and cube root of Z
     unsigned int* rho_max;  // n_mat, float bits of the max density per material
 };
 

@@ -193,6 +193,10 @@ extern "C" ocmc_status ocmc_run_noalloc(int device, int nx, int ny, int nz, cons
         return M.fail(OCMC_ERR_ARG, "launch shape needs more secondary-stack scratch than the 64 MiB static array "
                                    "(lower stack_capacity, block_threads or blocks_per_sm)");
     PRec* stacks = cv.take<PRec>((size_t)blocks * (threads / 32) * nstk * cap);
+    // the table build's own scratch: it is done with it before the transport uses the stacks
+    static_assert(2 * 64 * sizeof(PRec) >= NMAT_DEFAULT * (MAX_ELEM * sizeof(double2) + sizeof(MatConst)), "fits one warp's stacks");
+    t.elem = reinterpret_cast<double2*>(stacks);
+    t.mc = reinterpret_cast<MatConst*>(t.elem + NMAT_DEFAULT * MAX_ELEM);
     const size_t left_bytes = (size_t)blocks * (threads / 32) * sizeof(int);
     int* left = cv.used + left_bytes <= NOALLOC_BYTES ? cv.take<int>(left_bytes / sizeof(int)) : nullptr;
 
