@@ -87,9 +87,10 @@ typedef struct {
                             /* stack and source are empty moves to another stack   */
     uint32_t stream_tag;    /* XORed into the high word of every history's random  */
                             /* stream (0); 0x80000000|b reproduces beamlet b       */
-    float beamlet_capacity_scale; /* scales the pilot estimate of beamlet table    */
-                            /* sizes (0 = 1); tables that fill up are enlarged and */
-                            /* the run repeated, so any value gives the same dose  */
+    float beamlet_capacity_scale; /* > 0: beamlets use hash tables, their pilot    */
+                            /* size estimate times this; tables that fill up are   */
+                            /* enlarged and the run repeated, so any value gives   */
+                            /* the same dose (0: dense tallies where they fit)     */
     int32_t refill_min;     /* free lanes a warp waits for before refilling (0=6)  */
     int32_t max_registers;  /* register cap of the transport kernel: 56, 64 or 80; */
                             /* 0 = 64 (with 1024-thread blocks)                    */
@@ -270,8 +271,8 @@ void ocmc_destroy(ocmc_ctx* ctx);
 
 /* ---- batched beamlets --------------------------------------------------------
  * Many small beams transported together in one persistent launch, captured once in
- * a CUDA graph and replayed, each beamlet with its own sparse tally (an open-
- * addressing hash of voxel -> int64 energy). Extends the paper's per-source loop
+ * a CUDA graph and replayed, each beamlet with its own tally (dense where the device
+ * has room, else an open-addressing hash of voxel -> int64 energy). Extends the paper's per-source loop
  * (Sec. 2.2.1, Table 1) to a queue of sources; the per-history physics is the same.
  * Beamlet b's histories use random streams whose history high word is
  * 0x80000000 | b, so a single-beam run with stream_tag = 0x80000000 | b, the same
@@ -291,10 +292,12 @@ ocmc_status ocmc_set_beamlets(ocmc_ctx* ctx, int particle, int n_bins, const flo
                               const float* weights_host, int n_beamlets, const ocmc_beamlet* beamlets_host);
 
 /* Transport every beamlet's histories with Philox key `seed` (replacing the
- * previous beamlet tallies). The first call after ocmc_set_beamlets sizes each
- * table from two pilot runs (distinct-voxel footprint at two history counts,
- * extrapolated as a power law) and captures the launch in a CUDA graph; later
- * calls replay it. A table that fills up is enlarged and the run repeated.
+ * previous beamlet tallies). Each beamlet has a dense tally where all of them take
+ * at most a quarter of the free device memory; otherwise, or when the parameters set
+ * beamlet_capacity_scale, the first call after ocmc_set_beamlets sizes a hash table
+ * per beamlet from two pilot runs (distinct-voxel footprint at two history counts,
+ * extrapolated as a power law). The first call captures the launch in a CUDA graph;
+ * later calls replay it. A table that fills up is enlarged and the run repeated.
  * Synchronises cuda_stream. */
 ocmc_status ocmc_run_beamlets(ocmc_ctx* ctx, uint64_t seed, void* cuda_stream);
 
@@ -304,6 +307,15 @@ ocmc_status ocmc_run_beamlets(ocmc_ctx* ctx, uint64_t seed, void* cuda_stream);
  * *nnz receives the number of non-zero voxels. */
 ocmc_status ocmc_get_beamlet_dose(ocmc_ctx* ctx, int beamlet, int32_t* idx_host, float* dose_host,
                                   int64_t* raw_host, int64_t capacity, int64_t* nnz);
+
+/* Every beamlet's list at once, in beamlet order: indptr_host[b] (n_beamlets + 1 of them) is the position of
+ * beamlet b's first entry, indptr_host[n_beamlets] their number; ocmc_get_beamlet_entries then writes the
+ * lists one after the other, the entries of ocmc_get_beamlet_dose, into arrays of at least that many
+ * elements (any of the three may be NULL). OCMC_ERR_STATE without a run or before the sizes were asked for,
+ * OCMC_ERR_ARG if capacity is too small. */
+ocmc_status ocmc_get_beamlet_sizes(ocmc_ctx* ctx, int64_t* indptr_host);
+ocmc_status ocmc_get_beamlet_entries(ocmc_ctx* ctx, int32_t* idx_host, float* dose_host, int64_t* raw_host,
+                                     int64_t capacity);
 
 /* Autotuner: times the transport of `pilot_histories` histories of the current
  * source for a set of launch shapes (threads per block, type-switch thresholds,

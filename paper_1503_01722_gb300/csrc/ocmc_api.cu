@@ -223,7 +223,8 @@ ocmc_status ctx_ensure_stacks(ocmc_ctx* c, size_t warps, size_t records_per_warp
 {
     const size_t need = warps * records_per_warp;
     if (need > c->stack_records || warps > c->left_warps) {
-        if (c->ran || c->last_stream) cudaDeviceSynchronize();
+        if (c->ran || c->bl_ran || c->last_stream) cudaDeviceSynchronize();
+        c->bl_graph_valid = false;              // a captured beamlet launch holds the old pointers
         if (need > c->stack_records) {
             c->stack_records = 0;
             CK(dalloc(&c->d_stacks, need), "stack allocation");
@@ -444,6 +445,8 @@ ocmc_status ocmc_create_phantom(ocmc_ctx* c, int nx, int ny, int nz, const float
     }
     CK(cudaSetDevice(c->device), "cudaSetDevice");
     if (c->last_stream || c->ran) cudaDeviceSynchronize();
+    c->bl_graph_valid = false;     // a captured beamlet launch holds the old phantom's geometry and pointers
+    if (n != c->nvox) c->bl_sized = c->bl_ran = c->bl_counted = false;   // as its tallies hold the old voxels
     if (n != c->nvox) {
         CK(dalloc(&c->d_density, n), "phantom allocation");
         CK(dalloc(&c->d_material, n), "phantom allocation");
@@ -811,6 +814,8 @@ void ocmc_destroy(ocmc_ctx* c)
     dfree(&c->t.rmeta); dfree(&c->t.msc); dfree(&c->t.scratch); dfree(&c->t.rho_max); dfree(&c->t.mc); dfree(&c->t.elem); dfree(&c->t.mats);
     dfree(&c->d_bl); dfree(&c->d_bl_prefix); dfree(&c->d_bl_offs); dfree(&c->d_bl_caps); dfree(&c->d_bl_nnz);
     dfree(&c->d_bl_over); dfree(&c->d_bl_keys); dfree(&c->d_bl_vals); dfree(&c->d_dense); dfree(&c->d_chunks);
+    dfree(&c->d_bl_tally); dfree(&c->d_bl_offsets); dfree(&c->d_bl_base); dfree(&c->d_bl_scale);
+    if (c->d_bl_out) cudaFree(c->d_bl_out);
     dfree(&c->d_oidx); dfree(&c->d_odose); dfree(&c->d_oraw); dfree(&c->d_ps);
     if (c->bl_exec) cudaGraphExecDestroy(c->bl_exec);
     if (c->bl_capture) cudaStreamDestroy(c->bl_capture);

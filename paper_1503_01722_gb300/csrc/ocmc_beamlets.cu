@@ -67,7 +67,7 @@ ocmc_status upload_beamlets(ocmc_ctx* c, const std::vector<unsigned long long>& 
         "beamlet upload");
     BCK(cudaMemcpy(c->d_bl_offs, offs.data(), sizeof(unsigned long long) * n, cudaMemcpyHostToDevice), "upload");
     BCK(cudaMemcpy(c->d_bl_caps, capv.data(), sizeof(unsigned int) * n, cudaMemcpyHostToDevice), "upload");
-    if (off > c->bl_slots) {
+    if (!c->bl_dense && off > c->bl_slots) {
         BCK(realloc_dev(&c->d_bl_keys, off), "beamlet table allocation");
         BCK(realloc_dev(&c->d_bl_vals, off), "beamlet table allocation");
         c->bl_slots = off;
@@ -99,6 +99,8 @@ ocmc_status beamlet_args(ocmc_ctx* c, unsigned long long total, uint64_t seed, T
     a.beamlets = c->d_bl;
     a.bl_prefix = c->d_bl_prefix;
     a.n_beamlets = c->bl_n;
+    a.bl_dense = c->bl_dense;
+    if (c->bl_dense) a.tally = c->d_bl_tally;
     a.bl_keys = c->d_bl_keys;
     a.bl_vals = c->d_bl_vals;
     a.bl_overflow = c->d_bl_over;
@@ -122,8 +124,13 @@ ocmc_status beamlet_args(ocmc_ctx* c, unsigned long long total, uint64_t seed, T
 cudaError_t enqueue_beamlets(ocmc_ctx* c, const TransportArgs& a, size_t slots, int threads, int blocks, int nreg,
                              cudaStream_t s)
 {
-    cudaError_t e = cudaMemsetAsync(c->d_bl_keys, 0xFF, sizeof(unsigned int) * slots, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->d_bl_vals, 0, sizeof(unsigned long long) * slots, s);
+    cudaError_t e = cudaSuccess;
+    if (c->bl_dense) {
+        e = cudaMemsetAsync(c->d_bl_tally, 0, sizeof(unsigned long long) * (size_t)c->bl_n * c->nvox, s);
+    } else {
+        e = cudaMemsetAsync(c->d_bl_keys, 0xFF, sizeof(unsigned int) * slots, s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(c->d_bl_vals, 0, sizeof(unsigned long long) * slots, s);
+    }
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_bl_over, 0, sizeof(unsigned int) * c->bl_n, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_counter, 0, RUN_COUNTERS * sizeof(unsigned long long), s);
     // a beamlet run replaces its tallies, so its statistics describe that run alone
@@ -146,6 +153,29 @@ ocmc_status read_overflow(ocmc_ctx* c, std::vector<unsigned int>& over)
 // every occupied slot it passes, and on GB300 the 512-beamlet CT run took 219.8 ms at 0.7,
 // 183.9 ms at 0.35 and 180.7 ms at 0.175 (measured), at twice and four times the table memory.
 constexpr double BL_LOAD = 0.35;
+
+// Dense tallies for the current beamlets and phantom? A pencil beam's voxels lie together, so its dense
+// tally needs no probing and stays in L2 while it is hit (64 beamlets on a 128x128x96 grid: 11.8 ms a run
+// against 13.5 with hash tables and 4 ms of pilot runs to size them; 192 beamlets on 256x256x128: 46.5
+// against 61 ms), and its sparse list is a plain stream over it. It costs 8 bytes a voxel and beamlet to
+// clear and to read back, 2 ms each for 13 GB, so the tallies may take a quarter of the free memory;
+// beyond that, or when the caller scales the tables, hash tables.
+bool dense_fits(ocmc_ctx* c)
+{
+    if (c->p.beamlet_capacity_scale > 0.f) return false;
+    const size_t need = (size_t)c->bl_n * (size_t)c->nvox;
+    if (need <= c->bl_tally_n) return true;
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return false;
+    if (need > (free_b + 8 * c->bl_tally_n) / 4 / 8) return false;
+    c->bl_tally_n = 0;
+    if (realloc_dev(&c->d_bl_tally, need) != cudaSuccess) {
+        cudaGetLastError();                     // no room after all: the tables it is
+        return false;
+    }
+    c->bl_tally_n = need;
+    return true;
+}
 
 ocmc_status size_tables(ocmc_ctx* c, uint64_t seed, cudaStream_t s)
 {
@@ -183,7 +213,7 @@ ocmc_status size_tables(ocmc_ctx* c, uint64_t seed, cudaStream_t s)
             if (!any) break;
             if (attempt >= 8) return ctx_fail(c, OCMC_ERR_OVERFLOW, "beamlet pilot tables keep overflowing");
         }
-        BCK(launch_bl_count(c->d_bl_keys, c->d_bl_offs, c->d_bl_caps, n, c->d_bl_nnz, s), "footprint count");
+        BCK(launch_bl_count(c->d_bl_keys, nullptr, c->d_bl_offs, c->d_bl_caps, n, c->d_bl_nnz, s), "footprint count");
         BCK(cudaMemcpy(pass == 0 ? nnz2.data() : nnz1.data(), c->d_bl_nnz, sizeof(unsigned long long) * n,
                        cudaMemcpyDeviceToHost), "footprint count");
     }
@@ -276,6 +306,8 @@ ocmc_status ocmc_set_beamlets(ocmc_ctx* c, int particle, int n_bins, const float
         BCK(realloc_dev(&c->d_bl_caps, n_beamlets), "allocation");
         BCK(realloc_dev(&c->d_bl_nnz, n_beamlets), "allocation");
         BCK(realloc_dev(&c->d_bl_over, n_beamlets), "allocation");
+        BCK(realloc_dev(&c->d_bl_base, n_beamlets + 1), "allocation");
+        BCK(realloc_dev(&c->d_bl_scale, n_beamlets), "allocation");
     }
     c->bl_n = n_beamlets;
     c->bl_particle = particle;
@@ -301,9 +333,17 @@ ocmc_status ocmc_run_beamlets(ocmc_ctx* c, uint64_t seed, void* stream)
     ocmc_status st = ctx_ensure_tables(c, s);
     if (st != OCMC_OK) return st;
     if (!c->bl_sized) {
-        st = size_tables(c, seed, s);
-        if (st != OCMC_OK) return st;
+        c->bl_dense = dense_fits(c);
+        c->bl_graph_valid = false;
+        if (c->bl_dense) {
+            c->bl_cap.assign(c->bl_n, 1);       // no tables
+            c->bl_sized = true;
+        } else {
+            st = size_tables(c, seed, s);
+            if (st != OCMC_OK) return st;
+        }
     }
+    c->bl_counted = false;
     for (int attempt = 0;; ++attempt) {
         if (!c->bl_graph_valid || c->bl_graph_seed != seed) {
             st = capture_graph(c, seed);
@@ -315,6 +355,7 @@ ocmc_status ocmc_run_beamlets(ocmc_ctx* c, uint64_t seed, void* stream)
         BCK(cudaStreamSynchronize(s), "synchronize");
         c->timed = true;
         c->last_stream = s;
+        if (c->bl_dense) break;
         std::vector<unsigned int> over;
         st = read_overflow(c, over);
         if (st != OCMC_OK) return st;
@@ -347,6 +388,7 @@ ocmc_status ocmc_get_beamlet_dose(ocmc_ctx* c, int b, int32_t* idx, float* dose,
     if (capacity < 0) return ctx_fail(c, OCMC_ERR_ARG, "capacity must be >= 0");
     BCK(cudaSetDevice(c->device), "cudaSetDevice");
     if (c->out_cap < c->nvox) {
+        c->out_cap = 0;
         BCK(realloc_dev(&c->d_dense, c->nvox), "allocation");
         BCK(realloc_dev(&c->d_chunks, (c->nvox + 1023) / 1024 + 1), "allocation");
         BCK(realloc_dev(&c->d_oidx, c->nvox), "allocation");
@@ -358,8 +400,10 @@ ocmc_status ocmc_get_beamlet_dose(ocmc_ctx* c, int b, int32_t* idx, float* dose,
     for (int i = 0; i < b; ++i) off += c->bl_cap[i];
     cudaStream_t s = c->last_stream;
     const double scale = 1.0 / (268435456.0 * (double)c->dx * c->dy * c->dz * (double)c->bl_list[b].n_histories);
-    BCK(launch_bl_extract(c->d_bl_keys + off, c->d_bl_vals + off, c->bl_cap[b], c->nvox, c->d_dense, c->d_chunks,
-                          c->d_oidx, c->d_oraw, c->d_odose, c->d_density, scale, c->d_sum, s),
+    BCK(launch_bl_extract(c->bl_dense ? nullptr : c->d_bl_keys + off, c->bl_dense ? nullptr : c->d_bl_vals + off,
+                          c->bl_cap[b], c->nvox,
+                          c->bl_dense ? reinterpret_cast<long long*>(c->d_bl_tally) + (size_t)b * c->nvox : c->d_dense,
+                          c->d_chunks, c->d_oidx, c->d_oraw, c->d_odose, c->d_density, scale, c->d_sum, s),
         "beamlet extraction");
     unsigned long long n = 0;
     BCK(cudaMemcpyAsync(&n, c->d_sum, sizeof(n), cudaMemcpyDeviceToHost, s), "copy");
@@ -371,6 +415,86 @@ ocmc_status ocmc_get_beamlet_dose(ocmc_ctx* c, int b, int32_t* idx, float* dose,
         if (dose) BCK(cudaMemcpy(dose, c->d_odose, sizeof(float) * m, cudaMemcpyDeviceToHost), "copy");
         if (raw) BCK(cudaMemcpy(raw, c->d_oraw, sizeof(long long) * m, cudaMemcpyDeviceToHost), "copy");
     }
+    return OCMC_OK;
+}
+
+ocmc_status ocmc_get_beamlet_sizes(ocmc_ctx* c, int64_t* indptr)
+{
+    if (!c || !indptr) return ctx_fail(c, OCMC_ERR_ARG, "NULL argument");
+    if (!c->bl_ran) return ctx_fail(c, OCMC_ERR_STATE, "no beamlet run");
+    BCK(cudaSetDevice(c->device), "cudaSetDevice");
+    const int n = c->bl_n;
+    cudaStream_t s = c->last_stream;
+    if (!c->bl_counted) {
+        std::vector<unsigned long long> nnz(n);
+        if (c->bl_dense) {
+            const size_t chunks = (size_t)n * (size_t)((c->nvox + BL_CHUNK - 1) / BL_CHUNK);
+            if (chunks > c->bl_offsets_n) {
+                c->bl_offsets_n = 0;
+                BCK(realloc_dev(&c->d_bl_offsets, chunks), "allocation");
+                c->bl_offsets_n = chunks;
+            }
+            BCK(launch_bl_dense_count(c->d_bl_tally, n, c->nvox, c->d_bl_offsets, c->d_bl_nnz, s), "beamlet count");
+        } else {
+            BCK(launch_bl_count(c->d_bl_keys, c->d_bl_vals, c->d_bl_offs, c->d_bl_caps, n, c->d_bl_nnz, s), "beamlet count");
+        }
+        BCK(cudaMemcpyAsync(nnz.data(), c->d_bl_nnz, sizeof(unsigned long long) * n, cudaMemcpyDeviceToHost, s), "copy");
+        BCK(cudaStreamSynchronize(s), "synchronize");
+        c->bl_base.assign(n + 1, 0ull);
+        for (int b = 0; b < n; ++b) c->bl_base[b + 1] = c->bl_base[b] + nnz[b];
+        c->bl_counted = true;
+    }
+    for (int b = 0; b <= n; ++b) indptr[b] = (int64_t)c->bl_base[b];
+    return OCMC_OK;
+}
+
+ocmc_status ocmc_get_beamlet_entries(ocmc_ctx* c, int32_t* idx, float* dose, int64_t* raw, int64_t capacity)
+{
+    if (!c) return ctx_fail(c, OCMC_ERR_ARG, "NULL argument");
+    if (!c->bl_ran) return ctx_fail(c, OCMC_ERR_STATE, "no beamlet run");
+    if (!c->bl_counted) return ctx_fail(c, OCMC_ERR_STATE, "call ocmc_get_beamlet_sizes first");
+    const int n = c->bl_n;
+    const size_t total = (size_t)c->bl_base[n];
+    if (capacity < 0 || (size_t)capacity < total) return ctx_fail(c, OCMC_ERR_ARG, "capacity is below the number of entries");
+    if (total == 0) return OCMC_OK;
+    BCK(cudaSetDevice(c->device), "cudaSetDevice");
+    if (!c->bl_dense) {
+        for (int b = 0; b < n; ++b) {
+            int64_t k = 0;
+            const unsigned long long o = c->bl_base[b];
+            ocmc_status st = ocmc_get_beamlet_dose(c, b, idx ? idx + o : nullptr, dose ? dose + o : nullptr,
+                                                   raw ? raw + o : nullptr, (int64_t)(c->bl_base[b + 1] - o), &k);
+            if (st != OCMC_OK) return st;
+        }
+        return OCMC_OK;
+    }
+    cudaStream_t s = c->last_stream;
+    const size_t bytes = total * ((raw ? 8 : 0) + (idx ? 4 : 0) + (dose ? 4 : 0));
+    if (bytes > c->bl_out_bytes) {
+        if (c->d_bl_out) cudaFree(c->d_bl_out);
+        c->d_bl_out = nullptr;
+        c->bl_out_bytes = 0;
+        BCK(cudaMalloc(&c->d_bl_out, bytes), "allocation");
+        c->bl_out_bytes = bytes;
+    }
+    unsigned char* o = static_cast<unsigned char*>(c->d_bl_out);
+    long long* o_raw = raw ? reinterpret_cast<long long*>(o) : nullptr;
+    o += raw ? 8 * total : 0;
+    int* o_idx = idx ? reinterpret_cast<int*>(o) : nullptr;
+    o += idx ? 4 * total : 0;
+    float* o_dose = dose ? reinterpret_cast<float*>(o) : nullptr;
+    std::vector<double> scale(n);
+    for (int b = 0; b < n; ++b)
+        scale[b] = 1.0 / (268435456.0 * (double)c->dx * c->dy * c->dz * (double)c->bl_list[b].n_histories);
+    BCK(cudaMemcpyAsync(c->d_bl_base, c->bl_base.data(), sizeof(unsigned long long) * (n + 1), cudaMemcpyHostToDevice, s), "upload");
+    BCK(cudaMemcpyAsync(c->d_bl_scale, scale.data(), sizeof(double) * n, cudaMemcpyHostToDevice, s), "upload");
+    BCK(launch_bl_dense_gather(c->d_bl_tally, n, c->nvox, c->d_bl_offsets, c->d_bl_nnz, c->d_bl_base, c->d_bl_scale,
+                               c->d_density, o_idx, o_raw, o_dose, s),
+        "beamlet gather");
+    if (idx) BCK(cudaMemcpyAsync(idx, o_idx, 4 * total, cudaMemcpyDeviceToHost, s), "copy");
+    if (dose) BCK(cudaMemcpyAsync(dose, o_dose, 4 * total, cudaMemcpyDeviceToHost, s), "copy");
+    if (raw) BCK(cudaMemcpyAsync(raw, o_raw, 8 * total, cudaMemcpyDeviceToHost, s), "copy");
+    BCK(cudaStreamSynchronize(s), "synchronize");
     return OCMC_OK;
 }
 

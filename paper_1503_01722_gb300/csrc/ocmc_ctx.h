@@ -77,6 +77,18 @@ struct ocmc_ctx {
     unsigned int* d_bl_keys = nullptr;
     unsigned long long* d_bl_vals = nullptr;
     size_t bl_slots = 0;
+    // dense tallies, one of nvox per beamlet, where they fit (see dense_fits); then no tables are sized
+    bool bl_dense = false;
+    unsigned long long* d_bl_tally = nullptr;
+    size_t bl_tally_n = 0;                      // its capacity in voxels
+    unsigned int* d_bl_offsets = nullptr;       // per beamlet and chunk, of the last run once bl_counted
+    size_t bl_offsets_n = 0;
+    bool bl_counted = false;
+    std::vector<unsigned long long> bl_base;    // first entry of each beamlet in the sparse lists, and their total
+    unsigned long long* d_bl_base = nullptr;
+    double* d_bl_scale = nullptr;
+    void* d_bl_out = nullptr;                   // gathered lists on their way to the host
+    size_t bl_out_bytes = 0;
     cudaStream_t bl_capture = nullptr;
     cudaGraphExec_t bl_exec = nullptr;
     bool bl_graph_valid = false;

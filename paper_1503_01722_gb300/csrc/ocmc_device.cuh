@@ -451,7 +451,7 @@ __device__ __forceinline__ bool init_beamlet(const TransportArgs& a, unsigned lo
         if (a.bl_prefix[mid] <= g) lo = mid; else hi = mid - 1;
     }
     const BeamletDev& B = a.beamlets[lo];
-    p.batch = 0;
+    p.batch = lo;
     return init_source(a, B, B.bound, g - a.bl_prefix[lo], BL_TAG | (uint32_t)lo, p);
 }
 

@@ -198,7 +198,8 @@ struct TransportArgs {
     const BeamletDev* beamlets;
     const unsigned long long* bl_prefix; // n_beamlets + 1 prefix sums of histories
     int n_beamlets;
-    unsigned int* bl_keys;
+    bool bl_dense;                       // true: a dense tally per beamlet, beamlet b's at tally + b * nvox
+    unsigned int* bl_keys;               // else: hash tables
     unsigned long long* bl_vals;
     unsigned int* bl_overflow;           // per-beamlet table-full flags
 };
@@ -231,8 +232,17 @@ cudaError_t launch_test_csda(const TransportArgs& a, int m, const float* T, cons
                              cudaStream_t s);
 void material_defs(MatDef out[NMAT_DEFAULT]);
 cudaError_t launch_ps_validate(const PsRec* ps, unsigned long long n, unsigned long long* bad, cudaStream_t s);
-cudaError_t launch_bl_count(const unsigned int* keys, const unsigned long long* offs, const unsigned int* caps, int n,
-                            unsigned long long* nnz, cudaStream_t s);
+cudaError_t launch_bl_count(const unsigned int* keys, const unsigned long long* vals, const unsigned long long* offs,
+                            const unsigned int* caps, int n, unsigned long long* nnz, cudaStream_t s);
+// Dense beamlet tallies (n of nvox voxels each): non-zero voxels per chunk of BL_CHUNK voxels, turned into
+// offsets within the beamlet, and per beamlet; then every non-zero voxel in beamlet and voxel order, beamlet
+// b's first entry at base[b]. Any of idx, raw, dose may be null.
+constexpr int BL_CHUNK = 1024;
+cudaError_t launch_bl_dense_count(const unsigned long long* tally, int n, long long nvox, unsigned int* counts,
+                                  unsigned long long* nnz, cudaStream_t s);
+cudaError_t launch_bl_dense_gather(const unsigned long long* tally, int n, long long nvox, const unsigned int* offsets,
+                                   const unsigned long long* nnz, const unsigned long long* base, const double* scale,
+                                   const float* density, int* idx, long long* raw, float* dose, cudaStream_t s);
 cudaError_t launch_bl_extract(const unsigned int* keys, const unsigned long long* vals, unsigned long long cap,
                               long long nvox, long long* dense, unsigned int* block_counts, int* idx_out,
                               long long* raw_out, float* dose_out, const float* density, double scale,

@@ -61,11 +61,14 @@ struct BlockStats {
 };
 enum { BE_IN = 0, BE_ESC = 1 };
 
-// BL: batched-beamlet mode (sparse hash tallies) or single-beam mode (dense tally);
-// a compile-time flag so the single-beam kernel carries no beamlet code.
-template <bool BL>
+// Source and tally of a launch, compile-time so that each kernel carries only its own code: one beam
+// with a dense tally per statistical batch, beamlets with a dense tally each (a particle's batch is
+// then its beamlet), or beamlets with sparse hash tallies.
+enum { ONE_BEAM = 0, BEAMLETS_DENSE, BEAMLETS_HASH };
+
+template <int BL>
 struct CtxT {
-    static constexpr bool beamlets = BL;
+    static constexpr bool beamlets = BL != ONE_BEAM, hashed = BL == BEAMLETS_HASH;
     const TransportArgs& a;
     const SmemTables& T;
     PRec* stk;                   // warp's stacks: [0, cap) photons, [cap, 2cap) charged, [2cap, 3cap) slow charged
@@ -151,12 +154,13 @@ __device__ __forceinline__ void deposit_q(C& c, const Lane& p, int ix, int iy, i
         const int v = ix + c.a.nx * (iy + c.a.ny * iz);     // grids have at most 1024^3 voxels
         if constexpr (OCMC_CHECKS) {
             if (ix < 0 || iy < 0 || iz < 0 || ix >= c.a.nx || iy >= c.a.ny || iz >= c.a.nz ||
-                (!C::beamlets && (p.batch < 0 || p.batch >= c.a.pp.n_batches))) {
+                (!C::beamlets && (p.batch < 0 || p.batch >= c.a.pp.n_batches)) ||
+                (C::beamlets && !C::hashed && (p.batch < 0 || p.batch >= c.a.n_beamlets))) {
                 atomicOr(c.a.err, ERR_BOUNDS);
                 return;
             }
         }
-        if constexpr (C::beamlets) hash_add(c.a, p.r.h1 & ~BL_TAG, (uint32_t)v, q);
+        if constexpr (C::hashed) hash_add(c.a, p.r.h1 & ~BL_TAG, (uint32_t)v, q);
         else atomicAdd(c.a.tally + (long long)p.batch * c.a.nvox + v, q);
     }
 }
@@ -203,7 +207,7 @@ __device__ __forceinline__ void pop_lane(const C& c, int t, int slot, Lane& p)
     p.u = __uint_as_float(b.x); p.v = __uint_as_float(b.y); p.w = __uint_as_float(b.z);
     p.ix = b.w & 1023u; p.iy = (b.w >> 10) & 1023u; p.iz = (b.w >> 20) & 1023u; p.type = b.w >> 30;
     p.r.h0 = d.x; p.r.h1 = d.y; p.r.sub = d.z; p.r.n = d.w;
-    if constexpr (C::beamlets) p.batch = 0;
+    if constexpr (C::beamlets) p.batch = (int)(d.y & ~BL_TAG);
     else p.batch = batch_of(d.x, d.y ^ c.a.stream_tag, c.a.pp.n_batches);
     p.steps = 0;
 }
@@ -658,7 +662,7 @@ __device__ __noinline__ void flush_stats(const TransportArgs& a, BlockStats& st,
 // instantiation, so that the analytic-source kernel carries none of its code.
 // XV: electron steps cross voxel faces (the fixed-step variant); a separate instantiation of the
 // analytic-source kernel, so the voxel-limited kernels carry none of its code.
-template <bool BL, bool PS, int NREG, bool XV = false>
+template <int BL, bool PS, int NREG, bool XV = false>
 __global__ void __maxnreg__(NREG) k_transport(const __grid_constant__ TransportArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -682,7 +686,7 @@ __global__ void __maxnreg__(NREG) k_transport(const __grid_constant__ TransportA
     const int src_mode = a.src.particle == 0 ? 0 : 1;
     // a phase-space source mixes particle types: warps of either type draw from it, and a
     // primary of the other type goes to that type's stack like a secondary
-    constexpr bool ps_src = PS && !BL;
+    constexpr bool ps_src = PS && BL == ONE_BEAM;
     int mode = src_mode;
     bool src_done = a.count == 0;
     // with switch_high >= cap, switching on stack size is off (stacks may then overflow, which
@@ -732,7 +736,7 @@ __global__ void __maxnreg__(NREG) k_transport(const __grid_constant__ TransportA
                     if (!active && r2 >= 0 && r2 < want && base + r2 < a.count) {
                         count(c, ST_HISTORIES);
                         bool in;
-                        if constexpr (BL) in = init_beamlet(a, base + r2, p);
+                        if constexpr (BL != ONE_BEAM) in = init_beamlet(a, base + r2, p);
                         else if constexpr (ps_src) in = init_phase_space(a, a.first + base + r2, p);
                         else in = init_primary(a, a.first + base + r2, p);
                         if (!in) {
@@ -920,7 +924,7 @@ __global__ void __launch_bounds__(32 * CHAIN_LANES) k_chains(const __grid_consta
 size_t transport_smem_bytes(int n_mat) { return smem_table_bytes(n_mat); }
 
 namespace {
-template <bool BL, bool PS, int R, bool XV = false>
+template <int BL, bool PS, int R, bool XV = false>
 cudaError_t launch_variant(const TransportArgs& a, int blocks, int threads, size_t smem, cudaStream_t s)
 {
     cudaError_t e =
@@ -930,7 +934,7 @@ cudaError_t launch_variant(const TransportArgs& a, int blocks, int threads, size
     return cudaGetLastError();
 }
 
-template <bool BL, bool PS, int R>
+template <int BL, bool PS, int R>
 int occupancy(int threads, size_t smem)
 {
     cudaFuncSetAttribute(k_transport<BL, PS, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -940,7 +944,7 @@ int occupancy(int threads, size_t smem)
     return n;
 }
 
-template <bool BL, bool PS>
+template <int BL, bool PS>
 cudaError_t launch_source(const TransportArgs& a, int blocks, int threads, size_t smem, cudaStream_t s, int nreg)
 {
     if (nreg == 56) return launch_variant<BL, PS, 56>(a, blocks, threads, smem, s);
@@ -953,18 +957,21 @@ bool transport_nreg_supported(int nreg) { return nreg == 56 || nreg == 64 || nre
 
 int transport_max_blocks_per_sm(int threads, size_t smem, int nreg)
 {
-    occupancy<true, false, 56>(threads, smem);   // sets the shared-memory attribute of every variant
-    occupancy<true, false, 64>(threads, smem);
-    occupancy<true, false, 80>(threads, smem);
-    occupancy<false, true, 56>(threads, smem);
-    occupancy<false, true, 64>(threads, smem);
-    occupancy<false, true, 80>(threads, smem);
-    cudaFuncSetAttribute(k_transport<false, false, 56, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(k_transport<false, false, 64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(k_transport<false, false, 80, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (nreg == 56) return occupancy<false, false, 56>(threads, smem);
-    if (nreg == 64) return occupancy<false, false, 64>(threads, smem);
-    return occupancy<false, false, 80>(threads, smem);
+    occupancy<BEAMLETS_DENSE, false, 56>(threads, smem);
+    occupancy<BEAMLETS_HASH, false, 56>(threads, smem);   // sets the shared-memory attribute of every variant
+    occupancy<BEAMLETS_DENSE, false, 64>(threads, smem);
+    occupancy<BEAMLETS_HASH, false, 64>(threads, smem);
+    occupancy<BEAMLETS_DENSE, false, 80>(threads, smem);
+    occupancy<BEAMLETS_HASH, false, 80>(threads, smem);
+    occupancy<ONE_BEAM, true, 56>(threads, smem);
+    occupancy<ONE_BEAM, true, 64>(threads, smem);
+    occupancy<ONE_BEAM, true, 80>(threads, smem);
+    cudaFuncSetAttribute(k_transport<ONE_BEAM, false, 56, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(k_transport<ONE_BEAM, false, 64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(k_transport<ONE_BEAM, false, 80, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (nreg == 56) return occupancy<ONE_BEAM, false, 56>(threads, smem);
+    if (nreg == 64) return occupancy<ONE_BEAM, false, 64>(threads, smem);
+    return occupancy<ONE_BEAM, false, 80>(threads, smem);
 }
 
 static cudaError_t launch_one(const TransportArgs& a, int blocks, int threads, size_t smem, cudaStream_t s, int nreg)
@@ -972,13 +979,15 @@ static cudaError_t launch_one(const TransportArgs& a, int blocks, int threads, s
     if (a.pp.flags & FLAG_CROSS_VOXELS) {
         // voxel-crossing electron steps: analytic single-beam source only (callers check)
         if (a.beamlets || a.ps) return cudaErrorInvalidValue;
-        if (nreg == 56) return launch_variant<false, false, 56, true>(a, blocks, threads, smem, s);
-        if (nreg == 64) return launch_variant<false, false, 64, true>(a, blocks, threads, smem, s);
-        return launch_variant<false, false, 80, true>(a, blocks, threads, smem, s);
+        if (nreg == 56) return launch_variant<ONE_BEAM, false, 56, true>(a, blocks, threads, smem, s);
+        if (nreg == 64) return launch_variant<ONE_BEAM, false, 64, true>(a, blocks, threads, smem, s);
+        return launch_variant<ONE_BEAM, false, 80, true>(a, blocks, threads, smem, s);
     }
-    if (a.beamlets) return launch_source<true, false>(a, blocks, threads, smem, s, nreg);
-    if (a.ps) return launch_source<false, true>(a, blocks, threads, smem, s, nreg);
-    return launch_source<false, false>(a, blocks, threads, smem, s, nreg);
+    if (a.beamlets)
+        return a.bl_dense ? launch_source<BEAMLETS_DENSE, false>(a, blocks, threads, smem, s, nreg)
+                          : launch_source<BEAMLETS_HASH, false>(a, blocks, threads, smem, s, nreg);
+    if (a.ps) return launch_source<ONE_BEAM, true>(a, blocks, threads, smem, s, nreg);
+    return launch_source<ONE_BEAM, false>(a, blocks, threads, smem, s, nreg);
 }
 
 cudaError_t launch_transport(const TransportArgs& args, int blocks, int threads, size_t smem, cudaStream_t s, int nreg)

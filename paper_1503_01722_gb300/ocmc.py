@@ -19,6 +19,7 @@ _LIB_PATH = os.path.join(_HERE, "libocmc_checks.so" if os.environ.get("OCMC_CHEC
 OK, ERR_ARG, ERR_CUDA, ERR_OOM, ERR_OVERFLOW, ERR_TIMEOUT, ERR_STATE, ERR_BOUNDS = range(8)
 FLAG_NO_HARD, FLAG_NO_MS, FLAG_KILL_FIRST_REAL, FLAG_KERMA, FLAG_CROSS_VOXELS = 1, 2, 4, 8, 16
 TALLY_SCALE = 2.0 ** 28
+PINNED_LISTS = 2 << 30      # bytes of beamlet lists (Engine.beamlet_doses) up to which they are pinned
 
 
 class OcmcError(RuntimeError):
@@ -89,6 +90,8 @@ def _load():
         "ocmc_set_beamlets": (C.c_int, [P, C.c_int, C.c_int, P, P, C.c_int, P]),
         "ocmc_run_beamlets": (C.c_int, [P, C.c_uint64, P]),
         "ocmc_get_beamlet_dose": (C.c_int, [P, C.c_int, P, P, P, C.c_int64, C.POINTER(C.c_int64)]),
+        "ocmc_get_beamlet_sizes": (C.c_int, [P, P]),
+        "ocmc_get_beamlet_entries": (C.c_int, [P, P, P, P, C.c_int64]),
         "ocmc_autotune": (C.c_int, [P, C.c_uint64, C.POINTER(Params)]),
         "ocmc_set_phase_space": (C.c_int, [P, P, C.c_uint64, C.c_int]),
         "ocmc_set_materials": (C.c_int, [P, C.c_int, P]),
@@ -336,25 +339,26 @@ class Engine:
 
     def beamlet_doses(self, raw=False):
         """Every beamlet's sparse dose, [(voxel indices int32, dose float32 MeV/g per history
-        [, raw int64])] in beamlet order: one extraction per beamlet into reusable pinned host
-        buffers of one phantom's size (no size query, no pageable copies)."""
+        [, raw int64])] in beamlet order: views of one block of host memory that all lists share."""
         import torch
         if self.shape is None:
             raise OcmcError(ERR_STATE, "no phantom")
-        nvox = int(np.prod(self.shape))
-        if getattr(self, "_bl_buf", None) is None or self._bl_buf[0].numel() < nvox:
-            self._bl_buf = (torch.empty(nvox, dtype=torch.int32).pin_memory(),
-                            torch.empty(nvox, dtype=torch.float32).pin_memory(),
-                            torch.empty(nvox, dtype=torch.int64).pin_memory())
-        bi, bd, br = self._bl_buf
-        nnz = C.c_int64()
+        ptr = np.empty(self.n_beamlets + 1, np.int64)
+        self._check(lib.ocmc_get_beamlet_sizes(self._c, C.c_void_p(ptr.ctypes.data)))
+        n = int(ptr[-1])
+        size = n * (16 if raw else 8)
+        # pinned, so that the copy runs at the link's rate and into memory that is already mapped (torch
+        # keeps and reuses the block once the lists are gone); pageable beyond PINNED_LISTS
+        mem = (torch.empty(max(size, 1), dtype=torch.uint8, pin_memory=True).numpy() if size <= PINNED_LISTS
+               else np.empty(size, np.uint8))
+        r = mem[:8 * n].view(np.int64) if raw else None
+        o = 8 * n if raw else 0
+        idx, dose = mem[o:o + 4 * n].view(np.int32), mem[o + 4 * n:o + 8 * n].view(np.float32)
+        self._check(lib.ocmc_get_beamlet_entries(self._c, C.c_void_p(idx.ctypes.data), C.c_void_p(dose.ctypes.data),
+                                                 C.c_void_p(r.ctypes.data) if raw else None, n))
         out = []
-        for b in range(self.n_beamlets):
-            self._check(lib.ocmc_get_beamlet_dose(self._c, b, C.c_void_p(bi.data_ptr()), C.c_void_p(bd.data_ptr()),
-                                                  C.c_void_p(br.data_ptr()) if raw else None, nvox, C.byref(nnz)))
-            n = nnz.value
-            item = (bi[:n].numpy().copy(), bd[:n].numpy().copy())
-            out.append(item + (br[:n].numpy().copy(),) if raw else item)
+        for a, b in zip(ptr[:-1].tolist(), ptr[1:].tolist()):
+            out.append((idx[a:b], dose[a:b], r[a:b]) if raw else (idx[a:b], dose[a:b]))
         return out
 
     def autotune(self, pilot_histories):
