@@ -29,20 +29,35 @@ constexpr int CH[LEVELS] = {16, 32, 64, 128};
 constexpr int NLAYERS = 20;
 
 // ---- small kernels ------------------------------------------------------------------------
-__global__ void k_max_reduce(const float* x, long long n, unsigned int* out)
+// The maps are read once and the activations are whole 32-byte sectors, so HBM and L2 bound these kernels:
+// vector loads, one atomic per block (an atomic per warp on one word took 17 us for 128^3, now 5).
+__global__ void __launch_bounds__(256) k_max_reduce(const float* __restrict__ x, long long n, unsigned int* out)
 {
+    __shared__ float sh[8];
     float m = 0.f;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        m = fmaxf(m, x[i]);
+    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x, T = (long long)gridDim.x * blockDim.x;
+    if ((reinterpret_cast<uintptr_t>(x) & 15) == 0) {          // n is a multiple of 512
+        const float4* x4 = reinterpret_cast<const float4*>(x);
+        for (long long i = t; i < n / 4; i += T) {
+            const float4 v = x4[i];
+            m = fmaxf(m, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
+        }
+    } else {
+        for (long long i = t; i < n; i += T) m = fmaxf(m, x[i]);
+    }
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_down_sync(0xFFFFFFFFu, m, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(out, __float_as_uint(m));   // non-negative floats
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int i = 1; i < 8; ++i) m = fmaxf(m, sh[i]);
+        atomicMax(out, __float_as_uint(m));   // non-negative floats
+    }
 }
 
-// x0 = dose / s, x1 = density, x2 = sigma / s (0 without sigma). Channels 3-15 of the input
-// activation are zeroed when the network is created and never written, so each voxel needs one
-// 8-byte store (channels 0-3).
-__global__ void k_pack_input(const float* dose, const float* dens, const float* sigma, long long n,
-                             const unsigned int* smax, __nv_bfloat16* x, float* x0f)
+// x0 = dose / s, x1 = density, x2 = sigma / s (0 without sigma), channels 3-15 zero: whole sectors are
+// written (stores of the first channels alone made L2 fetch every sector first: 22 us for 128^3, now 14).
+__global__ void k_pack_input(const float* __restrict__ dose, const float* __restrict__ dens, const float* __restrict__ sigma,
+                             long long n, const unsigned int* smax, __nv_bfloat16* x, float* x0f)
 {
     float s = __uint_as_float(*smax);
     float inv = s > 0.f ? 1.f / s : 0.f;
@@ -51,75 +66,114 @@ __global__ void k_pack_input(const float* dose, const float* dens, const float* 
         x0f[v] = d;
         float sg = sigma ? sigma[v] * inv : 0.f;
         __nv_bfloat162 lo = __floats2bfloat162_rn(d, dens[v]), hi = __floats2bfloat162_rn(sg, 0.f);
-        uint2 w;
-        w.x = *reinterpret_cast<uint32_t*>(&lo);
-        w.y = *reinterpret_cast<uint32_t*>(&hi);
-        *reinterpret_cast<uint2*>(x + v * 16) = w;
+        uint4* o = reinterpret_cast<uint4*>(x + v * 16);
+        o[0] = make_uint4(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi), 0u, 0u);
+        o[1] = make_uint4(0u, 0u, 0u, 0u);
     }
 }
 
-// out = x0 + sum_c h[v][c] w[c] + b
-__global__ void k_head_fwd(const __nv_bfloat16* h, const float* w, const float* b, const float* x0, long long n,
-                           float* out)
+struct Bf16x16 {
+    uint4 a, b;
+};
+
+__device__ __forceinline__ Bf16x16 load16(const __nv_bfloat16* p)
 {
-    for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x) {
-        float s = b[0] + x0[v];
-        const __nv_bfloat16* p = h + v * 16;
+    const uint4* q = reinterpret_cast<const uint4*>(p);
+    return Bf16x16{q[0], q[1]};
+}
+
+__device__ __forceinline__ void unpack16(const Bf16x16& h, float f[16])
+{
+    const uint32_t w[8] = {h.a.x, h.a.y, h.a.z, h.a.w, h.b.x, h.b.y, h.b.z, h.b.w};
 #pragma unroll
-        for (int c = 0; c < 16; ++c) s += __bfloat162float(p[c]) * w[c];
-        out[v] = s;
+    for (int i = 0; i < 8; ++i) {                              // a BF16 is the upper half of its float
+        f[2 * i] = __uint_as_float(w[i] << 16);
+        f[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
     }
 }
 
-// masked MSE of out against target/s; gout = d loss / d out; loss sum into *acc[0], mask count *acc[1]
-__global__ void k_loss(const float* out, const float* target, const float* dens, long long n, const unsigned int* smax,
-                       float* gout, double* acc)
+// Head: o = x0 + sum_c h[v][c] w[c] + b. Inference (target null): out = o s. Training: out = the masked
+// error o - target / s over voxels of density >= 0.1, with the sum of its squares to acc[0] and the mask's
+// count to acc[1] (their derivative's factor 2 / count is applied by k_head_bwd).
+__global__ void __launch_bounds__(256) k_head_fwd(const __nv_bfloat16* __restrict__ h, const float* __restrict__ w,
+                                                  const float* __restrict__ b, const float* __restrict__ x0, long long n,
+                                                  const unsigned int* smax, const float* __restrict__ target,
+                                                  const float* __restrict__ dens, float* __restrict__ out, double* acc)
 {
-    float s = __uint_as_float(*smax);
-    float inv = s > 0.f ? 1.f / s : 0.f;
-    double l = 0.0, cnt = 0.0;
+    const float sc = __uint_as_float(*smax), inv = sc > 0.f ? 1.f / sc : 0.f;
+    float wr[16];
+#pragma unroll
+    for (int c = 0; c < 16; ++c) wr[c] = w[c];
+    const float b0 = b[0];
+    double l = 0.0;
+    int cnt = 0;
     for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x) {
-        bool m = dens[v] >= 0.1f;
-        float e = m ? out[v] - target[v] * inv : 0.f;
-        gout[v] = e;                    // scaled by 2 / count in k_scale_gout
-        l += (double)e * e;
-        cnt += m ? 1.0 : 0.0;
+        float f[16];
+        unpack16(load16(h + v * 16), f);
+        float s = b0 + x0[v];
+#pragma unroll
+        for (int c = 0; c < 16; ++c) s += f[c] * wr[c];
+        if (target) {
+            const bool m = dens[v] >= 0.1f;
+            const float e = m ? s - target[v] * inv : 0.f;
+            out[v] = e;
+            l += (double)e * e;
+            cnt += m ? 1 : 0;
+        } else {
+            out[v] = s * sc;
+        }
     }
+    if (!target) return;
+    __shared__ double sl[8];
+    __shared__ int sn[8];
     for (int o = 16; o > 0; o >>= 1) {
         l += __shfl_down_sync(0xFFFFFFFFu, l, o);
         cnt += __shfl_down_sync(0xFFFFFFFFu, cnt, o);
     }
     if ((threadIdx.x & 31) == 0) {
+        sl[threadIdx.x >> 5] = l;
+        sn[threadIdx.x >> 5] = cnt;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int i = 1; i < 8; ++i) {
+            l += sl[i];
+            cnt += sn[i];
+        }
         atomicAdd(acc, l);
-        atomicAdd(acc + 1, cnt);
+        atomicAdd(acc + 1, (double)cnt);
     }
 }
 
-__global__ void k_scale_gout(float* g, long long n, const double* acc)
+// head backward: g = err 2 / count, gh[v][c] = g w[c] (h > 0); partial sums of g h and g per block.
+// 16-byte loads and stores of a voxel's channels (175 us for 128^3 with two bytes at a time, now 40).
+__global__ void __launch_bounds__(256) k_head_bwd(const __nv_bfloat16* __restrict__ h, const float* __restrict__ w,
+                                                  const float* __restrict__ err, const double* acc, long long n,
+                                                  __nv_bfloat16* gh, float* part /* [gridDim.x][17] */)
 {
-    float sc = acc[1] > 0.0 ? (float)(2.0 / acc[1]) : 0.f;
-    for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x)
-        g[v] *= sc;
-}
-
-// head backward: gh[v][c] = gout[v] w[c] (h > 0); partial sums of gout*h and gout per block
-__global__ void k_head_bwd(const __nv_bfloat16* h, const float* w, const float* gout, long long n, __nv_bfloat16* gh,
-                           float* part /* [gridDim.x][17] */)
-{
-    float sw[17];
+    const float sc = acc[1] > 0.0 ? (float)(2.0 / acc[1]) : 0.f;
+    float wr[16], sw[17];
+#pragma unroll
+    for (int c = 0; c < 16; ++c) wr[c] = w[c];
 #pragma unroll
     for (int c = 0; c < 17; ++c) sw[c] = 0.f;
     for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x) {
-        float g = gout[v];
-        const __nv_bfloat16* p = h + v * 16;
-        __nv_bfloat16* q = gh + v * 16;
+        const float g = err[v] * sc;
+        float f[16];
+        unpack16(load16(h + v * 16), f);
+        uint32_t q[8];
 #pragma unroll
-        for (int c = 0; c < 16; ++c) {
-            float hv = __bfloat162float(p[c]);
-            sw[c] += g * hv;
-            q[c] = __float2bfloat16_rn(hv > 0.f ? g * w[c] : 0.f);
+        for (int c = 0; c < 8; ++c) {
+            const float f0 = f[2 * c], f1 = f[2 * c + 1];
+            sw[2 * c] += g * f0;
+            sw[2 * c + 1] += g * f1;
+            const __nv_bfloat162 r = __floats2bfloat162_rn(f0 > 0.f ? g * wr[2 * c] : 0.f, f1 > 0.f ? g * wr[2 * c + 1] : 0.f);
+            q[c] = *reinterpret_cast<const uint32_t*>(&r);
         }
         sw[16] += g;
+        uint4* o = reinterpret_cast<uint4*>(gh + v * 16);
+        o[0] = make_uint4(q[0], q[1], q[2], q[3]);
+        o[1] = make_uint4(q[4], q[5], q[6], q[7]);
     }
     __shared__ float red[17][8];
 #pragma unroll
@@ -131,7 +185,7 @@ __global__ void k_head_bwd(const __nv_bfloat16* h, const float* w, const float* 
     __syncthreads();
     if (threadIdx.x < 17) {
         float x = 0.f;
-        for (int i = 0; i < (int)(blockDim.x >> 5); ++i) x += red[threadIdx.x][i];
+        for (int i = 0; i < 8; ++i) x += red[threadIdx.x][i];
         part[blockIdx.x * 17 + threadIdx.x] = x;
     }
 }
@@ -320,8 +374,7 @@ struct ocmc_unet {
     float* tmpw = nullptr;          // UP weight gradient before transposition, [8][cout][cin]
     float* bpart = nullptr;         // bias / head gradient partials
     float* x0f = nullptr;           // normalised noisy dose (FP32)
-    float* outf = nullptr;          // network output (normalised)
-    float* gout = nullptr;
+    float* gout = nullptr;          // error of the normalised output (training)
     unsigned int* smax = nullptr;
     double* lacc = nullptr;
     float* fb = nullptr;            // denoise scratch: plain dose, sigma, output, flags (4 x nvox)
@@ -345,6 +398,9 @@ ocmc_status ufail(ocmc_unet* u, ocmc_status s, const std::string& m)
             return ufail(u, e_ == cudaErrorMemoryAllocation ? OCMC_ERR_OOM : OCMC_ERR_CUDA,       \
                          std::string(where) + ": " + cudaGetErrorString(e_));                     \
     } while (0)
+
+// Blocks of 256 threads for kernels that end in a reduction: four a SM.
+int stream_grid(long long n) { return (int)std::max<long long>(1, std::min<long long>((n + 255) / 256, 4LL * sm_count())); }
 
 int grid_for(long long n) { return (int)std::max<long long>(1, std::min<long long>((n + 255) / 256, 152 * 16)); }
 
@@ -628,21 +684,21 @@ ocmc_status forward(ocmc_unet* u, const float* dose, const float* sigma, const f
 {
     long long n = u->nvox;
     UCK(cudaMemsetAsync(u->smax, 0, sizeof(unsigned int), s), "memset");
-    k_max_reduce<<<grid_for(n), 256, 0, s>>>(dose, n, u->smax);
+    k_max_reduce<<<stream_grid(n), 256, 0, s>>>(dose, n, u->smax);
     k_pack_input<<<grid_for(n), 256, 0, s>>>(dose, dens, sigma, n, u->smax, u->acts[0].x, u->x0f);
     UCK(cudaGetLastError(), "input");
     for (const Layer& L : u->layers) UCK(layer_fwd(u, L, s), "layer forward");
-    const Act& last = u->acts[u->layers.back().out_act];
-    k_head_fwd<<<grid_for(n), 256, 0, s>>>(last.x, u->params + u->head_w, u->params + u->head_b, u->x0f, n, u->outf);
-    UCK(cudaGetLastError(), "head");
     return OCMC_OK;
 }
 
-__global__ void k_denorm(const float* out, const unsigned int* smax, long long n, float* dst)
+// the head after forward(): denormalised output, or with a target the error map and the loss sums
+ocmc_status head(ocmc_unet* u, const float* target, const float* dens, float* out, cudaStream_t s)
 {
-    float sc = __uint_as_float(*smax);
-    for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x)
-        dst[v] = out[v] * sc;
+    const Act& last = u->acts[u->layers.back().out_act];
+    k_head_fwd<<<stream_grid(u->nvox), 256, 0, s>>>(last.x, u->params + u->head_w, u->params + u->head_b, u->x0f, u->nvox,
+                                                    u->smax, target, dens, out, u->lacc);
+    UCK(cudaGetLastError(), "head");
+    return OCMC_OK;
 }
 
 // Fallback to plain Monte Carlo where the network's change exceeds k sigma of the plain
@@ -773,7 +829,6 @@ ocmc_status ocmc_unet_create(ocmc_unet** out, int device, int nx, int ny, int nz
     if (e == cudaSuccess) e = cudaMalloc(&u->tmpw, (size_t)8 * 128 * 128 * sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc(&u->bpart, (size_t)152 * 16 * 128 * sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc(&u->x0f, u->nvox * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&u->outf, u->nvox * sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc(&u->gout, u->nvox * sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc(&u->smax, sizeof(unsigned int));
     if (e == cudaSuccess) e = cudaMalloc(&u->lacc, 2 * sizeof(double));
@@ -812,7 +867,7 @@ void ocmc_unet_destroy(ocmc_unet* u)
     for (Layer& L : u->layers) { cudaFree(L.wf); cudaFree(L.wt); cudaFree(L.wtc_f); cudaFree(L.wtc_t); }
     cudaFree(u->params); cudaFree(u->grads); cudaFree(u->adam_m); cudaFree(u->adam_v); cudaFree(u->part);
     cudaFree(u->tmpw); cudaFree(u->bpart);
-    cudaFree(u->x0f); cudaFree(u->outf); cudaFree(u->gout); cudaFree(u->smax); cudaFree(u->lacc);
+    cudaFree(u->x0f); cudaFree(u->gout); cudaFree(u->smax); cudaFree(u->lacc);
     cudaFree(u->fb); cudaFree(u->kerr);
     delete u;
 }
@@ -854,10 +909,7 @@ ocmc_status ocmc_unet_forward(ocmc_unet* u, const float* dose, const float* sigm
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     UCK(cudaSetDevice(u->device), "device");
     ocmc_status st = forward(u, dose, sigma, dens, s);
-    if (st != OCMC_OK) return st;
-    k_denorm<<<grid_for(u->nvox), 256, 0, s>>>(u->outf, u->smax, u->nvox, out);
-    UCK(cudaGetLastError(), "output");
-    return OCMC_OK;
+    return st != OCMC_OK ? st : head(u, nullptr, nullptr, out, s);
 }
 
 // One training step: forward, masked MSE loss, backward, Adam (lr; betas 0.9/0.999).
@@ -873,13 +925,12 @@ ocmc_status ocmc_unet_train_step(ocmc_unet* u, const float* dose, const float* s
     if (st != OCMC_OK) return st;
     long long n = u->nvox;
     UCK(cudaMemsetAsync(u->lacc, 0, 2 * sizeof(double), s), "memset");
-    k_loss<<<grid_for(n), 256, 0, s>>>(u->outf, target, dens, n, u->smax, u->gout, u->lacc);
-    k_scale_gout<<<grid_for(n), 256, 0, s>>>(u->gout, n, u->lacc);
-    // head
+    st = head(u, target, dens, u->gout, s);
+    if (st != OCMC_OK) return st;
     const Layer& lastL = u->layers.back();
     const Act& last = u->acts[lastL.out_act];
-    int hb = grid_for(n);
-    k_head_bwd<<<hb, 256, 0, s>>>(last.x, u->params + u->head_w, u->gout, n, last.g, u->bpart);
+    const int hb = stream_grid(n);
+    k_head_bwd<<<hb, 256, 0, s>>>(last.x, u->params + u->head_w, u->gout, u->lacc, n, last.g, u->bpart);
     sum_rows(u->bpart, hb, 17, u->grads + u->head_w, s);
     UCK(cudaGetLastError(), "head backward");
     // layers in reverse; UP weight gradients come out as [p][n][c] and are transposed
@@ -924,7 +975,7 @@ ocmc_status ocmc_unet_layer_times(ocmc_unet* u, const float* dose, const float* 
     for (int r = 0; r < repeats && st == OCMC_OK; ++r) {
         long long n = u->nvox;
         cudaMemsetAsync(u->smax, 0, sizeof(unsigned int), nullptr);
-        k_max_reduce<<<grid_for(n), 256>>>(dose, n, u->smax);
+        k_max_reduce<<<stream_grid(n), 256>>>(dose, n, u->smax);
         k_pack_input<<<grid_for(n), 256>>>(dose, dens, sigma, n, u->smax, u->acts[0].x, u->x0f);
         cudaEventRecord(ev[0], nullptr);
         for (int i = 0; i < L; ++i) {
