@@ -213,40 +213,84 @@ __global__ void __launch_bounds__(1024) k_sum_rows(const float* part, int parts,
     }
 }
 
-// The same sums for wide rows, four columns per thread (the block-per-32-columns form above would
-// launch m / 32 blocks of mostly idle threads): identical order of additions (parts in 32
-// consecutive groups, each group summed from zero, the group sums added in order from zero).
-__global__ void k_sum_rows4(const float4* part, int parts, long long m4, float4* out)
+// The same sums for rows of a multiple of four columns: 32 groups of consecutive parts by 8 threads of four
+// columns, so that every load is a 128-byte segment and a block's reads are independent; identical order of
+// additions. Bound by reading the partials (33.6 MB of a 64 -> 64 layer: 28 us in the form above).
+// dst(j): where column j goes (the UP layers' gradients come out transposed).
+__global__ void __launch_bounds__(256) k_sum_rows4(const float4* __restrict__ part, int parts, long long m4,
+                                                   float* __restrict__ out, int tn, int tc)
 {
+    __shared__ float4 sh[32][9];
+    const int x = threadIdx.x & 7, y = threadIdx.x >> 3;
+    const long long j = blockIdx.x * 8ll + x;
     const int L = (parts + 31) / 32;
-    for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < m4; j += (long long)gridDim.x * blockDim.x) {
-        float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int y = 0; y < 32; ++y) {
-            const int i0 = y * L, i1 = min(parts, i0 + L);
-            float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-            for (int i = i0; i < i1; ++i) {
-                const float4 v = part[(long long)i * m4 + j];
-                s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
-            }
-            t.x += s.x; t.y += s.y; t.z += s.z; t.w += s.w;
+    const int i0 = min(parts, y * L), i1 = min(parts, i0 + L);
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (j < m4) {
+#pragma unroll 8
+        for (int i = i0; i < i1; ++i) {
+            const float4 v = __ldcs(part + (long long)i * m4 + j);
+            s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
         }
-        out[j] = t;
+    }
+    sh[y][x] = s;
+    __syncthreads();
+    // 32 column sums, one thread each
+    if (threadIdx.x < 32) {
+        const int c4 = threadIdx.x >> 2, e = threadIdx.x & 3;
+        const long long col = (blockIdx.x * 8ll + c4) * 4 + e;
+        if (col < 4 * m4) {
+            float t = 0.f;
+#pragma unroll
+            for (int k = 0; k < 32; ++k) t += reinterpret_cast<const float*>(&sh[k][c4])[e];
+            long long o = col;
+            if (tc) {                      // column (tap, n, c) of [taps][tn][tc] goes to (tap, c, n)
+                const int c = (int)(col % tc), n = (int)(col / tc % tn);
+                o = (col / ((long long)tn * tc) * tc + c) * tn + n;
+            }
+            out[o] = t;
+        }
     }
 }
 
 int sm_count();
 
-void sum_rows(const float* part, int parts, long long m, float* out, cudaStream_t s)
+void sum_rows(const float* part, int parts, long long m, float* out, cudaStream_t s, int tn = 0, int tc = 0)
 {
-    // wide rows with few parts, or rows wide enough for a thread per four columns to keep the GPU
-    // busy; otherwise (narrow rows of many parts) the block form
-    if (m % 4 == 0 && m >= 8192 && (parts <= 32 || m >= 131072)) {
-        const long long m4 = m / 4;
-        k_sum_rows4<<<(unsigned)std::min<long long>((m4 + 255) / 256, 8LL * sm_count()), 256, 0, s>>>(
-            reinterpret_cast<const float4*>(part), parts, m4, reinterpret_cast<float4*>(out));
+    if (m % 4 == 0) {
+        k_sum_rows4<<<(unsigned)((m / 4 + 7) / 8), 256, 0, s>>>(reinterpret_cast<const float4*>(part), parts, m / 4, out, tn, tc);
         return;
     }
     k_sum_rows<<<(unsigned)((m + 31) / 32), dim3(32, 32), 0, s>>>(part, parts, (int)m, out);
+}
+
+// Bias gradients of all layers (and the head's sums) from their partials in one launch: blockIdx.y is the
+// layer, its columns by blockIdx.x, summed as in k_sum_rows.
+constexpr int NBIAS = NLAYERS + 1;
+struct BiasSums {
+    int parts[NBIAS], m[NBIAS];
+    long long src[NBIAS], dst[NBIAS];      // offsets of the partials and of the sums
+};
+
+__global__ void __launch_bounds__(1024) k_sum_biases(const float* __restrict__ part, const BiasSums b, float* __restrict__ out)
+{
+    __shared__ float sh[32][33];
+    const int l = blockIdx.y, m = b.m[l], parts = b.parts[l], j = blockIdx.x * 32 + threadIdx.x;
+    if ((int)blockIdx.x * 32 >= m) return;
+    const int L = (parts + 31) / 32;
+    const int i0 = threadIdx.y * L, i1 = min(parts, i0 + L);
+    float s = 0.f;
+    if (j < m) {
+#pragma unroll 8
+        for (int i = i0; i < i1; ++i) s += part[b.src[l] + (long long)i * m + j];
+    }
+    sh[threadIdx.y][threadIdx.x] = s;
+    __syncthreads();
+    if (threadIdx.y == 0 && j < m) {
+        float t = 0.f;
+        for (int y = 0; y < 32; ++y) t += sh[y][threadIdx.x];
+        out[b.dst[l] + j] = t;
+    }
 }
 
 // bias gradient partials: per block sums of dy[v][n] over its voxels, in a fixed order (thread
@@ -262,17 +306,26 @@ __global__ void k_bias_part(const __nv_bfloat16* dy, int stride, int c0, int cou
     float acc[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) acc[e] = 0.f;
-    if (r < rpp)
-        for (long long v = (long long)blockIdx.x * rpp + r; v < n; v += (long long)gridDim.x * rpp) {
-            const uint4 q = *reinterpret_cast<const uint4*>(dy + v * stride + c0 + 8 * g);
-            const __nv_bfloat162* b = reinterpret_cast<const __nv_bfloat162*>(&q);
+    if (r < rpp) {
+        const long long step = (long long)gridDim.x * rpp;
+        for (long long v = (long long)blockIdx.x * rpp + r; v < n; v += 8 * step) {
+            uint4 q[8];                        // eight loads in flight, added in order
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const float2 f = __bfloat1622float2(b[e]);
-                acc[2 * e] += f.x;
-                acc[2 * e + 1] += f.y;
+            for (int k = 0; k < 8; ++k)
+                q[k] = v + k * step < n ? *reinterpret_cast<const uint4*>(dy + (v + k * step) * stride + c0 + 8 * g)
+                                        : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const __nv_bfloat162* b = reinterpret_cast<const __nv_bfloat162*>(&q[k]);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float2 f = __bfloat1622float2(b[e]);
+                    acc[2 * e] += f.x;
+                    acc[2 * e + 1] += f.y;
+                }
             }
         }
+    }
 #pragma unroll
     for (int e = 0; e < 8; ++e) sh[threadIdx.x * 8 + e] = acc[e];
     __syncthreads();
@@ -371,8 +424,9 @@ struct ocmc_unet {
     long long step = 0;
     float* part = nullptr;          // weight-gradient partials
     size_t part_n = 0;
-    float* tmpw = nullptr;          // UP weight gradient before transposition, [8][cout][cin]
-    float* bpart = nullptr;         // bias / head gradient partials
+    float* bpart = nullptr;         // bias / head gradient partials of a backward pass, summed at its end
+    long long bpart_used = 0;
+    BiasSums bias;
     float* x0f = nullptr;           // normalised noisy dose (FP32)
     float* gout = nullptr;          // error of the normalised output (training)
     unsigned int* smax = nullptr;
@@ -484,18 +538,6 @@ cudaError_t launch_conv(const ConvArgs& a, cudaStream_t s)
     return a.cin % 32 == 0 ? launch_conv_bk<32>(a, s) : launch_conv_bk<16>(a, s);
 }
 
-__global__ void k_transpose_pnc(const float* src, int taps, int n, int c, float* dst)
-{
-    long long total = (long long)taps * n * c;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-        int ci = (int)(i % c);
-        long long q = i / c;
-        int ni = (int)(q % n);
-        int t = (int)(q / n);
-        dst[((long long)t * c + ci) * n + ni] = src[i];
-    }
-}
-
 // Weight gradient of a 3x3x3 convolution over grid g (input and output) into dW [27][cin][cout]:
 // on tcgen05 where that kernel covers the channel counts (tc), else on mma.sync.
 cudaError_t launch_wgrad3(Grid3 g, Slice x, Slice dy, int cin, int cout, float* part, size_t part_cap, float* dW,
@@ -541,7 +583,7 @@ cudaError_t launch_wgrad3(Grid3 g, Slice x, Slice dy, int cin, int cout, float* 
 
 // Weight gradient of one layer into dW (FP32, [taps][cin][cout]).
 cudaError_t launch_wgrad(Mode mode, Grid3 gin, Grid3 gout, Slice x, Slice dy, int cin, int cout, float* part,
-                         size_t part_cap, float* dW, bool tc, int* err, cudaStream_t s)
+                         size_t part_cap, float* dW, bool tc, int* err, cudaStream_t s, bool transpose = false)
 {
     // UP layers are handled as DOWN over (dy, x) with the roles of the grids swapped:
     // dW[p][c][n] = sum_u x[u][c] dy[2u+p][n]  ==  sum_u (DOWN gather of dy)[u][n] x[u][c]
@@ -558,7 +600,9 @@ cudaError_t launch_wgrad(Mode mode, Grid3 gin, Grid3 gout, Slice x, Slice dy, in
     long long rows = gout.n();
     int bc = std::min(cin, 64), bn = std::min(cout, 64);
     int tiles = (cin / bc) * (cout / bn);
-    long long chunks = std::max<long long>(1, std::min<long long>(64, (rows + 2047) / 2048));
+    // eight blocks per SM over (chunks, taps, tiles), chunks of at least 128 rows (2048-row chunks left the
+    // 64-channel layers on 32 and 128 blocks: 60 and 57 us at 128^3, 16 -> 32 99 us)
+    long long chunks = std::max<long long>(1, std::min<long long>(sm_count() / tiles, (rows + 127) / 128));
     while (chunks > 1 && (size_t)chunks * taps * cin * cout > part_cap) chunks /= 2;
     if ((size_t)chunks * taps * cin * cout > part_cap) return cudaErrorMemoryAllocation;
     a.rows_per_chunk = (rows + chunks - 1) / chunks;
@@ -572,7 +616,7 @@ cudaError_t launch_wgrad(Mode mode, Grid3 gin, Grid3 gout, Slice x, Slice dy, in
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     long long m = (long long)taps * cin * cout;
-    sum_rows(part, (int)chunks, m, dW, s);
+    sum_rows(part, (int)chunks, m, dW, s, transpose ? cin : 0, transpose ? cout : 0);
     return cudaGetLastError();
 }
 
@@ -602,6 +646,16 @@ cudaError_t layer_fwd(ocmc_unet* u, const Layer& L, cudaStream_t s)
     return launch_conv(a, s);
 }
 
+// place of layer k's bias partials (k = NLAYERS: the head's sums): after those of the layers before it in the pass
+void add_bias_sum(ocmc_unet* u, int k, int parts, int m, size_t dst)
+{
+    u->bias.parts[k] = parts;
+    u->bias.m[k] = m;
+    u->bias.src[k] = u->bpart_used;
+    u->bias.dst[k] = (long long)dst;
+    u->bpart_used += (long long)parts * m;
+}
+
 // backward of layer L: weight and bias gradients, then the data gradient into the
 // gradient slice of its input (masked by that input's ReLU, accumulated for skips)
 cudaError_t layer_bwd(ocmc_unet* u, const Layer& L, bool need_dx, cudaStream_t s)
@@ -611,12 +665,10 @@ cudaError_t layer_bwd(ocmc_unet* u, const Layer& L, bool need_dx, cudaStream_t s
     cudaError_t e;
     if (L.mode == UP) {
         // dW[p][c][n] = sum_u x[u][c] dy[2u+p][n]: a DOWN-gather weight gradient over the coarse
-        // grid with operands (dy as gathered input, x as rows), computed into [p][n][c], then transposed
-        e = launch_wgrad(DOWN, u->g[L.lout], u->g[L.lin], dy, x, L.cout, L.cin, u->part, u->part_n, u->tmpw, u->tc,
-                         u->kerr, s);
+        // grid with operands (dy as gathered input, x as rows), computed as [p][n][c] and transposed by the sum
+        e = launch_wgrad(DOWN, u->g[L.lout], u->g[L.lin], dy, x, L.cout, L.cin, u->part, u->part_n, u->grads + L.woff, u->tc,
+                         u->kerr, s, true);
         if (e != cudaSuccess) return e;
-        long long m = 8LL * L.cin * L.cout;          // [p][n][c] -> grads [p][c][n]
-        k_transpose_pnc<<<grid_for(m), 256, 0, s>>>(u->tmpw, 8, L.cout, L.cin, u->grads + L.woff);
     } else {
         e = launch_wgrad(L.mode, u->g[L.lin], u->g[L.lout], x, dy, L.cin, L.cout, u->part, u->part_n,
                          u->grads + L.woff, u->tc, u->kerr, s);
@@ -624,9 +676,10 @@ cudaError_t layer_bwd(ocmc_unet* u, const Layer& L, bool need_dx, cudaStream_t s
     }
     long long nout = u->g[L.lout].n();
     // four blocks per SM stream dy once; few partials keep their fixed-order sum short
-    int blocks = (int)std::min<long long>(grid_for(nout * L.cout), 4LL * sm_count());
-    k_bias_part<<<blocks, 256, 0, s>>>(dy.ptr, dy.stride, dy.c0, L.cout, nout, u->bpart);
-    sum_rows(u->bpart, blocks, L.cout, u->grads + L.boff, s);
+    const int blocks = (int)std::min<long long>(grid_for(nout * L.cout), 4LL * sm_count());
+    const int k = (int)(&L - u->layers.data());
+    add_bias_sum(u, k, blocks, L.cout, L.boff);
+    k_bias_part<<<blocks, 256, 0, s>>>(dy.ptr, dy.stride, dy.c0, L.cout, nout, u->bpart + u->bias.src[k]);
     e = cudaGetLastError();
     if (e != cudaSuccess || !need_dx) return e;
     ConvArgs a;
@@ -826,8 +879,9 @@ ocmc_status ocmc_unet_create(ocmc_unet** out, int device, int nx, int ny, int nz
     if (e == cudaSuccess) e = cudaMalloc(&u->adam_v, pbytes);
     u->part_n = (size_t)8 << 20;
     if (e == cudaSuccess) e = cudaMalloc(&u->part, u->part_n * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&u->tmpw, (size_t)8 * 128 * 128 * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&u->bpart, (size_t)152 * 16 * 128 * sizeof(float));
+    size_t bias_n = 17;
+    for (const Layer& L : u->layers) bias_n += L.cout;
+    if (e == cudaSuccess) e = cudaMalloc(&u->bpart, bias_n * 4 * sm_count() * sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc(&u->x0f, u->nvox * sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc(&u->gout, u->nvox * sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc(&u->smax, sizeof(unsigned int));
@@ -866,7 +920,7 @@ void ocmc_unet_destroy(ocmc_unet* u)
     for (Act& A : u->acts) { cudaFree(A.x); cudaFree(A.g); }
     for (Layer& L : u->layers) { cudaFree(L.wf); cudaFree(L.wt); cudaFree(L.wtc_f); cudaFree(L.wtc_t); }
     cudaFree(u->params); cudaFree(u->grads); cudaFree(u->adam_m); cudaFree(u->adam_v); cudaFree(u->part);
-    cudaFree(u->tmpw); cudaFree(u->bpart);
+    cudaFree(u->bpart);
     cudaFree(u->x0f); cudaFree(u->gout); cudaFree(u->smax); cudaFree(u->lacc);
     cudaFree(u->fb); cudaFree(u->kerr);
     delete u;
@@ -930,14 +984,17 @@ ocmc_status ocmc_unet_train_step(ocmc_unet* u, const float* dose, const float* s
     const Layer& lastL = u->layers.back();
     const Act& last = u->acts[lastL.out_act];
     const int hb = stream_grid(n);
+    u->bpart_used = 0;
+    add_bias_sum(u, NLAYERS, hb, 17, u->head_w);
     k_head_bwd<<<hb, 256, 0, s>>>(last.x, u->params + u->head_w, u->gout, u->lacc, n, last.g, u->bpart);
-    sum_rows(u->bpart, hb, 17, u->grads + u->head_w, s);
     UCK(cudaGetLastError(), "head backward");
-    // layers in reverse; UP weight gradients come out as [p][n][c] and are transposed
+    // layers in reverse
     for (int i = (int)u->layers.size() - 1; i >= 0; --i) {
         const Layer& L = u->layers[i];
         UCK(layer_bwd(u, L, i > 0, s), "layer backward");
     }
+    k_sum_biases<<<dim3(4, NBIAS), dim3(32, 32), 0, s>>>(u->bpart, u->bias, u->grads);
+    UCK(cudaGetLastError(), "bias gradients");
     if (lr > 0.f) {
         u->step++;
         const float b1 = 0.9f, b2 = 0.999f;
@@ -1023,13 +1080,13 @@ ocmc_status ocmc_unet_test_layer(int device, int mode, int nx, int ny, int nz, i
     for (long long i = 0; i < ni * cin; ++i) hx[i] = __float2bfloat16_rn(x[i]);
     for (long long i = 0; i < no * cout; ++i) hdy[i] = __float2bfloat16_rn(dy[i]);
     __nv_bfloat16 *dX = nullptr, *dY = nullptr, *dDY = nullptr, *dDX = nullptr, *wf = nullptr, *wt = nullptr;
-    float *w32 = nullptr, *part = nullptr, *dW = nullptr, *dW2 = nullptr;
+    float *w32 = nullptr, *part = nullptr, *dW = nullptr;
     size_t part_n = (size_t)64 * 27 * 256 * 256;
     cudaError_t e = cudaSuccess;
     auto A = [&](void** p, size_t b) { if (e == cudaSuccess) e = cudaMalloc(p, b); };
     A((void**)&dX, ni * cin * 2); A((void**)&dY, no * cout * 2); A((void**)&dDY, no * cout * 2);
     A((void**)&dDX, ni * cin * 2); A((void**)&wf, nw * 2); A((void**)&wt, nw * 2); A((void**)&w32, nw * 4);
-    A((void**)&part, part_n * 4); A((void**)&dW, nw * 4); A((void**)&dW2, nw * 4);
+    A((void**)&part, part_n * 4); A((void**)&dW, nw * 4);
     __nv_bfloat16 *pf = nullptr, *pt = nullptr;
     int* kerr = nullptr;
     const bool tcf = tc_supported(m, cin, cout), tct = tc_supported(dgrad_mode(m), cout, cin);
@@ -1064,12 +1121,8 @@ ocmc_status ocmc_unet_test_layer(int device, int mode, int nx, int ny, int nz, i
     }
     if (e == cudaSuccess) {
         if (m == UP) {
-            e = launch_wgrad(DOWN, go, gi, Slice{dDY, cout, 0}, Slice{dX, cin, 0}, cout, cin, part, part_n, dW2, true,
-                             kerr, nullptr);
-            if (e == cudaSuccess) {
-                k_transpose_pnc<<<grid_for(nw), 256>>>(dW2, 8, cout, cin, dW);
-                e = cudaGetLastError();
-            }
+            e = launch_wgrad(DOWN, go, gi, Slice{dDY, cout, 0}, Slice{dX, cin, 0}, cout, cin, part, part_n, dW, true,
+                             kerr, nullptr, true);
         } else {
             e = launch_wgrad(m, gi, go, Slice{dX, cin, 0}, Slice{dDY, cout, 0}, cin, cout, part, part_n, dW, true, kerr,
                              nullptr);
@@ -1087,7 +1140,7 @@ ocmc_status ocmc_unet_test_layer(int device, int mode, int nx, int ny, int nz, i
         for (long long i = 0; i < ni * cin; ++i) dx[i] = __bfloat162float(hdx[i]);
     }
     cudaFree(dX); cudaFree(dY); cudaFree(dDY); cudaFree(dDX); cudaFree(wf); cudaFree(wt); cudaFree(w32);
-    cudaFree(part); cudaFree(dW); cudaFree(dW2); cudaFree(pf); cudaFree(pt); cudaFree(kerr);
+    cudaFree(part); cudaFree(dW); cudaFree(pf); cudaFree(pt); cudaFree(kerr);
     if (e != cudaSuccess) return OCMC_ERR_CUDA;
     return flag ? OCMC_ERR_TIMEOUT : OCMC_OK;
 }

@@ -372,11 +372,12 @@ __device__ __forceinline__ long long wsrc(const WgradArgs& a, long long r, int t
 
 // Weight-gradient partials: block (chunk, tap) computes the [BC x BN] tile
 // sum_{rows in chunk} x[src(row, tap)][c] * dy[row][n]; rows are the GEMM's K.
-// gridDim.z covers (cin / BC) x (cout / BN) tiles.
+// gridDim.z covers (cin / BC) x (cout / BN) tiles. Bound by the latency of its loads, so a K step is as
+// many rows as keep every thread loading (about 8 KB a step) and the caller gives about eight blocks a SM.
 template <int BC, int BN>
 __global__ void __launch_bounds__(THREADS) k_wgrad(const WgradArgs a)
 {
-    constexpr int KR = 32;                 // rows per K step
+    constexpr int KR = BC + BN <= 48 ? 96 : BC + BN <= 96 ? 64 : 32;   // rows per K step
     constexpr int XST = BC + 8, YST = BN + 8;
     __shared__ __align__(16) __nv_bfloat16 sX[2][KR * XST];
     __shared__ __align__(16) __nv_bfloat16 sY[2][KR * YST];

@@ -36,6 +36,7 @@
 #include <algorithm>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 
 #include "ocmc_umma.cuh"
 #include "ocmc_unet_kernels.cuh"
@@ -259,60 +260,88 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_conv3_tc(const __grid_constan
         int lt = 0;
         for (int tile = blockIdx.x; tile < a.ntiles && !*abort; tile += gridDim.x, ++lt) {
             const int acc = lt & 1, ua = lt >> 1;
-            if (!mbar_wait(&t_full[acc], ua & 1, abort, WAIT_NS)) break;
-            fence_after_sync();
             const int tx = tile % a.tiles_x, r = tile / a.tiles_x;
             const int x = tx * TX + (row & 7), y = (r % a.tiles_y) * TY + (row >> 3), z0 = (r / a.tiles_y) * TZ;
+            const bool inside = x < a.g.nx && y < a.g.ny;
+            const long long vox0 = x + (long long)a.g.nx * (y + (long long)a.g.ny * z0), plane = (long long)a.g.nx * a.g.ny;
+            // a data gradient's ReLU mask comes from global memory: loaded two slices ahead, the first two while
+            // the tile's MMAs still run (loaded where it was used, its latency made the masked 16 -> 16 layer
+            // over 128^3 take 108 us, twice the forward one). The slice loop stays a loop: unrolled, the
+            // epilogue no longer fits the instruction cache (forward layer 57 -> 74 us).
+            constexpr int MQ = NSL / 8;
+            uint4 m0[MQ], m1[MQ], m2[MQ];
+            auto load_mask = [&](uint4* m, int s) {
+                if (s < TZ && inside && z0 + s < a.g.nz) {
+                    const uint4* mk = reinterpret_cast<const uint4*>(a.mask + (vox0 + s * plane) * a.mask_stride + a.mask_c0 + n0);
+#pragma unroll
+                    for (int j = 0; j < MQ; ++j) m[j] = __ldg(mk + j);
+                }
+            };
+            if (a.mask) {
+                load_mask(m0, 0);
+                load_mask(m1, 1);
+            }
+            if (!mbar_wait(&t_full[acc], ua & 1, abort, WAIT_NS)) break;
+            fence_after_sync();
             // (with z-stacked taps output slice s is accumulator slice s + 2)
             const uint32_t tbase = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(acc * C::ASLICES * NSL) +
                                    (uint32_t)(C::ZS ? 2 * NSL : 0);
+            auto slices = [&](auto masked) {
+                constexpr bool MASKED = decltype(masked)::value;
 #pragma unroll 1
-            for (int s = 0; s < TZ; ++s) {
-                float v[NSL];
+                for (int s = 0; s < TZ; ++s) {
+                    if constexpr (MASKED) load_mask(m2, s + 2);
+                    float v[NSL];
 #pragma unroll
-                for (int j = 0; j < NSL / 16; ++j) tmem_ld16(tbase + (uint32_t)(s * NSL + 16 * j), v + 16 * j);
-                const int z = z0 + s;
-                if (x < a.g.nx && y < a.g.ny && z < a.g.nz) {
-                    const long long vox = x + (long long)a.g.nx * (y + (long long)a.g.ny * z);
-                    __nv_bfloat16* o = a.out.ptr + vox * a.out.stride + a.out.c0 + n0;
-                    const __nv_bfloat16* mk = a.mask ? a.mask + vox * a.mask_stride + a.mask_c0 + n0 : nullptr;
+                    for (int j = 0; j < NSL / 16; ++j) tmem_ld16(tbase + (uint32_t)(s * NSL + 16 * j), v + 16 * j);
+                    if (inside && z0 + s < a.g.nz) {
+                        __nv_bfloat16* o = a.out.ptr + (vox0 + s * plane) * a.out.stride + a.out.c0 + n0;
 #pragma unroll
-                    for (int j = 0; j < NSL / 8; ++j) {
-                        float f[8];
+                        for (int j = 0; j < MQ; ++j) {
+                            float f[8];
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) f[e] = v[8 * j + e] + sbias[8 * j + e];
-                        if (a.accumulate) {
-                            uint4 old = *reinterpret_cast<const uint4*>(o + 8 * j);
-                            const __nv_bfloat162* ob = reinterpret_cast<const __nv_bfloat162*>(&old);
+                            for (int e = 0; e < 8; ++e) f[e] = v[8 * j + e] + sbias[8 * j + e];
+                            if (a.accumulate) {
+                                uint4 old = *reinterpret_cast<const uint4*>(o + 8 * j);
+                                const __nv_bfloat162* ob = reinterpret_cast<const __nv_bfloat162*>(&old);
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                float2 p = __bfloat1622float2(ob[e]);
-                                f[2 * e] += p.x;
-                                f[2 * e + 1] += p.y;
+                                for (int e = 0; e < 4; ++e) {
+                                    float2 p = __bfloat1622float2(ob[e]);
+                                    f[2 * e] += p.x;
+                                    f[2 * e + 1] += p.y;
+                                }
                             }
-                        }
-                        if (a.relu) {
+                            if (a.relu) {
 #pragma unroll
-                            for (int e = 0; e < 8; ++e) f[e] = fmaxf(f[e], 0.f);
-                        }
-                        if (mk) {
-                            uint4 mv = *reinterpret_cast<const uint4*>(mk + 8 * j);
-                            const __nv_bfloat162* mb = reinterpret_cast<const __nv_bfloat162*>(&mv);
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                float2 p = __bfloat1622float2(mb[e]);
-                                if (!(p.x > 0.f)) f[2 * e] = 0.f;
-                                if (!(p.y > 0.f)) f[2 * e + 1] = 0.f;
+                                for (int e = 0; e < 8; ++e) f[e] = fmaxf(f[e], 0.f);
                             }
-                        }
-                        uint4 w;
-                        __nv_bfloat162* wb2 = reinterpret_cast<__nv_bfloat162*>(&w);
+                            if constexpr (MASKED) {
+                                const __nv_bfloat162* mb = reinterpret_cast<const __nv_bfloat162*>(&m0[j]);
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) wb2[e] = __floats2bfloat162_rn(f[2 * e], f[2 * e + 1]);
-                        *reinterpret_cast<uint4*>(o + 8 * j) = w;
+                                for (int e = 0; e < 4; ++e) {
+                                    float2 p = __bfloat1622float2(mb[e]);
+                                    if (!(p.x > 0.f)) f[2 * e] = 0.f;
+                                    if (!(p.y > 0.f)) f[2 * e + 1] = 0.f;
+                                }
+                            }
+                            uint4 w;
+                            __nv_bfloat162* wb2 = reinterpret_cast<__nv_bfloat162*>(&w);
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) wb2[e] = __floats2bfloat162_rn(f[2 * e], f[2 * e + 1]);
+                            *reinterpret_cast<uint4*>(o + 8 * j) = w;
+                        }
+                    }
+                    if constexpr (MASKED) {
+#pragma unroll
+                        for (int j = 0; j < MQ; ++j) {
+                            m0[j] = m1[j];
+                            m1[j] = m2[j];
+                        }
                     }
                 }
-            }
+            };
+            if (a.mask) slices(std::true_type{});
+            else slices(std::false_type{});
             fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive(&t_empty[acc]);
@@ -499,32 +528,52 @@ __global__ void __launch_bounds__(UP_THREADS, 1) k_up_tc(const __grid_constant__
         int it = 0;
         for (int tile = blockIdx.x; tile < a.ntiles && !*abort; tile += gridDim.x, ++it) {
             const int acc = it % C::NACC, ua = it / C::NACC;
-            if (!mbar_wait(&t_full[acc], ua & 1, abort, WAIT_NS)) break;
-            fence_after_sync();
             const int tx = tile % a.tiles_x, r = tile / a.tiles_x;
             const int x = tx * TX + (row & 7), y = (r % a.tiles_y) * TY + (row >> 3), z = r / a.tiles_y;
             const bool inside = x < a.g.nx && y < a.g.ny;
             const uint32_t tbase = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(acc * N);
-#pragma unroll 1
-            for (int p = p0; p < p0 + 4; ++p) {
-                const int ox = 2 * x + (p & 1), oy = 2 * y + ((p >> 1) & 1), oz = 2 * z + (p >> 2);
-                const bool ok = inside && ox < a.gfine.nx && oy < a.gfine.ny && oz < a.gfine.nz;
-                const long long vox = ox + (long long)a.gfine.nx * (oy + (long long)a.gfine.ny * oz);
+            // mask and previous value of the warp's four parities (16 channels at a time), the first ones
+            // loaded while the tile's MMAs still run
+            constexpr int J = COUT / 16;
+            uint4 mv[4][2], ov[4][2];
+            long long vox[4];
+            bool ok[4];
 #pragma unroll
-                for (int j = 0; j < COUT / 16; ++j) {
+            for (int k = 0; k < 4; ++k) {
+                const int p = p0 + k, ox = 2 * x + (p & 1), oy = 2 * y + ((p >> 1) & 1), oz = 2 * z + (p >> 2);
+                ok[k] = inside && ox < a.gfine.nx && oy < a.gfine.ny && oz < a.gfine.nz;
+                vox[k] = ox + (long long)a.gfine.nx * (oy + (long long)a.gfine.ny * oz);
+            }
+            auto load_extra = [&](int j) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        if (a.mask && ok[k])
+                            mv[k][h] = __ldg(reinterpret_cast<const uint4*>(a.mask + vox[k] * a.mask_stride + a.mask_c0 + 16 * j) + h);
+                        if (a.accumulate && ok[k])
+                            ov[k][h] = reinterpret_cast<const uint4*>(a.out.ptr + vox[k] * a.out.stride + a.out.c0 + 16 * j)[h];
+                    }
+            };
+            load_extra(0);
+            if (!mbar_wait(&t_full[acc], ua & 1, abort, WAIT_NS)) break;
+            fence_after_sync();
+#pragma unroll
+            for (int j = 0; j < J; ++j) {
+                if (j) load_extra(j);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
                     float v[16];
-                    tmem_ld16(tbase + (uint32_t)(p * COUT + 16 * j), v);   // every lane: the load is warp-wide
-                    if (!ok) continue;
-                    __nv_bfloat16* o = a.out.ptr + vox * a.out.stride + a.out.c0 + 16 * j;
-                    const __nv_bfloat16* mk = a.mask ? a.mask + vox * a.mask_stride + a.mask_c0 + 16 * j : nullptr;
+                    tmem_ld16(tbase + (uint32_t)((p0 + k) * COUT + 16 * j), v);   // every lane: the load is warp-wide
+                    if (!ok[k]) continue;
+                    __nv_bfloat16* o = a.out.ptr + vox[k] * a.out.stride + a.out.c0 + 16 * j;
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         float f[8];
 #pragma unroll
                         for (int e = 0; e < 8; ++e) f[e] = v[8 * h + e] + sbias[16 * j + 8 * h + e];
                         if (a.accumulate) {
-                            uint4 old = *reinterpret_cast<const uint4*>(o + 8 * h);
-                            const __nv_bfloat162* ob = reinterpret_cast<const __nv_bfloat162*>(&old);
+                            const __nv_bfloat162* ob = reinterpret_cast<const __nv_bfloat162*>(&ov[k][h]);
 #pragma unroll
                             for (int e = 0; e < 4; ++e) {
                                 float2 t2 = __bfloat1622float2(ob[e]);
@@ -536,9 +585,8 @@ __global__ void __launch_bounds__(UP_THREADS, 1) k_up_tc(const __grid_constant__
 #pragma unroll
                             for (int e = 0; e < 8; ++e) f[e] = fmaxf(f[e], 0.f);
                         }
-                        if (mk) {
-                            uint4 mv = *reinterpret_cast<const uint4*>(mk + 8 * h);
-                            const __nv_bfloat162* mb = reinterpret_cast<const __nv_bfloat162*>(&mv);
+                        if (a.mask) {
+                            const __nv_bfloat162* mb = reinterpret_cast<const __nv_bfloat162*>(&mv[k][h]);
 #pragma unroll
                             for (int e = 0; e < 4; ++e) {
                                 float2 t2 = __bfloat1622float2(mb[e]);
