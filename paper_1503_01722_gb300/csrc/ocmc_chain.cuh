@@ -1,0 +1,34 @@
+// ocmc_chain.cuh -- chained launches: a network pass is a chain of some twenty (forward) to a hundred
+// (training) kernels of 5 to 100 us, each waiting for the one before it. Launched as programmatic
+// dependents, a kernel's blocks are set up (barriers, tensor memory, weights) while the last blocks of the
+// kernel before it still run, and the launch itself costs the chain nothing.
+#pragma once
+#include <cuda_runtime.h>
+#include <utility>
+
+namespace ocmc {
+
+// Returns once the kernel before this one in the stream has completed and its writes are visible; at once
+// in a kernel that was launched plainly. Before it a kernel may only read what no kernel of its chain writes
+// (a chain starts with a plain launch, so everything older has completed).
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Lets the next kernel of the chain start once every block of this one has called it or ended.
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class... P, class... A>
+cudaError_t launch_chained(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... a)
+{
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, k, std::forward<A>(a)...);
+}
+
+}  // namespace ocmc

@@ -59,6 +59,8 @@ __global__ void __launch_bounds__(256) k_max_reduce(const float* __restrict__ x,
 __global__ void k_pack_input(const float* __restrict__ dose, const float* __restrict__ dens, const float* __restrict__ sigma,
                              long long n, const unsigned int* smax, __nv_bfloat16* x, float* x0f)
 {
+    chain_next();
+    chain_wait();
     float s = __uint_as_float(*smax);
     float inv = s > 0.f ? 1.f / s : 0.f;
     for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x) {
@@ -100,6 +102,8 @@ __global__ void __launch_bounds__(256) k_head_fwd(const __nv_bfloat16* __restric
                                                   const unsigned int* smax, const float* __restrict__ target,
                                                   const float* __restrict__ dens, float* __restrict__ out, double* acc)
 {
+    chain_next();
+    chain_wait();
     const float sc = __uint_as_float(*smax), inv = sc > 0.f ? 1.f / sc : 0.f;
     float wr[16];
 #pragma unroll
@@ -151,6 +155,8 @@ __global__ void __launch_bounds__(256) k_head_bwd(const __nv_bfloat16* __restric
                                                   const float* __restrict__ err, const double* acc, long long n,
                                                   __nv_bfloat16* gh, float* part /* [gridDim.x][17] */)
 {
+    chain_next();
+    chain_wait();
     const float sc = acc[1] > 0.0 ? (float)(2.0 / acc[1]) : 0.f;
     float wr[16], sw[17];
 #pragma unroll
@@ -220,6 +226,8 @@ __global__ void __launch_bounds__(1024) k_sum_rows(const float* part, int parts,
 __global__ void __launch_bounds__(256) k_sum_rows4(const float4* __restrict__ part, int parts, long long m4,
                                                    float* __restrict__ out, int tn, int tc)
 {
+    chain_next();
+    chain_wait();
     __shared__ float4 sh[32][9];
     const int x = threadIdx.x & 7, y = threadIdx.x >> 3;
     const long long j = blockIdx.x * 8ll + x;
@@ -255,13 +263,14 @@ __global__ void __launch_bounds__(256) k_sum_rows4(const float4* __restrict__ pa
 
 int sm_count();
 
-void sum_rows(const float* part, int parts, long long m, float* out, cudaStream_t s, int tn = 0, int tc = 0)
+cudaError_t sum_rows(const float* part, int parts, long long m, float* out, cudaStream_t s, int tn = 0, int tc = 0)
 {
     if (m % 4 == 0) {
-        k_sum_rows4<<<(unsigned)((m / 4 + 7) / 8), 256, 0, s>>>(reinterpret_cast<const float4*>(part), parts, m / 4, out, tn, tc);
-        return;
+        return launch_chained(k_sum_rows4, dim3((unsigned)((m / 4 + 7) / 8)), dim3(256), 0, s,
+                              reinterpret_cast<const float4*>(part), parts, m / 4, out, tn, tc);
     }
     k_sum_rows<<<(unsigned)((m + 31) / 32), dim3(32, 32), 0, s>>>(part, parts, (int)m, out);
+    return cudaGetLastError();
 }
 
 // Bias gradients of all layers (and the head's sums) from their partials in one launch: blockIdx.y is the
@@ -274,6 +283,8 @@ struct BiasSums {
 
 __global__ void __launch_bounds__(1024) k_sum_biases(const float* __restrict__ part, const BiasSums b, float* __restrict__ out)
 {
+    chain_next();
+    chain_wait();
     __shared__ float sh[32][33];
     const int l = blockIdx.y, m = b.m[l], parts = b.parts[l], j = blockIdx.x * 32 + threadIdx.x;
     if ((int)blockIdx.x * 32 >= m) return;
@@ -300,6 +311,8 @@ __global__ void __launch_bounds__(1024) k_sum_biases(const float* __restrict__ p
 // multiples of 8.
 __global__ void k_bias_part(const __nv_bfloat16* dy, int stride, int c0, int cout, long long n, float* part)
 {
+    chain_next();
+    chain_wait();
     __shared__ float sh[256 * 8];
     const int G = cout / 8, rpp = blockDim.x / G;
     const int g = threadIdx.x % G, r = threadIdx.x / G;
@@ -479,8 +492,7 @@ cudaError_t launch_conv_tile(const ConvArgs& a, dim3 grid, cudaStream_t s)
         attr = cudaFuncSetAttribute(k_conv<BK, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     });
     if (attr != cudaSuccess) return attr;
-    k_conv<BK, BN><<<grid, THREADS, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(k_conv<BK, BN>, grid, dim3(THREADS), smem, s, a);
 }
 
 int sm_count()
@@ -548,8 +560,7 @@ cudaError_t launch_wgrad3(Grid3 g, Slice x, Slice dy, int cin, int cout, float* 
         int parts = 0;
         cudaError_t e = launch_wgrad3_tc(g, x, dy, cin, cout, part, part_cap, err, s, &parts);
         if (e != cudaSuccess) return e;
-        sum_rows(part, parts, 27LL * cin * cout, dW, s);
-        return cudaGetLastError();
+        return sum_rows(part, parts, 27LL * cin * cout, dW, s);
     }
     Wgrad3Args a;
     a.g = g;
@@ -577,8 +588,7 @@ cudaError_t launch_wgrad3(Grid3 g, Slice x, Slice dy, int cin, int cout, float* 
     else k_wgrad3<32, 32><<<grid, THREADS, 0, s>>>(a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    sum_rows(part, (int)chunks, m, dW, s);
-    return cudaGetLastError();
+    return sum_rows(part, (int)chunks, m, dW, s);
 }
 
 // Weight gradient of one layer into dW (FP32, [taps][cin][cout]).
@@ -608,16 +618,15 @@ cudaError_t launch_wgrad(Mode mode, Grid3 gin, Grid3 gout, Slice x, Slice dy, in
     a.rows_per_chunk = (rows + chunks - 1) / chunks;
     a.partial = part;
     dim3 grid((unsigned)chunks, (unsigned)taps, (unsigned)tiles);
-#define WG(BC, BN) k_wgrad<BC, BN><<<grid, THREADS, 0, s>>>(a)
+    cudaError_t e = cudaSuccess;
+#define WG(BC, BN) e = launch_chained(k_wgrad<BC, BN>, grid, dim3(THREADS), 0, s, a)
     if (bc == 16) { if (bn == 16) WG(16, 16); else if (bn == 32) WG(16, 32); else WG(16, 64); }
     else if (bc == 32) { if (bn == 16) WG(32, 16); else if (bn == 32) WG(32, 32); else WG(32, 64); }
     else { if (bn == 16) WG(64, 16); else if (bn == 32) WG(64, 32); else WG(64, 64); }
 #undef WG
-    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     long long m = (long long)taps * cin * cout;
-    sum_rows(part, (int)chunks, m, dW, s, transpose ? cin : 0, transpose ? cout : 0);
-    return cudaGetLastError();
+    return sum_rows(part, (int)chunks, m, dW, s, transpose ? cin : 0, transpose ? cout : 0);
 }
 
 Slice slice_of(const ocmc_unet* u, int act, int c0, bool grad)
@@ -679,8 +688,8 @@ cudaError_t layer_bwd(ocmc_unet* u, const Layer& L, bool need_dx, cudaStream_t s
     const int blocks = (int)std::min<long long>(grid_for(nout * L.cout), 4LL * sm_count());
     const int k = (int)(&L - u->layers.data());
     add_bias_sum(u, k, blocks, L.cout, L.boff);
-    k_bias_part<<<blocks, 256, 0, s>>>(dy.ptr, dy.stride, dy.c0, L.cout, nout, u->bpart + u->bias.src[k]);
-    e = cudaGetLastError();
+    e = launch_chained(k_bias_part, dim3(blocks), dim3(256), 0, s, dy.ptr, dy.stride, dy.c0, L.cout, nout,
+                       u->bpart + u->bias.src[k]);
     if (e != cudaSuccess || !need_dx) return e;
     ConvArgs a;
     std::memset(&a, 0, sizeof(a));
@@ -738,8 +747,8 @@ ocmc_status forward(ocmc_unet* u, const float* dose, const float* sigma, const f
     long long n = u->nvox;
     UCK(cudaMemsetAsync(u->smax, 0, sizeof(unsigned int), s), "memset");
     k_max_reduce<<<stream_grid(n), 256, 0, s>>>(dose, n, u->smax);
-    k_pack_input<<<grid_for(n), 256, 0, s>>>(dose, dens, sigma, n, u->smax, u->acts[0].x, u->x0f);
     UCK(cudaGetLastError(), "input");
+    UCK(launch_chained(k_pack_input, dim3(grid_for(n)), dim3(256), 0, s, dose, dens, sigma, n, u->smax, u->acts[0].x, u->x0f), "input");
     for (const Layer& L : u->layers) UCK(layer_fwd(u, L, s), "layer forward");
     return OCMC_OK;
 }
@@ -748,9 +757,9 @@ ocmc_status forward(ocmc_unet* u, const float* dose, const float* sigma, const f
 ocmc_status head(ocmc_unet* u, const float* target, const float* dens, float* out, cudaStream_t s)
 {
     const Act& last = u->acts[u->layers.back().out_act];
-    k_head_fwd<<<stream_grid(u->nvox), 256, 0, s>>>(last.x, u->params + u->head_w, u->params + u->head_b, u->x0f, u->nvox,
-                                                    u->smax, target, dens, out, u->lacc);
-    UCK(cudaGetLastError(), "head");
+    UCK(launch_chained(k_head_fwd, dim3(stream_grid(u->nvox)), dim3(256), 0, s, last.x, u->params + u->head_w,
+                       u->params + u->head_b, u->x0f, u->nvox, u->smax, target, dens, out, u->lacc),
+        "head");
     return OCMC_OK;
 }
 
@@ -975,10 +984,10 @@ ocmc_status ocmc_unet_train_step(ocmc_unet* u, const float* dose, const float* s
     if (!u || !dose || !dens || !target) return ufail(u, OCMC_ERR_ARG, "NULL argument");
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     UCK(cudaSetDevice(u->device), "device");
+    UCK(cudaMemsetAsync(u->lacc, 0, 2 * sizeof(double), s), "memset");
     ocmc_status st = forward(u, dose, sigma, dens, s);
     if (st != OCMC_OK) return st;
     long long n = u->nvox;
-    UCK(cudaMemsetAsync(u->lacc, 0, 2 * sizeof(double), s), "memset");
     st = head(u, target, dens, u->gout, s);
     if (st != OCMC_OK) return st;
     const Layer& lastL = u->layers.back();
@@ -986,15 +995,15 @@ ocmc_status ocmc_unet_train_step(ocmc_unet* u, const float* dose, const float* s
     const int hb = stream_grid(n);
     u->bpart_used = 0;
     add_bias_sum(u, NLAYERS, hb, 17, u->head_w);
-    k_head_bwd<<<hb, 256, 0, s>>>(last.x, u->params + u->head_w, u->gout, u->lacc, n, last.g, u->bpart);
-    UCK(cudaGetLastError(), "head backward");
+    UCK(launch_chained(k_head_bwd, dim3(hb), dim3(256), 0, s, last.x, u->params + u->head_w, u->gout, u->lacc, n, last.g,
+                       u->bpart),
+        "head backward");
     // layers in reverse
     for (int i = (int)u->layers.size() - 1; i >= 0; --i) {
         const Layer& L = u->layers[i];
         UCK(layer_bwd(u, L, i > 0, s), "layer backward");
     }
-    k_sum_biases<<<dim3(4, NBIAS), dim3(32, 32), 0, s>>>(u->bpart, u->bias, u->grads);
-    UCK(cudaGetLastError(), "bias gradients");
+    UCK(launch_chained(k_sum_biases, dim3(4, NBIAS), dim3(32, 32), 0, s, u->bpart, u->bias, u->grads), "bias gradients");
     if (lr > 0.f) {
         u->step++;
         const float b1 = 0.9f, b2 = 0.999f;

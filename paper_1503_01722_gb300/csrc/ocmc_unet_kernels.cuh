@@ -23,6 +23,8 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include "ocmc_chain.cuh"
+
 namespace ocmc {
 namespace unet {
 
@@ -149,6 +151,8 @@ __global__ void __launch_bounds__(THREADS) k_conv(const ConvArgs a)
     constexpr int AST = BK + 8;        // smem row strides (bf16)
     constexpr int BST = BN + 8;
     extern __shared__ __align__(16) unsigned char conv_smem[];
+    chain_next();
+    chain_wait();
     __nv_bfloat16* sA = reinterpret_cast<__nv_bfloat16*>(conv_smem);                  // [NSTAGE][BM * AST]
     __nv_bfloat16* sB = sA + NSTAGE * BM * AST;                                        // [NSTAGE][BK * BST]
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -381,6 +385,8 @@ __global__ void __launch_bounds__(THREADS) k_wgrad(const WgradArgs a)
     constexpr int XST = BC + 8, YST = BN + 8;
     __shared__ __align__(16) __nv_bfloat16 sX[2][KR * XST];
     __shared__ __align__(16) __nv_bfloat16 sY[2][KR * YST];
+    chain_next();
+    chain_wait();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int t = blockIdx.y;
     const int tiles_n = a.cout / BN;
@@ -489,6 +495,8 @@ __global__ void __launch_bounds__(THREADS, 4) k_wgrad3(const Wgrad3Args a)
     constexpr int CX = BC / 8, CY = BN / 8;
     __shared__ __align__(16) __nv_bfloat16 sX[NST][XS];
     __shared__ __align__(16) __nv_bfloat16 sY[NST][YS];
+    chain_next();
+    chain_wait();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int dz = blockIdx.y;
     const int tiles_n = a.cout / BN;

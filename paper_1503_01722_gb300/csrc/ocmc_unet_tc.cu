@@ -152,6 +152,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_conv3_tc(const __grid_constan
     __syncthreads();
     fence_after_sync();
     const uint32_t tmem = *tmem_slot;
+    chain_next();
+    if (warp != 0) chain_wait();        // the producer waits after it has asked for the weights
 
     if (warp == 0) {
         // ---- producer: weights once, then one halo chunk per (tile, chunk) ----
@@ -160,6 +162,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_conv3_tc(const __grid_constan
             const uint8_t* wsrc = reinterpret_cast<const uint8_t*>(a.wpack) + (size_t)blockIdx.y * C::W_BYTES;
             for (uint32_t off = 0; off < C::W_BYTES; off += 32768u)
                 bulk_load(sw + off, wsrc + off, min(32768u, C::W_BYTES - off), w_full);
+            chain_wait();
             int it = 0;
             int last[NS];
 #pragma unroll
@@ -454,6 +457,8 @@ __global__ void __launch_bounds__(UP_THREADS, 1) k_up_tc(const __grid_constant__
     __syncthreads();
     fence_after_sync();
     const uint32_t tmem = *tmem_slot;
+    chain_next();
+    if (warp != 0) chain_wait();        // the producer waits after it has asked for the weights
 
     if (warp == 0) {
         // ---- producer: weights once, then every channel group of one tile per stage ----
@@ -462,6 +467,7 @@ __global__ void __launch_bounds__(UP_THREADS, 1) k_up_tc(const __grid_constant__
             const uint8_t* wsrc = reinterpret_cast<const uint8_t*>(a.wpack);
             for (uint32_t off = 0; off < C::W_BYTES; off += 32768u)
                 bulk_load(sw + off, wsrc + off, min(32768u, C::W_BYTES - off), w_full);
+            chain_wait();
             int it = 0;
             int last[NS];
 #pragma unroll
@@ -699,6 +705,8 @@ __global__ void __launch_bounds__(DOWN_THREADS, 1) k_down_tc(const TcArgs a, con
     __syncthreads();
     fence_after_sync();
     const uint32_t tmem = *tmem_slot;
+    chain_next();
+    if (warp != 0) chain_wait();        // warp 0 reads nothing but the weights
 
     if (warp == 0) {
         // ---- weights, then MMA issue: D[128 x COUT] = sum over parities of A_p[128 x CIN] W_p ----
@@ -923,8 +931,7 @@ cudaError_t launch_cfg(const ConvArgs& a, const __nv_bfloat16* wpack, int* err, 
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int slices = a.cout / NSL;
     const dim3 blocks((unsigned)std::max(1, std::min(t.ntiles, sms / slices)), (unsigned)slices);
-    k_conv3_tc<CIN, NSL, TZ, NS><<<blocks, TC_THREADS, C::SMEM, s>>>(m, t);
-    return cudaGetLastError();
+    return launch_chained(k_conv3_tc<CIN, NSL, TZ, NS>, blocks, dim3(TC_THREADS), C::SMEM, s, m, t);
 }
 
 template <int CIN, int COUT>
@@ -970,8 +977,7 @@ cudaError_t launch_up_cfg(const ConvArgs& a, const __nv_bfloat16* wpack, int* er
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    k_up_tc<CIN, COUT><<<(unsigned)std::max(1, std::min(t.ntiles, sms)), UP_THREADS, C::SMEM, s>>>(m, t);
-    return cudaGetLastError();
+    return launch_chained(k_up_tc<CIN, COUT>, dim3((unsigned)std::max(1, std::min(t.ntiles, sms))), dim3(UP_THREADS), C::SMEM, s, m, t);
 }
 
 template <int CIN, int COUT>
@@ -1004,9 +1010,8 @@ cudaError_t launch_down_cfg(const ConvArgs& a, const __nv_bfloat16* wpack, int* 
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    k_down_tc<CIN, COUT><<<(unsigned)std::max(1, std::min(t.ntiles, sms)), DOWN_THREADS, C::SMEM, s>>>(
-        t, a.in.ptr + a.in.c0, a.in.stride);
-    return cudaGetLastError();
+    return launch_chained(k_down_tc<CIN, COUT>, dim3((unsigned)std::max(1, std::min(t.ntiles, sms))), dim3(DOWN_THREADS), C::SMEM, s,
+                          t, (const __nv_bfloat16*)(a.in.ptr + a.in.c0), a.in.stride);
 }
 
 // Output channels per block: the whole layer where its weights fit next to the halo stages,

@@ -128,6 +128,8 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
     __syncthreads();
     fence_after_sync();
     const uint32_t tmem = *tmem_slot;
+    chain_next();
+    chain_wait();
     const uint32_t in_bytes = 9u * C::AT * a.pa;
 
     if (warp == 0) {
@@ -322,9 +324,8 @@ cudaError_t launch_wg_cfg(Grid3 g, Slice x, Slice dy, int cout, float* part, siz
             return cudaErrorInvalidValue;
     }
     const uint32_t smem = std::max<uint32_t>(WG_MIN_SMEM, (uint32_t)a.ns * a.stage + WG_TAIL);
-    k_wgrad3_tc<CIN, NSL><<<dim3((unsigned)blocks, (unsigned)slices), WG_THREADS, smem, s>>>(mx, md, a);
     *parts = (int)blocks;
-    return cudaGetLastError();
+    return launch_chained(k_wgrad3_tc<CIN, NSL>, dim3((unsigned)blocks, (unsigned)slices), dim3(WG_THREADS), smem, s, mx, md, a);
 }
 
 }  // namespace
