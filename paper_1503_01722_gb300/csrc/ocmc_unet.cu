@@ -553,13 +553,14 @@ cudaError_t launch_conv(const ConvArgs& a, cudaStream_t s)
 // Weight gradient of a 3x3x3 convolution over grid g (input and output) into dW [27][cin][cout]:
 // on tcgen05 where that kernel covers the channel counts (tc), else on mma.sync.
 cudaError_t launch_wgrad3(Grid3 g, Slice x, Slice dy, int cin, int cout, float* part, size_t part_cap, float* dW,
-                          bool tc, int* err, cudaStream_t s)
+                          bool tc, int* err, cudaStream_t s, float* bias, int* bias_parts)
 {
     if (tc && wgrad3_tc_fits(cin, cout, g.nx) && x.c0 % 8 == 0 && x.stride % 8 == 0 && dy.c0 % 8 == 0 &&
         dy.stride % 8 == 0) {
         int parts = 0;
-        cudaError_t e = launch_wgrad3_tc(g, x, dy, cin, cout, part, part_cap, err, s, &parts);
+        cudaError_t e = launch_wgrad3_tc(g, x, dy, cin, cout, part, part_cap, bias, err, s, &parts);
         if (e != cudaSuccess) return e;
+        if (bias) *bias_parts = 4 * parts;
         return sum_rows(part, parts, 27LL * cin * cout, dW, s);
     }
     Wgrad3Args a;
@@ -591,9 +592,11 @@ cudaError_t launch_wgrad3(Grid3 g, Slice x, Slice dy, int cin, int cout, float* 
     return sum_rows(part, (int)chunks, m, dW, s);
 }
 
-// Weight gradient of one layer into dW (FP32, [taps][cin][cout]).
+// Weight gradient of one layer into dW (FP32, [taps][cin][cout]; with transpose [taps][cout][cin]). With bias,
+// the tensor-memory kernel also writes *bias_parts rows of bias-gradient sums there (0 stays for the others).
 cudaError_t launch_wgrad(Mode mode, Grid3 gin, Grid3 gout, Slice x, Slice dy, int cin, int cout, float* part,
-                         size_t part_cap, float* dW, bool tc, int* err, cudaStream_t s, bool transpose = false)
+                         size_t part_cap, float* dW, bool tc, int* err, cudaStream_t s, bool transpose = false,
+                         float* bias = nullptr, int* bias_parts = nullptr)
 {
     // UP layers are handled as DOWN over (dy, x) with the roles of the grids swapped:
     // dW[p][c][n] = sum_u x[u][c] dy[2u+p][n]  ==  sum_u (DOWN gather of dy)[u][n] x[u][c]
@@ -605,7 +608,7 @@ cudaError_t launch_wgrad(Mode mode, Grid3 gin, Grid3 gout, Slice x, Slice dy, in
     a.dy = dy;
     a.cin = cin;
     a.cout = cout;
-    if (mode == CONV3) return launch_wgrad3(gout, x, dy, cin, cout, part, part_cap, dW, tc, err, s);
+    if (mode == CONV3) return launch_wgrad3(gout, x, dy, cin, cout, part, part_cap, dW, tc, err, s, bias, bias_parts);
     const int taps = 8;
     long long rows = gout.n();
     int bc = std::min(cin, 64), bn = std::min(cout, 64);
@@ -672,6 +675,7 @@ cudaError_t layer_bwd(ocmc_unet* u, const Layer& L, bool need_dx, cudaStream_t s
     Slice dy = slice_of(u, L.out_act, L.out_c0, true);
     Slice x = slice_of(u, L.in_act, L.in_c0, false);
     cudaError_t e;
+    int bias_parts = 0;
     if (L.mode == UP) {
         // dW[p][c][n] = sum_u x[u][c] dy[2u+p][n]: a DOWN-gather weight gradient over the coarse
         // grid with operands (dy as gathered input, x as rows), computed as [p][n][c] and transposed by the sum
@@ -679,17 +683,21 @@ cudaError_t layer_bwd(ocmc_unet* u, const Layer& L, bool need_dx, cudaStream_t s
                          u->kerr, s, true);
         if (e != cudaSuccess) return e;
     } else {
-        e = launch_wgrad(L.mode, u->g[L.lin], u->g[L.lout], x, dy, L.cin, L.cout, u->part, u->part_n,
-                         u->grads + L.woff, u->tc, u->kerr, s);
+        e = launch_wgrad(L.mode, u->g[L.lin], u->g[L.lout], x, dy, L.cin, L.cout, u->part, u->part_n, u->grads + L.woff, u->tc,
+                         u->kerr, s, false, u->bpart + u->bpart_used, &bias_parts);
         if (e != cudaSuccess) return e;
     }
-    long long nout = u->g[L.lout].n();
-    // four blocks per SM stream dy once; few partials keep their fixed-order sum short
-    const int blocks = (int)std::min<long long>(grid_for(nout * L.cout), 4LL * sm_count());
     const int k = (int)(&L - u->layers.data());
-    add_bias_sum(u, k, blocks, L.cout, L.boff);
-    e = launch_chained(k_bias_part, dim3(blocks), dim3(256), 0, s, dy.ptr, dy.stride, dy.c0, L.cout, nout,
-                       u->bpart + u->bias.src[k]);
+    if (bias_parts) {
+        add_bias_sum(u, k, bias_parts, L.cout, L.boff);
+    } else {
+        const long long nout = u->g[L.lout].n();
+        // four blocks per SM stream dy once; few partials keep their fixed-order sum short
+        const int blocks = (int)std::min<long long>(grid_for(nout * L.cout), 4LL * sm_count());
+        add_bias_sum(u, k, blocks, L.cout, L.boff);
+        e = launch_chained(k_bias_part, dim3(blocks), dim3(256), 0, s, dy.ptr, dy.stride, dy.c0, L.cout, nout,
+                           u->bpart + u->bias.src[k]);
+    }
     if (e != cudaSuccess || !need_dx) return e;
     ConvArgs a;
     std::memset(&a, 0, sizeof(a));

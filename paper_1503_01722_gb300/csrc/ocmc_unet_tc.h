@@ -48,11 +48,12 @@ cudaError_t launch_down_tc(const ConvArgs& a, const __nv_bfloat16* wpack, int* e
 // along x whose line stages fit shared memory (wgrad3_tc_fits): dW[t][c][n] = sum over voxels v
 // of grid g of x[v + d_t][c] dy[v][n]. Writes one partial [27][cin][cout] per block into part
 // (at most part_cap floats) and their count to *parts; the caller sums them in order. err (device
-// int, may be null) is set to 1 if a wait inside the kernel timed out.
+// int, may be null) is set to 1 if a wait inside the kernel timed out. bias (may be null): 4 *parts rows of
+// cout sums of dy, whose total is the bias gradient.
 bool wgrad3_tc_supported(int cin, int cout);
 bool wgrad3_tc_fits(int cin, int cout, int nx);
-cudaError_t launch_wgrad3_tc(Grid3 g, Slice x, Slice dy, int cin, int cout, float* part, size_t part_cap, int* err,
-                             cudaStream_t s, int* parts);
+cudaError_t launch_wgrad3_tc(Grid3 g, Slice x, Slice dy, int cin, int cout, float* part, size_t part_cap,
+                             float* bias, int* err, cudaStream_t s, int* parts);
 
 // The CUDA driver's cuTensorMapEncodeTiled (null if the installed driver does not provide it).
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder();

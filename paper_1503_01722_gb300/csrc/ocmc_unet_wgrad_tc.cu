@@ -32,8 +32,8 @@
 // its column blockIdx.x, and the caller sums the partials in a fixed order.
 //
 // Warp roles (192 threads): warp 0 issues the TMA copies (its lanes share each line's copies), warp
-// 1 owns tensor memory and one of its lanes issues the MMAs, warps 2-5 read the accumulators out at
-// the end (each warp its 32-lane quarter of tensor memory). Every wait gives up after two seconds,
+// 1 owns tensor memory and one of its lanes issues the MMAs, warps 2-5 sum dy over the lines (the bias
+// gradient) and read the accumulators out at the end (each warp its 32-lane quarter of tensor memory). Every wait gives up after two seconds,
 // sets the error flag, lets the copies and MMAs in flight finish and frees tensor memory before the
 // block exits.
 #include <cuda.h>
@@ -66,6 +66,7 @@ struct WgArgs {
     uint32_t pa, pb, stage;      // input atom, dy copy (P rows each, rounded up to 1 KB), stage bytes
     int ns;                      // stages
     float* partial;              // [gridDim.x][27][CIN][cout]
+    float* bias;                 // [gridDim.x][4][cout] sums of dy, or null
     int* err;
 };
 
@@ -116,7 +117,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
     if (threadIdx.x == 0) {
         for (int i = 0; i < NS; ++i) {
             mbar_init(&full[i], 1);
-            mbar_init(&empty[i], 1);
+            mbar_init(&empty[i], a.bias ? 5 : 1);   // the MMAs and the four warps that sum dy
         }
         mbar_init(done, 1);
         mbar_init(drain, 1);
@@ -205,6 +206,41 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
         // ---- epilogue: accumulators -> this block's slice of its partial dW ----
         const int q = warp & 3;                       // the tensor-memory lane quarter of this warp
         const int m = 32 * q + lane;
+        if (a.bias) {
+            // while the MMAs run: the bias gradient's sums from the staged dy line (copy 0), 16 bytes (eight
+            // channels) of a voxel at a time. A voxel's 16-byte pieces lie where TMA's swizzle put them: piece
+            // index XOR bits 7 and up of the row's address.
+            constexpr int GN = NSL / 8;
+            const int g = lane % GN, row0 = m / GN;
+            float acc[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) acc[e] = 0.f;
+            for (long long i = 0; i < nrows && !*abort; ++i) {
+                const int st = (int)(i % NS), u = (int)(i / NS);
+                if (!mbar_wait(&full[st], u & 1, abort, WG_WAIT_NS)) break;
+                const uint8_t* sb = smem + (size_t)st * a.stage + in_bytes;
+                for (int p = row0; p < a.P; p += 128 / GN) {
+                    const int piece = g ^ (((p * C::SPAN_B) >> 7) & (GN - 1));
+                    const uint4 w = *reinterpret_cast<const uint4*>(sb + p * C::SPAN_B + 16 * piece);
+                    const uint32_t h[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        acc[2 * e] += __uint_as_float(h[e] << 16);
+                        acc[2 * e + 1] += __uint_as_float(h[e] & 0xFFFF0000u);
+                    }
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&empty[st]);
+            }
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                for (int o = GN; o < 32; o <<= 1) acc[e] += __shfl_xor_sync(0xFFFFFFFFu, acc[e], o);
+            if (lane < GN) {
+                float* o = a.bias + ((size_t)blockIdx.x * 4 + q) * a.cout + n0 + 8 * g;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) o[e] = acc[e];
+            }
+        }
         if (mbar_wait(done, 0, abort, WG_WAIT_NS)) {
             fence_after_sync();
             float* P = a.partial + (size_t)blockIdx.x * 27 * CIN * a.cout;
@@ -259,7 +295,7 @@ uint32_t wg_stage_bytes(int cin, int nsl, int P)
 }
 
 template <int CIN, int NSL>
-cudaError_t launch_wg_cfg(Grid3 g, Slice x, Slice dy, int cout, float* part, size_t part_cap, int* err,
+cudaError_t launch_wg_cfg(Grid3 g, Slice x, Slice dy, int cout, float* part, size_t part_cap, float* bias, int* err,
                           cudaStream_t s, int* parts)
 {
     using C = WgCfg<CIN, NSL>;
@@ -285,6 +321,7 @@ cudaError_t launch_wg_cfg(Grid3 g, Slice x, Slice dy, int cout, float* part, siz
     a.ns = (int)std::min<uint32_t>(WG_MAX_STAGES, WG_STAGE_BUDGET / a.stage);
     a.err = err;
     a.partial = part;
+    a.bias = bias;
     if (a.ns < 1) return cudaErrorNotSupported;
     const int slices = cout / NSL;
     const long long m = 27LL * CIN * cout;
@@ -342,20 +379,20 @@ bool wgrad3_tc_fits(int cin, int cout, int nx)
     return wg_stage_bytes(cin, wg_slice(cin, cout), P) <= WG_STAGE_BUDGET;
 }
 
-cudaError_t launch_wgrad3_tc(Grid3 g, Slice x, Slice dy, int cin, int cout, float* part, size_t part_cap, int* err,
+cudaError_t launch_wgrad3_tc(Grid3 g, Slice x, Slice dy, int cin, int cout, float* part, size_t part_cap, float* bias, int* err,
                              cudaStream_t s, int* parts)
 {
     if (!wgrad3_tc_fits(cin, cout, g.nx) || x.c0 % 8 || x.stride % 8 || dy.c0 % 8 || dy.stride % 8 || g.ny < 1 ||
         g.nz < 1)
         return cudaErrorInvalidValue;
     const int nsl = wg_slice(cin, cout);
-    if (cin == 16) return nsl == 32 ? launch_wg_cfg<16, 32>(g, x, dy, cout, part, part_cap, err, s, parts)
-                                    : launch_wg_cfg<16, 16>(g, x, dy, cout, part, part_cap, err, s, parts);
-    if (cin == 32) return nsl == 32 ? launch_wg_cfg<32, 32>(g, x, dy, cout, part, part_cap, err, s, parts)
-                                    : launch_wg_cfg<32, 16>(g, x, dy, cout, part, part_cap, err, s, parts);
-    if (cin == 64) return nsl == 32 ? launch_wg_cfg<64, 32>(g, x, dy, cout, part, part_cap, err, s, parts)
-                                    : launch_wg_cfg<64, 16>(g, x, dy, cout, part, part_cap, err, s, parts);
-    return launch_wg_cfg<128, 16>(g, x, dy, cout, part, part_cap, err, s, parts);
+    if (cin == 16) return nsl == 32 ? launch_wg_cfg<16, 32>(g, x, dy, cout, part, part_cap, bias, err, s, parts)
+                                    : launch_wg_cfg<16, 16>(g, x, dy, cout, part, part_cap, bias, err, s, parts);
+    if (cin == 32) return nsl == 32 ? launch_wg_cfg<32, 32>(g, x, dy, cout, part, part_cap, bias, err, s, parts)
+                                    : launch_wg_cfg<32, 16>(g, x, dy, cout, part, part_cap, bias, err, s, parts);
+    if (cin == 64) return nsl == 32 ? launch_wg_cfg<64, 32>(g, x, dy, cout, part, part_cap, bias, err, s, parts)
+                                    : launch_wg_cfg<64, 16>(g, x, dy, cout, part, part_cap, bias, err, s, parts);
+    return launch_wg_cfg<128, 16>(g, x, dy, cout, part, part_cap, bias, err, s, parts);
 }
 
 }  // namespace unet
