@@ -5,6 +5,7 @@
 #include <cstdio>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 using namespace ocmc;
@@ -181,6 +182,7 @@ ocmc_status ensure_tally(ocmc_ctx* c)
     if (c->d_tally && c->tally_B == c->p.n_batches) return OCMC_OK;
     CK(dalloc(&c->d_tally, (size_t)c->p.n_batches * c->nvox), "tally allocation");
     CK(cudaMemset(c->d_tally, 0, sizeof(long long) * (size_t)c->p.n_batches * c->nvox), "tally reset");
+    c->tally_zero = true;
     c->tally_B = c->p.n_batches;
     c->nb.assign(c->tally_B, 0.0);
     c->ran = false;
@@ -217,6 +219,41 @@ void ctx_fill_args(const ocmc_ctx* c, TransportArgs& a) { fill_args(c, a); }
 void ctx_launch_shape(const ocmc_ctx* c, int* threads, int* blocks, int* cap, int* nreg)
 {
     launch_shape(c, threads, blocks, cap, nreg);
+}
+
+// The status that the run's error bits stand for.
+ocmc_status ctx_flag_status(ocmc_ctx* c, int e)
+{
+    if (e & ERR_PHANTOM) return fail(c, OCMC_ERR_ARG, "phantom contains invalid values");
+    if (e & ERR_BOUNDS) return fail(c, OCMC_ERR_BOUNDS, "a bounds check failed (checks build); the access was skipped");
+    if (e & ERR_OVERFLOW) return fail(c, OCMC_ERR_OVERFLOW, "a secondary stack overflowed; particles were dropped");
+    if (e & ERR_LIMIT) return fail(c, OCMC_ERR_TIMEOUT, "a particle hit the step or sampling iteration limit");
+    return OCMC_OK;
+}
+
+// Enqueues the dose (and, if asked for, sigma) of the current tally on the last run's stream; null outputs are
+// the context's own buffers.
+ocmc_status ctx_finalize(ocmc_ctx* c, float* dose, float* sigma, bool want_sigma)
+{
+    if (!c->have_phantom || !c->d_tally) return fail(c, OCMC_ERR_STATE, "no phantom/tally");
+    CK(cudaSetDevice(c->device), "cudaSetDevice");
+    double n = 0.0;
+    for (double v : c->nb) n += v;
+    if (!(n > 0.0)) return fail(c, OCMC_ERR_STATE, "no histories have been run");
+    cudaStream_t s = c->last_stream;
+    std::vector<float> inv(c->tally_B);
+    for (int b = 0; b < c->tally_B; ++b) inv[b] = c->nb[b] > 0 ? (float)(n / c->nb[b]) : 0.f;
+    if (c->tally_B > MAX_REG_BATCHES) {
+        if (c->invnb_cap < c->tally_B) {
+            CK(dalloc(&c->d_invnb, c->tally_B), "allocation");
+            c->invnb_cap = c->tally_B;
+        }
+        CK(cudaMemcpyAsync(c->d_invnb, inv.data(), sizeof(float) * c->tally_B, cudaMemcpyHostToDevice, s), "upload");
+    }
+    CK(launch_finalize(c->d_tally, c->d_density, c->tally_B, c->nvox, (double)c->dx * c->dy * c->dz, inv.data(), c->d_invnb,
+                       1.0 / n, dose ? dose : c->d_dose, want_sigma ? (sigma ? sigma : c->d_sigma) : nullptr, s),
+       "finalize launch");
+    return OCMC_OK;
 }
 
 ocmc_status ctx_ensure_stacks(ocmc_ctx* c, size_t warps, size_t records_per_warp)
@@ -314,20 +351,33 @@ ocmc_status ocmc_init(ocmc_ctx** out, int device, const ocmc_params* p)
     c->p = q;
     cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, device);
     cudaError_t r = cudaSuccess;
-    if (r == cudaSuccess) r = dalloc(&c->t.ph, MAX_STAGED * NE * 4);
-    if (r == cudaSuccess) r = dalloc(&c->t.el, MAX_STAGED * NE * 4);
-    if (r == cudaSuccess) r = dalloc(&c->t.el2, MAX_STAGED * NE * 2);
-    if (r == cudaSuccess) r = dalloc(&c->t.phmaj, NE);
-    if (r == cudaSuccess) r = dalloc(&c->t.elmaj, NE);
-    if (r == cudaSuccess) r = dalloc(&c->t.rinv, MAX_STAGED * NR);
-    if (r == cudaSuccess) r = dalloc(&c->t.msA, NG);
-    if (r == cudaSuccess) r = dalloc(&c->t.rmeta, 2 * MAX_STAGED);
-    if (r == cudaSuccess) r = dalloc(&c->t.msc, 2 * MAX_STAGED);
-    if (r == cudaSuccess) r = dalloc(&c->t.scratch, MAX_STAGED * NE);
-    if (r == cudaSuccess) r = dalloc(&c->t.rho_max, MAX_STAGED);
-    if (r == cudaSuccess) r = dalloc(&c->t.mats, MAX_STAGED);
-    if (r == cudaSuccess) r = dalloc(&c->t.mc, MAX_STAGED);
-    if (r == cudaSuccess) r = dalloc(&c->t.elem, MAX_STAGED * MAX_ELEM);
+    // the context's small arrays in one allocation (a cudaMalloc each took most of ocmc_init)
+    size_t used = 0;
+    auto place = [&](auto** p, size_t n) {
+        *p = reinterpret_cast<std::remove_reference_t<decltype(*p)>>(c->d_pool + used);
+        used = (used + n * sizeof(**p) + 255) / 256 * 256;
+    };
+    for (int pass = 0; pass < 2 && r == cudaSuccess; ++pass) {     // first the size, then the addresses
+        if (pass) r = cudaMalloc(reinterpret_cast<void**>(&c->d_pool), used);
+        used = 0;
+        place(&c->t.ph, MAX_STAGED * NE);
+        place(&c->t.el, MAX_STAGED * NE);
+        place(&c->t.el2, MAX_STAGED * NE);
+        place(&c->t.phmaj, NE);
+        place(&c->t.elmaj, NE);
+        place(&c->t.rinv, MAX_STAGED * NR);
+        place(&c->t.msA, NG);
+        place(&c->t.rmeta, 2 * MAX_STAGED);
+        place(&c->t.msc, 2 * MAX_STAGED);
+        place(&c->t.scratch, MAX_STAGED * NE);
+        place(&c->t.rho_max, MAX_STAGED);
+        place(&c->t.mats, MAX_STAGED);
+        place(&c->t.mc, MAX_STAGED);
+        place(&c->t.elem, MAX_STAGED * MAX_ELEM);
+        place(&c->d_stats, ST_COUNT + 1);                          // the error flag behind them: one clear
+        place(&c->d_counter, RUN_COUNTERS);
+        place(&c->d_sum, 1);
+    }
     {
         MatDef d[NMAT_DEFAULT];
         material_defs(d);
@@ -336,12 +386,9 @@ ocmc_status ocmc_init(ocmc_ctx** out, int device, const ocmc_params* p)
         c->slot_of = {0, 1, 2};
         c->t.n_mat = NMAT_DEFAULT;
     }
-    if (r == cudaSuccess) r = dalloc(&c->d_stats, ST_COUNT);
-    if (r == cudaSuccess) r = dalloc(&c->d_counter, RUN_COUNTERS);
-    if (r == cudaSuccess) r = dalloc(&c->d_sum, 1);
-    if (r == cudaSuccess) r = dalloc(&c->d_err, 1);
-    if (r == cudaSuccess) r = cudaMemset(c->d_stats, 0, ST_COUNT * sizeof(unsigned long long));
-    if (r == cudaSuccess) r = cudaMemset(c->d_err, 0, sizeof(int));
+    if (r == cudaSuccess) r = cudaHostAlloc(reinterpret_cast<void**>(&c->h_flags), 2 * sizeof(int), cudaHostAllocDefault);
+    if (r == cudaSuccess) c->d_err = reinterpret_cast<int*>(c->d_stats + ST_COUNT);
+    if (r == cudaSuccess) r = cudaMemset(c->d_stats, 0, (ST_COUNT + 1) * sizeof(unsigned long long));
     if (r == cudaSuccess) r = cudaEventCreate(&c->ev0);
     if (r == cudaSuccess) r = cudaEventCreate(&c->ev1);
     if (r != cudaSuccess) {
@@ -466,14 +513,13 @@ ocmc_status ocmc_create_phantom(ocmc_ctx* c, int nx, int ny, int nz, const float
     c->tables_valid = false;
     if (c->d_tally && c->tally_B == c->p.n_batches) {
         CK(cudaMemset(c->d_tally, 0, sizeof(long long) * (size_t)c->tally_B * n), "tally reset");
+        c->tally_zero = true;
         c->nb.assign(c->tally_B, 0.0);
         c->ran = false;
-        CK(cudaMemset(c->d_stats, 0, ST_COUNT * sizeof(unsigned long long)), "stats reset");
-        CK(cudaMemset(c->d_err, 0, sizeof(int)), "stats reset");
+        CK(cudaMemset(c->d_stats, 0, (ST_COUNT + 1) * sizeof(unsigned long long)), "stats reset");
         return OCMC_OK;
     }
-    CK(cudaMemset(c->d_stats, 0, ST_COUNT * sizeof(unsigned long long)), "stats reset");
-    CK(cudaMemset(c->d_err, 0, sizeof(int)), "stats reset");
+    CK(cudaMemset(c->d_stats, 0, (ST_COUNT + 1) * sizeof(unsigned long long)), "stats reset");
     return ensure_tally(c);
 }
 
@@ -619,6 +665,7 @@ ocmc_status ocmc_run_range(ocmc_ctx* c, uint64_t first, uint64_t count, uint64_t
     a.switch_low = c->p.switch_low ? c->p.switch_low : 8;
     a.refill_min = c->p.refill_min ? c->p.refill_min : 6;
     CK(cudaEventRecord(c->ev0, s), "event");
+    c->tally_zero = false;
     // A range is transported in launches of at most RUN_CHUNK histories: on GB300 a single launch
     // of 1e9 histories ran 15 % slower per history than ten launches of 1e8 (measured). Ranges
     // compose, so the tally is the same bit for bit.
@@ -647,41 +694,23 @@ static ocmc_status check_err_flag(ocmc_ctx* c)
 {
     int e = 0;
     CK(cudaMemcpy(&e, c->d_err, sizeof(int), cudaMemcpyDeviceToHost), "error flag");
-    if (e & ERR_PHANTOM) return fail(c, OCMC_ERR_ARG, "phantom contains invalid values");
-    if (e & ERR_BOUNDS) return fail(c, OCMC_ERR_BOUNDS, "a bounds check failed (checks build); the access was skipped");
-    if (e & ERR_OVERFLOW) return fail(c, OCMC_ERR_OVERFLOW, "a secondary stack overflowed; particles were dropped");
-    if (e & ERR_LIMIT) return fail(c, OCMC_ERR_TIMEOUT, "a particle hit the step or sampling iteration limit");
-    return OCMC_OK;
+    return ctx_flag_status(c, e);
 }
 
 ocmc_status ocmc_get_dose(ocmc_ctx* c, float* dose, float* sigma, int on_device)
 {
     if (!c || !dose) return fail(c, OCMC_ERR_ARG, "NULL argument");
-    if (!c->have_phantom || !c->d_tally) return fail(c, OCMC_ERR_STATE, "no phantom/tally");
-    CK(cudaSetDevice(c->device), "cudaSetDevice");
-    double n = 0.0;
-    for (double v : c->nb) n += v;
-    if (!(n > 0.0)) return fail(c, OCMC_ERR_STATE, "no histories have been run");
-    cudaStream_t s = c->last_stream;
-    if (c->invnb_cap < c->tally_B) {
-        CK(dalloc(&c->d_invnb, c->tally_B), "allocation");
-        c->invnb_cap = c->tally_B;
-    }
-    std::vector<float> inv(c->tally_B);
-    for (int b = 0; b < c->tally_B; ++b) inv[b] = c->nb[b] > 0 ? (float)(n / c->nb[b]) : 0.f;
-    CK(cudaMemcpyAsync(c->d_invnb, inv.data(), sizeof(float) * c->tally_B, cudaMemcpyHostToDevice, s), "upload");
     // device outputs are written in place; host outputs go through the context's buffers
-    float* dd = on_device ? dose : c->d_dose;
-    float* ds = sigma ? (on_device ? sigma : c->d_sigma) : nullptr;
-    CK(launch_finalize(c->d_tally, c->d_density, c->tally_B, c->nvox, (double)c->dx * c->dy * c->dz, c->d_invnb,
-                       1.0 / n, dd, ds, s),
-       "finalize launch");
+    ocmc_status st = ctx_finalize(c, on_device ? dose : nullptr, on_device ? sigma : nullptr, sigma != nullptr);
+    if (st != OCMC_OK) return st;
+    cudaStream_t s = c->last_stream;
     if (!on_device) {
         CK(cudaMemcpyAsync(dose, c->d_dose, sizeof(float) * c->nvox, cudaMemcpyDeviceToHost, s), "dose copy");
         if (sigma) CK(cudaMemcpyAsync(sigma, c->d_sigma, sizeof(float) * c->nvox, cudaMemcpyDeviceToHost, s), "sigma copy");
     }
+    CK(cudaMemcpyAsync(c->h_flags, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, s), "error flag");
     CK(cudaStreamSynchronize(s), "synchronize");
-    return check_err_flag(c);
+    return ctx_flag_status(c, c->h_flags[0]);
 }
 
 ocmc_status ocmc_get_raw_tally(ocmc_ctx* c, int64_t* out, int on_device)
@@ -705,17 +734,26 @@ ocmc_status ocmc_add_raw_tally(ocmc_ctx* c, const int64_t* in, int on_device, ui
     if (st != OCMC_OK) return st;
     long long n = (long long)c->tally_B * c->nvox;
     const long long* src = reinterpret_cast<const long long*>(in);
-    long long* tmp = nullptr;
-    if (!on_device) {
-        CK(cudaMalloc(&tmp, sizeof(long long) * n), "allocation");
-        cudaError_t e = cudaMemcpy(tmp, in, sizeof(long long) * n, cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) { cudaFree(tmp); return cuda_fail(c, e, "tally upload"); }
-        src = tmp;
+    cudaStream_t s = c->last_stream;
+    if (c->tally_zero) {
+        // onto a tally that nothing was added to since it was cleared: a copy, a third of the traffic
+        CK(cudaMemcpyAsync(c->d_tally, in, sizeof(long long) * n, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s),
+           "tally upload");
+        c->tally_zero = false;
+        CK(cudaStreamSynchronize(s), "tally add");
+    } else {
+        long long* tmp = nullptr;
+        if (!on_device) {
+            CK(cudaMalloc(&tmp, sizeof(long long) * n), "allocation");
+            cudaError_t e = cudaMemcpy(tmp, in, sizeof(long long) * n, cudaMemcpyHostToDevice);
+            if (e != cudaSuccess) { cudaFree(tmp); return cuda_fail(c, e, "tally upload"); }
+            src = tmp;
+        }
+        cudaError_t e = launch_add_tally(c->d_tally, src, n, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (tmp) cudaFree(tmp);
+        if (e != cudaSuccess) return cuda_fail(c, e, "tally add");
     }
-    cudaError_t e = launch_add_tally(c->d_tally, src, n, c->last_stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->last_stream);
-    if (tmp) cudaFree(tmp);
-    if (e != cudaSuccess) return cuda_fail(c, e, "tally add");
     add_histories(c, first, count);
     c->ran = true;
     return OCMC_OK;
@@ -725,11 +763,13 @@ ocmc_status ocmc_reset_tally(ocmc_ctx* c)
 {
     if (!c) return fail(c, OCMC_ERR_ARG, "ctx is NULL");
     CK(cudaSetDevice(c->device), "cudaSetDevice");
-    if (c->last_stream || c->ran) CK(cudaStreamSynchronize(c->last_stream), "synchronize");
-    if (c->d_tally) CK(cudaMemset(c->d_tally, 0, sizeof(long long) * (size_t)c->tally_B * c->nvox), "tally reset");
+    if (c->last_stream) CK(cudaStreamSynchronize(c->last_stream), "synchronize");   // the clears are on the default stream
+    if (c->d_tally) {
+        CK(cudaMemset(c->d_tally, 0, sizeof(long long) * (size_t)c->tally_B * c->nvox), "tally reset");
+        c->tally_zero = true;
+    }
     c->nb.assign(c->tally_B, 0.0);
-    CK(cudaMemset(c->d_stats, 0, ST_COUNT * sizeof(unsigned long long)), "stats reset");
-    CK(cudaMemset(c->d_err, 0, sizeof(int)), "stats reset");
+    CK(cudaMemset(c->d_stats, 0, (ST_COUNT + 1) * sizeof(unsigned long long)), "stats reset");
     c->ran = false;
     c->timed = false;
     return OCMC_OK;
@@ -807,11 +847,9 @@ void ocmc_destroy(ocmc_ctx* c)
     if (!c) return;
     cudaSetDevice(c->device);
     cudaDeviceSynchronize();
-    dfree(&c->d_density); dfree(&c->d_material); dfree(&c->d_tally); dfree(&c->d_stats);
-    dfree(&c->d_counter); dfree(&c->d_sum); dfree(&c->d_err); dfree(&c->d_stacks); dfree(&c->d_left); dfree(&c->d_dose);
-    dfree(&c->d_sigma); dfree(&c->d_invnb);
-    dfree(&c->t.ph); dfree(&c->t.el); dfree(&c->t.el2); dfree(&c->t.phmaj); dfree(&c->t.elmaj); dfree(&c->t.rinv); dfree(&c->t.msA);
-    dfree(&c->t.rmeta); dfree(&c->t.msc); dfree(&c->t.scratch); dfree(&c->t.rho_max); dfree(&c->t.mc); dfree(&c->t.elem); dfree(&c->t.mats);
+    dfree(&c->d_density); dfree(&c->d_material); dfree(&c->d_tally); dfree(&c->d_pool);
+    dfree(&c->d_stacks); dfree(&c->d_left); dfree(&c->d_dose); dfree(&c->d_sigma); dfree(&c->d_invnb);
+    if (c->h_flags) cudaFreeHost(c->h_flags);
     dfree(&c->d_bl); dfree(&c->d_bl_prefix); dfree(&c->d_bl_offs); dfree(&c->d_bl_caps); dfree(&c->d_bl_nnz);
     dfree(&c->d_bl_over); dfree(&c->d_bl_keys); dfree(&c->d_bl_vals); dfree(&c->d_dense); dfree(&c->d_chunks);
     dfree(&c->d_bl_tally); dfree(&c->d_bl_offsets); dfree(&c->d_bl_base); dfree(&c->d_bl_scale);

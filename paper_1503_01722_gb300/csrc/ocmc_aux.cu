@@ -19,15 +19,26 @@ __device__ __forceinline__ float i64_to_f32(long long x)
 
 // D_v = sum_b tally / (2^28 rho_v V N) in MeV/g per source particle (Sec. 2.2 "Materials");
 // sigma_D by the batch method (Sec. 3.1): sqrt(sum_b (D_b - D)^2 / (B (B - 1))) with the batch
-// means D_b = tally_b / (2^28 rho_v V n_b). Grid-stride over voxels. The integer sum is exact; the
-// rest is FP32, like the outputs (FP64 here made this kernel 13x slower than its memory traffic on
-// GB300's narrow FP64 pipe).
-__global__ void k_finalize(const long long* __restrict__ tally, const float* __restrict__ density, int B, long long nvox,
-                           float voxel_volume, const float* __restrict__ w_nb, float inv_n, float* dose,
-                           float* sigma)
+// means D_b = tally_b / (2^28 rho_v V n_b). The integer sum is exact; the rest is FP32, like the
+// outputs (FP64 here made this kernel 13x slower than its memory traffic on GB300's narrow FP64 pipe).
+// Bound by HBM: 8 B + 12 bytes a voxel. With NB > 0 a voxel's batches (B <= NB) are all loaded before
+// the first is used and stay in registers for the second sum; NB = 0 reads them twice, for any B.
+struct BatchWeights {
+    float w[MAX_REG_BATCHES];
+};
+
+template <int NB>
+__global__ void __launch_bounds__(256) k_finalize(const long long* __restrict__ tally, const float* __restrict__ density, int B,
+                                                  long long nvox, float voxel_volume, const BatchWeights wk,
+                                                  const float* __restrict__ w_nb, float inv_n, float* dose, float* sigma)
 {
     for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < nvox;
          v += (long long)gridDim.x * blockDim.x) {
+        long long q[NB > 0 ? NB : 1];
+        if constexpr (NB > 0) {
+#pragma unroll
+            for (int b = 0; b < NB; ++b) q[b] = b < B ? __ldcs(tally + (long long)b * nvox + v) : 0ll;
+        }
         const float rho = density[v];
         if (!(rho > 0.f)) {
             dose[v] = 0.f;
@@ -36,17 +47,29 @@ __global__ void k_finalize(const long long* __restrict__ tally, const float* __r
         }
         const float scale = inv_n / (rho * voxel_volume * 268435456.f);   // MeV/g per history per unit
         long long tot = 0;
-        for (int b = 0; b < B; ++b) tot += tally[(long long)b * nvox + v];
+        if constexpr (NB > 0) {
+#pragma unroll
+            for (int b = 0; b < NB; ++b) tot += q[b];
+        } else {
+            for (int b = 0; b < B; ++b) tot += tally[(long long)b * nvox + v];
+        }
         const float tf = i64_to_f32(tot);
         dose[v] = tf * scale;
         if (sigma) {
             // batch b's mean relative to the whole: tally_b * (N / n_b) - tot, in units of 2^32 tally
             // units so that the squares stay in FP32's range for any int64 tally
             float ss = 0.f;
+            auto add = [&](long long t, float w) {
+                const float d = fmaf(i64_to_f32(t), w, -tf) * 2.3283064365386963e-10f;
+                ss = fmaf(d, d, ss);
+            };
             if (B > 1) {
-                for (int b = 0; b < B; ++b) {
-                    const float d = fmaf(i64_to_f32(tally[(long long)b * nvox + v]), w_nb[b], -tf) * 2.3283064365386963e-10f;
-                    ss = fmaf(d, d, ss);
+                if constexpr (NB > 0) {
+#pragma unroll
+                    for (int b = 0; b < NB; ++b)
+                        if (b < B) add(q[b], wk.w[b]);
+                } else {
+                    for (int b = 0; b < B; ++b) add(tally[(long long)b * nvox + v], w_nb[b]);
                 }
                 ss /= (float)B * (float)(B - 1);
             }
@@ -452,11 +475,17 @@ cudaError_t launch_sum_tally(const long long* tally, long long n, unsigned long 
 }
 
 cudaError_t launch_finalize(const long long* tally, const float* density, int B, long long nvox, double voxel_volume,
-                            const float* w_nb, double inv_n, float* dose, float* sigma, cudaStream_t s)
+                            const float* w_host, const float* w_nb, double inv_n, float* dose, float* sigma, cudaStream_t s)
 {
-    int blocks = (int)std::min<long long>((nvox + 255) / 256, 152 * 16);
-    k_finalize<<<blocks > 0 ? blocks : 1, 256, 0, s>>>(tally, density, B, nvox, (float)voxel_volume, w_nb,
-                                                       (float)inv_n, dose, sigma);
+    const unsigned blocks = (unsigned)std::max<long long>(1, std::min<long long>((nvox + 255) / 256, 152 * 16));
+    BatchWeights wk{};
+    for (int b = 0; b < B && b < MAX_REG_BATCHES; ++b) wk.w[b] = w_host[b];
+    const float V = (float)voxel_volume, in = (float)inv_n;
+    if (B <= 4) k_finalize<4><<<blocks, 256, 0, s>>>(tally, density, B, nvox, V, wk, w_nb, in, dose, sigma);
+    else if (B <= 12) k_finalize<12><<<blocks, 256, 0, s>>>(tally, density, B, nvox, V, wk, w_nb, in, dose, sigma);
+    else if (B <= MAX_REG_BATCHES)
+        k_finalize<MAX_REG_BATCHES><<<blocks, 256, 0, s>>>(tally, density, B, nvox, V, wk, w_nb, in, dose, sigma);
+    else k_finalize<0><<<blocks, 256, 0, s>>>(tally, density, B, nvox, V, wk, w_nb, in, dose, sigma);
     return cudaGetLastError();
 }
 

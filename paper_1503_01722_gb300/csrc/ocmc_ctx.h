@@ -36,19 +36,22 @@ struct ocmc_ctx {
     std::vector<ocmc::MatDef> mats;
     std::vector<ocmc::MatDef> staged;
     std::vector<int> slot_of;                // defined index -> staged slot, -1 if not staged
-    // tables
+    // tables, statistics and counters: all in d_pool
+    unsigned char* d_pool = nullptr;
     ocmc::Tables t{};
     bool tables_valid = false;               // material and phantom parts both current
     bool mat_tables_valid = false;           // material part current (kept across phantoms of the same staged set)
     // tally and its history counts per batch
     long long* d_tally = nullptr;
+    bool tally_zero = false;                 // cleared, and nothing added since
     int tally_B = 0;
     std::vector<double> nb;
     // run scratch
     unsigned long long* d_stats = nullptr;
     unsigned long long* d_counter = nullptr;
     unsigned long long* d_sum = nullptr;
-    int* d_err = nullptr;
+    int* d_err = nullptr;           // behind d_stats
+    int* h_flags = nullptr;         // pinned: error bits on their way to the host (the run's, a network's)
     ocmc::PRec* d_stacks = nullptr;
     size_t stack_records = 0;
     int* d_left = nullptr;          // per warp: photons left to k_chains
@@ -106,6 +109,8 @@ namespace ocmc {
 ocmc_status ctx_fail(ocmc_ctx* c, ocmc_status s, const std::string& msg);
 ocmc_status ctx_cuda_fail(ocmc_ctx* c, cudaError_t e, const char* where);
 ocmc_status ctx_ensure_tables(ocmc_ctx* c, cudaStream_t s);
+ocmc_status ctx_flag_status(ocmc_ctx* c, int bits);
+ocmc_status ctx_finalize(ocmc_ctx* c, float* dose, float* sigma, bool want_sigma);
 void ctx_fill_args(const ocmc_ctx* c, TransportArgs& a);
 void ctx_launch_shape(const ocmc_ctx* c, int* threads, int* blocks, int* cap, int* nreg);
 ocmc_status ctx_ensure_stacks(ocmc_ctx* c, size_t warps, size_t records_per_warp);
