@@ -78,6 +78,28 @@ const char* check_params(const ocmc_params* p)
     return nullptr;
 }
 
+// Whether every material is below nd and every density in [0, 30]: loops without branches, which the
+// compiler vectorises (the voxel-by-voxel check with its early returns took 1.8 of a 128^3 phantom's
+// 2.1 ms). A density's bits: at most those of 30, or -0.
+bool values_valid(const float* density, const uint8_t* material, long long n, int nd)
+{
+    for (long long v0 = 0; v0 < n; v0 += 65536) {
+        const int k = (int)std::min<long long>(65536, n - v0);
+        const uint8_t* m = material + v0;
+        uint8_t top = 0;
+        for (int i = 0; i < k; ++i) top = m[i] > top ? m[i] : top;
+        const float* d = density + v0;
+        uint32_t bad = 0;
+        for (int i = 0; i < k; ++i) {
+            uint32_t u;
+            std::memcpy(&u, d + i, 4);
+            bad |= (uint32_t)(u > 0x41F00000u) & (uint32_t)(u != 0x80000000u);
+        }
+        if (bad || top >= nd) return false;
+    }
+    return true;
+}
+
 unsigned long long batch_count(unsigned long long N, int b, int B)
 {
     return N > (unsigned long long)b ? (N - b - 1) / B + 1 : 0ull;
@@ -460,13 +482,14 @@ ocmc_status ocmc_create_phantom(ocmc_ctx* c, int nx, int ny, int nz, const float
     long long n = (long long)nx * ny * nz;
     const int nd = (int)c->mats.size();
     bool used[MAX_MAT] = {false};
-    for (long long v = 0; v < n; ++v) {
-        if (material[v] >= nd)
-            return fail(c, OCMC_ERR_ARG, "material index must be below the number of defined materials (" +
-                                             std::to_string(nd) + ")");
-        if (!(density[v] >= 0.f && density[v] <= 30.f)) return fail(c, OCMC_ERR_ARG, "density must be in [0, 30] g/cm^3");
-        used[material[v]] = true;
-    }
+    if (nd > MAX_STAGED || !values_valid(density, material, n, nd))
+        for (long long v = 0; v < n; ++v) {
+            if (material[v] >= nd)
+                return fail(c, OCMC_ERR_ARG, "material index must be below the number of defined materials (" +
+                                                 std::to_string(nd) + ")");
+            if (!(density[v] >= 0.f && density[v] <= 30.f)) return fail(c, OCMC_ERR_ARG, "density must be in [0, 30] g/cm^3");
+            used[material[v]] = true;
+        }
     // staging: every defined material when they fit in a block's shared memory, else the
     // phantom's own materials in increasing index order (the uploaded indices are compacted)
     std::vector<int> slot(nd, -1);
