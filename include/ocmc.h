@@ -91,7 +91,8 @@ typedef struct {
                             /* size estimate times this; tables that fill up are   */
                             /* enlarged and the run repeated, so any value gives   */
                             /* the same dose (0: dense tallies where they fit)     */
-    int32_t refill_min;     /* free lanes a warp waits for before refilling (0=6)  */
+    int32_t refill_min;     /* free lanes a warp waits for before it refills (0:   */
+                            /* 12 in a warp of photons, 6 of charged particles)    */
     int32_t max_registers;  /* register cap of the transport kernel: 56, 64 or 80; */
                             /* 0 = 64 (with 1024-thread blocks)                    */
     float e_class_split;    /* MeV; > 0: charged particles waiting below this      */

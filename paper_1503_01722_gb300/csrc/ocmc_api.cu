@@ -686,7 +686,8 @@ ocmc_status ocmc_run_range(ocmc_ctx* c, uint64_t first, uint64_t count, uint64_t
     a.e_split = c->p.e_class_split;
     a.switch_high = c->p.switch_high ? c->p.switch_high : cap - cap / 16;
     a.switch_low = c->p.switch_low ? c->p.switch_low : 8;
-    a.refill_min = c->p.refill_min ? c->p.refill_min : 6;
+    a.refill_g = c->p.refill_min ? c->p.refill_min : REFILL_G;
+    a.refill_e = c->p.refill_min ? c->p.refill_min : REFILL_E;
     CK(cudaEventRecord(c->ev0, s), "event");
     c->tally_zero = false;
     // A range is transported in launches of at most RUN_CHUNK histories: on GB300 a single launch

@@ -160,6 +160,12 @@ struct PsRec {
 
 constexpr int RUN_COUNTERS = 2;
 
+// Free lanes before a refill when the parameters leave it to the library. A refill runs with the other
+// lanes idle: as long as several steps of a photon, about one of a charged particle. 1e7 photons of 6 MV on
+// the slab phantom: 12.5 ms at 6 free lanes, 11.7 at 8, 11.2 at 12, 11.2 at 14 (phase space of 2e6: 3.49,
+// 3.31, 3.12, 3.09); 1e7 electrons: 69.8, 69.9, 72.0, 73.1.
+constexpr int REFILL_G = 12, REFILL_E = 6;
+
 struct TransportArgs {
     // geometry
     int nx, ny, nz;
@@ -180,7 +186,8 @@ struct TransportArgs {
     int nstk;                   // 2 (photons, charged) or 3 (photons, charged >= e_split, charged < e_split)
     float e_split;              // MeV; energy-class boundary of the charged stacks when nstk == 3
     int switch_high, switch_low;
-    int refill_min;                      // free lanes needed before a warp refills (>= 1)
+    int refill_g, refill_e;              // free lanes needed before a warp of photons or of charged particles refills (>= 1)
+    int src_warps;                       // warps of each block that draw histories
     int src_share;                       // histories a warp draws at once, at most (1 to 32)
     int* left_out;                       // per warp: photons it ends with and leaves to k_chains (null: none)
     unsigned long long* n_left_out;

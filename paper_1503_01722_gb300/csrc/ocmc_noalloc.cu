@@ -239,7 +239,8 @@ extern "C" ocmc_status ocmc_run_noalloc(int device, int nx, int ny, int nz, cons
     a.e_split = p.e_class_split;
     a.switch_high = p.switch_high ? p.switch_high : cap - cap / 16;   // below the capacity: switching stays on
     a.switch_low = p.switch_low ? p.switch_low : 8;
-    a.refill_min = p.refill_min ? p.refill_min : 6;
+    a.refill_g = p.refill_min ? p.refill_min : REFILL_G;
+    a.refill_e = p.refill_min ? p.refill_min : REFILL_E;
     a.hist_counter = counter;
     a.stats = stats;
     a.err = err;

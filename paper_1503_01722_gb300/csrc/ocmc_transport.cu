@@ -688,12 +688,13 @@ __global__ void __maxnreg__(NREG) k_transport(const __grid_constant__ TransportA
     // primary of the other type goes to that type's stack like a secondary
     constexpr bool ps_src = PS && BL == ONE_BEAM;
     int mode = src_mode;
-    bool src_done = a.count == 0;
+    bool src_done = a.count == 0 || wib >= a.src_warps;
     // with switch_high >= cap, switching on stack size is off (stacks may then overflow, which
     // is reported); otherwise a warp also switches when another stack nears its capacity
     const int emergency = a.switch_high < a.cap ? a.cap - 128 : 0x7FFFFFFF;
     // most iterations only step: nothing to schedule while few lanes are free and no stack is large
-    const int plan_free = min(a.refill_min, 32 - a.switch_low), plan_top = min(a.switch_high, emergency);
+    const int plan_g = min(a.refill_g, 32 - a.switch_low), plan_e = min(a.refill_e, 32 - a.switch_low);
+    const int plan_top = min(a.switch_high, emergency);
     // per-warp scheduler counters live in shared memory (iterations, photon and charged lane-steps):
     // none of them takes a register under the register cap
     unsigned int* wc = s_wc[wib];
@@ -710,17 +711,23 @@ __global__ void __maxnreg__(NREG) k_transport(const __grid_constant__ TransportA
         Pend sec;
         sec.type = -1;
         unsigned act = __ballot_sync(FULL, active);
-        if (32 - __popc(act) >= plan_free || max(tops.x, max(tops.y, tops.z)) >= plan_top) {
+        if (32 - __popc(act) >= (mode ? plan_e : plan_g) || max(tops.x, max(tops.y, tops.z)) >= plan_top) {
             int top0 = min(tops.x, a.cap), top1 = min(tops.y, a.cap), top2 = a.nstk == 3 ? min(tops.z, a.cap) : 0;
             int nfree = 32 - __popc(act);
             // refill when enough lanes are free: the refill code runs on the free lanes only,
             // so waiting for several of them spreads its cost
-            if (nfree >= a.refill_min || nfree == 32) {
+            const int pool = mode == 1 ? top2 : (mode == 2 ? top1 : 0);   // the other charged stack
+            if (nfree >= (mode ? a.refill_e : a.refill_g) || nfree == 32) {
                 int topm = mode == 0 ? top0 : (mode == 1 ? top1 : top2);
                 int rank = __popc(~act & lt);
-                int take = min(nfree, topm);
+                const int own = min(nfree, topm);
+                // The classes are apart so that the lanes of a warp do alike steps (1e7 electrons of the slab
+                // phantom: 69.8 ms, 76.3 with one class). Once the source is empty a lane without work costs
+                // more than a mixed warp: 5e4 electrons of 15 MeV 1.08 ms with classes kept apart, 0.86 mixed.
+                const int mix = src_done ? min(nfree - own, pool) : 0, take = own + mix;
                 if (!active && rank < take) {
-                    pop_lane(c, mode, topm - 1 - rank, p);
+                    const bool o = rank < own;
+                    pop_lane(c, o ? mode : 3 - mode, o ? topm - 1 - rank : pool - 1 - (rank - own), p);
                     active = true;
                 }
                 int want = min(nfree - take, a.src_share);
@@ -753,11 +760,14 @@ __global__ void __maxnreg__(NREG) k_transport(const __grid_constant__ TransportA
                 }
                 __syncwarp();
                 if (lane == 0) {
-                    c.top[mode] = topm - take;
+                    c.top[mode] = topm - own;
+                    if (mix) c.top[3 - mode] = pool - mix;
                     if (wc[0] >= FLUSH_ITERS) flush_stats(a, s_st, wc);
                 }
                 __syncwarp();
-                if (mode == 0) top0 = topm - take; else if (mode == 1) top1 = topm - take; else top2 = topm - take;
+                if (mode == 0) top0 = topm - own;
+                else if (mode == 1) top1 = topm - own, top2 -= mix;
+                else top2 = topm - own, top1 -= mix;
                 act = __ballot_sync(FULL, active);
                 if (__any_sync(FULL, fate != LIVE)) {
                     if (fate != LIVE) finish(c, p, sec, fate);
@@ -768,7 +778,7 @@ __global__ void __maxnreg__(NREG) k_transport(const __grid_constant__ TransportA
             }
             int nact = __popc(act);
             const int topm = mode == 0 ? top0 : (mode == 1 ? top1 : top2);
-            bool m_avail = topm > 0 || ((ps_src || mode == src_mode) && !src_done);
+            bool m_avail = topm > 0 || (src_done ? (mode == 1 ? top2 : (mode == 2 ? top1 : 0)) > 0 : ps_src || mode == src_mode);
             // the other mode: the fullest other stack that has work (or that the source feeds)
             int other = -1, topo = 0;
 #pragma unroll
@@ -848,7 +858,7 @@ __global__ void __maxnreg__(NREG) k_transport(const __grid_constant__ TransportA
         if (!a.left_in) {
             atomicAdd(a.stats + ST_WARPS, 1ull);
             atomicMax(a.stats + ST_T_START_INV, ~t0);
-            atomicMax(a.stats + ST_T_SRC_INV, ~ts);
+            if (s_time[wib][1]) atomicMax(a.stats + ST_T_SRC_INV, ~ts);
         }
         atomicMax(a.stats + ST_T_END, t_end);
     }
@@ -924,6 +934,8 @@ __global__ void __launch_bounds__(32 * CHAIN_LANES) k_chains(const __grid_consta
 size_t transport_smem_bytes(int n_mat) { return smem_table_bytes(n_mat); }
 
 namespace {
+constexpr unsigned long long SRC_LANES = 28;
+
 template <int BL, bool PS, int R, bool XV = false>
 cudaError_t launch_variant(const TransportArgs& a, int blocks, int threads, size_t smem, cudaStream_t s)
 {
@@ -993,11 +1005,15 @@ static cudaError_t launch_one(const TransportArgs& a, int blocks, int threads, s
 cudaError_t launch_transport(const TransportArgs& args, int blocks, int threads, size_t smem, cudaStream_t s, int nreg)
 {
     TransportArgs a = args;
-    // A run with fewer histories than lanes is spread over all warps: a chain of steps takes longer in
-    // a fuller warp, and whole warps would stay without work (5e4 electrons of 15 MeV on 4864 warps:
-    // 1.30 ms with 32 histories a draw, 1.06 ms with 11).
-    const unsigned long long warps = (unsigned long long)blocks * (threads / 32), per = (a.count + warps - 1) / warps;
-    a.src_share = (int)std::min<unsigned long long>(32, std::max<unsigned long long>(1, per));
+    // A run with fewer histories than lanes is spread over all blocks, and in each over as few warps as
+    // hold its share at SRC_LANES a warp: whole blocks stay without work when every warp draws 32 at once,
+    // and a step of 10 lanes costs a warp as much as one of 30 (5e4 electrons of 15 MeV on 152 blocks of 32
+    // warps: 12 warps with 28 lanes 0.71 ms, 24 with 14 0.81, 32 with 11 0.84; 1e5 photons 0.82, 0.83, 0.85).
+    // Warps in fours, as a block's warps are dealt out to the four schedulers in turn.
+    const unsigned long long warps = (unsigned long long)blocks * (threads / 32), per = (a.count + blocks - 1) / blocks;
+    const unsigned long long busy = (per + SRC_LANES - 1) / SRC_LANES;
+    a.src_warps = (int)std::min<unsigned long long>(threads / 32, (busy + 3) / 4 * 4);
+    a.src_share = (int)std::min<unsigned long long>(32, (per + a.src_warps - 1) / a.src_warps);
     int* left = a.left_out;                      // one count per warp; null: no room for it, every warp finishes its photons
     a.n_left_out = a.hist_counter + 1;
     cudaError_t e = launch_one(a, blocks, threads, smem, s, nreg);
