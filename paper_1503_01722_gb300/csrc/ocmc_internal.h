@@ -187,6 +187,7 @@ struct TransportArgs {
     float e_split;              // MeV; energy-class boundary of the charged stacks when nstk == 3
     int switch_high, switch_low;
     int refill_g, refill_e;              // free lanes needed before a warp of photons or of charged particles refills (>= 1)
+    bool held;                           // a warp's hard events of electrons wait for one another
     int src_warps;                       // warps of each block that draw histories
     int src_share;                       // histories a warp draws at once, at most (1 to 32)
     int* left_out;                       // per warp: photons it ends with and leaves to k_chains (null: none)

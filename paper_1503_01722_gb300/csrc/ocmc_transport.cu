@@ -47,6 +47,7 @@ namespace {
 constexpr unsigned FULL = 0xFFFFFFFFu;
 constexpr int MAX_WARPS = 32;
 constexpr int STEP_LIMIT = 1 << 22;
+constexpr int HELD_MIN = 6;
 constexpr int CHAIN_LANES = 8;    // a warp flies chains together while at most this many photons are left in it
 constexpr int CHAIN_STEPS = 24;   // flights in a row that make a chain (a photon makes about 6 in water)
 constexpr uint32_t CHAIN_MAX_N = 4u * STEP_LIMIT;   // draws after which a photon is left to its steps and their limit
@@ -353,9 +354,36 @@ __device__ __forceinline__ void hard_event(C& c, Lane& p, int m, float sM, float
     p.E = Tk - W;
 }
 
-// One condensed-history step.
+// The candidate hard event of a lane that has waited with it: what charged_step does otherwise at the end
+// of the step, with the material and the random block fetched again. (Written out in both places: with one
+// function for both, the kernel without waiting ran 0.3 % slower.)
 template <class C>
-__device__ __forceinline__ int charged_step(C& c, Lane& p, Pend& sec)
+__device__ __forceinline__ int held_candidate(C& c, Lane& p, float sighat, Pend& sec)
+{
+    const TransportArgs& a = c.a;
+    const SmemTables& T = c.T;
+    if (vox_bad(c, p)) return GONE;
+    const int m = __ldg(a.material + (p.ix + a.nx * (p.iy + a.ny * p.iz))), mb = m * MS4;
+    if (p.r.n & 3u) p.r.buf = philox_block(p.r.n >> 2, p.r.h0, p.r.h1, p.r.sub, a.key0, a.key1);
+    EIdx e2 = e_index(p.E);
+    float4 A2 = T.el[mb + e2.i], B2 = T.el[mb + e2.i + 1];
+    float sM = p.E > 2.f * a.pp.w_cc ? lerp1(A2.z, B2.z, e2.f) : 0.f;
+    float sB = p.E > a.pp.w_cb ? lerp1(A2.w, B2.w, e2.f) : 0.f;
+    float tot = sM + sB;
+    if (tot > sighat * 1.00001f) count_rare(c, ST_VIOL, 1);
+    if (rng_u(p.r, a.key0, a.key1) * sighat < tot) {
+        hard_event(c, p, m, sM, tot, sec);
+        if (p.E < a.pp.e_abs_e) return ABSORBED;
+    } else {
+        count(c, ST_HARD_FICT);
+    }
+    return LIVE;
+}
+
+// One condensed-history step. With HELD a candidate hard event at its end is left to held_candidate, and
+// *held receives its majorant.
+template <bool HELD, class C>
+__device__ __forceinline__ int charged_step(C& c, Lane& p, Pend& sec, float* held)
 {
     const TransportArgs& a = c.a;
     const SmemTables& T = c.T;
@@ -423,6 +451,10 @@ __device__ __forceinline__ int charged_step(C& c, Lane& p, Pend& sec)
     if (geo) return LIVE;
     if (p.E < a.pp.e_abs_e) return ABSORBED;
     if (lim == 3 && !crossed) {
+        if constexpr (HELD) {
+            *held = sighat;
+            return LIVE;
+        }
         EIdx e2 = e_index(p.E);
         float4 A2 = T.el[mb + e2.i], B2 = T.el[mb + e2.i + 1];
         float sM = p.E > 2.f * a.pp.w_cc ? lerp1(A2.z, B2.z, e2.f) : 0.f;
@@ -656,13 +688,30 @@ __device__ __noinline__ void flush_stats(const TransportArgs& a, BlockStats& st,
     }
 }
 
+// A particle that never ends: dropped, with its energy counted.
+template <class C>
+__device__ __forceinline__ int step_limit(C& c, const Lane& p)
+{
+    atomicOr(c.a.err, ERR_LIMIT);
+    count_rare(c, ST_DROPPED, 1);
+    count_rare(c, ST_E_DROPPED, fx(p.E));
+    return GONE;
+}
+
 // NREG: register cap per thread. More registers spill less; fewer registers let more
 // warps share an SM (80: 3 x 256 threads, 64: 2 x 512, 56: 3 x 384 on GB300).
 // PS: the source is a phase space (per-history records of mixed particle types); a separate
 // instantiation, so that the analytic-source kernel carries none of its code.
-// XV: electron steps cross voxel faces (the fixed-step variant); a separate instantiation of the
-// analytic-source kernel, so the voxel-limited kernels carry none of its code.
-template <int BL, bool PS, int NREG, bool XV = false>
+// STEPS: the kind of electron steps, again an instantiation of the analytic-source kernel each.
+// CROSS lets them cross voxel faces (the fixed-step variant). HELD takes apart what only a few lanes of a
+// warp do after a step. A candidate hard event, whose code is as long as the step's, waits until HELD_MIN
+// of the warp or a quarter of its lanes have one; those make no step meanwhile (6 % more iterations). A
+// particle that ended without a secondary is put away when its lane is about to be refilled, which it
+// waits for anyway. 5e6 electrons of 15 MeV on the half-slab phantom: 35.2 -> 32.3 ms (HELD_MIN 3: 33.9,
+// 4: 33.1, 6 to 16: 32.5); 6e5 on water 3.71 -> 3.42 ms. The electrons of a photon beam have fewer
+// events a step and lose by waiting (1e8 photons of 6 MV: 95.9 ms, 99.5 with it).
+enum { PLAIN = 0, CROSS, HELD };
+template <int BL, bool PS, int NREG, int STEPS = PLAIN>
 __global__ void __maxnreg__(NREG) k_transport(const __grid_constant__ TransportArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -704,14 +753,31 @@ __global__ void __maxnreg__(NREG) k_transport(const __grid_constant__ TransportA
     bool active = false, just_switched = false;
     Lane p;
     int left = 0;                // photons this warp leaves to fly_chains
+    int fate = LIVE;
+    Pend sec;
+    sec.type = -1;
+    float held = 0.f;            // > 0: the lane waits with a candidate hard event of this majorant
     for (;;) {
         __syncwarp();
-        const int4 tops = *reinterpret_cast<const int4*>(c.top);
-        int fate = LIVE;
-        Pend sec;
-        sec.type = -1;
         unsigned act = __ballot_sync(FULL, active);
-        if (32 - __popc(act) >= (mode ? plan_e : plan_g) || max(tops.x, max(tops.y, tops.z)) >= plan_top) {
+        if constexpr (STEPS == HELD) {
+            // what the last step emitted goes to its stack at once; particles that ended without emitting
+            // anything keep until the free lanes are about to be refilled
+            if (__any_sync(FULL, sec.type >= 0) ||
+                (32 - __popc(act) >= (mode ? a.refill_e : a.refill_g) && __any_sync(FULL, fate != LIVE))) {
+                if (fate != LIVE || sec.type >= 0) finish(c, p, sec, fate);
+                fate = LIVE;
+                sec.type = -1;
+                __syncwarp();
+            }
+        } else {
+            fate = LIVE;
+            sec.type = -1;
+        }
+        const int4 tops = *reinterpret_cast<const int4*>(c.top);
+        const int fullest = max(tops.x, max(tops.y, tops.z));
+        bool settle = false;     // the waiting candidates now, no steps
+        if (32 - __popc(act) >= (mode ? plan_e : plan_g) || fullest >= plan_top) {
             int top0 = min(tops.x, a.cap), top1 = min(tops.y, a.cap), top2 = a.nstk == 3 ? min(tops.z, a.cap) : 0;
             int nfree = 32 - __popc(act);
             // refill when enough lanes are free: the refill code runs on the free lanes only,
@@ -769,7 +835,7 @@ __global__ void __maxnreg__(NREG) k_transport(const __grid_constant__ TransportA
                 else if (mode == 1) top1 = topm - own, top2 -= mix;
                 else top2 = topm - own, top1 -= mix;
                 act = __ballot_sync(FULL, active);
-                if (__any_sync(FULL, fate != LIVE)) {
+                if (STEPS != HELD && __any_sync(FULL, fate != LIVE)) {
                     if (fate != LIVE) finish(c, p, sec, fate);
                     if (act == 0) continue;
                     fate = LIVE;
@@ -792,7 +858,7 @@ __global__ void __maxnreg__(NREG) k_transport(const __grid_constant__ TransportA
             }
             const bool o_avail = other >= 0;
             if (nact == 0) {
-                if (m_avail) continue;
+                if (m_avail || (STEPS == HELD && __any_sync(FULL, fate != LIVE))) continue;
                 if (o_avail) { mode = other; continue; }
                 break;
             }
@@ -809,8 +875,11 @@ __global__ void __maxnreg__(NREG) k_transport(const __grid_constant__ TransportA
             // few photons left in the warp, nothing to refill from and one of them in a long chain of
             // fictitious events: the warp ends and leaves them to k_chains, after the other stacks' work
             const bool chain = a.left_out && !sw && mode == 0 && !m_avail && nact <= CHAIN_LANES && !just_switched &&
-                               __any_sync(FULL, active && p.steps >= CHAIN_STEPS && p.r.n < CHAIN_MAX_N);
-            if (sw || chain) {
+                               __any_sync(FULL, active && p.steps >= CHAIN_STEPS && p.r.n < CHAIN_MAX_N) &&
+                               !(STEPS == HELD && __any_sync(FULL, fate != LIVE));
+            if (STEPS == HELD && sw && __any_sync(FULL, held > 0.f)) {
+                settle = true;
+            } else if (sw || chain) {
                 if (active) {
                     push(c, mode ? charged_stack(a, p.E) : 0, p, p.E, p.u, p.v, p.w, p.type, p.r.sub, p.r.n);
                     active = false;
@@ -822,23 +891,37 @@ __global__ void __maxnreg__(NREG) k_transport(const __grid_constant__ TransportA
             }
             just_switched = false;
         }
+        const unsigned step = STEPS != HELD ? act : settle ? 0u : act & ~__ballot_sync(FULL, held > 0.f);
         if (lane == 0) {
             atomicAdd(wc, 1u);
-            atomicAdd(wc + (mode ? 2 : 1), (unsigned)__popc(act));
+            atomicAdd(wc + (mode ? 2 : 1), (unsigned)__popc(step));
         }
-        if (active) {
+        if constexpr (STEPS == HELD) {
+            bool done = step >> lane & 1u;
+            if (done) fate = mode ? charged_step<true>(c, p, sec, &held) : photon_step(c, p, sec);
+            // (all of them while a stack is within one iteration's pushes of the point where the warp must
+            // switch: it then switches at once)
+            const int waits = __popc(__ballot_sync(FULL, held > 0.f));
+            if (waits && (settle || waits >= HELD_MIN || 4 * waits >= __popc(act) || fullest >= emergency - 96)) {
+                if (held > 0.f) {
+                    fate = held_candidate(c, p, held, sec);
+                    held = 0.f;
+                    done = true;
+                }
+            }
+            if (done && !(held > 0.f)) {
+                if (fate == LIVE && ++p.steps > STEP_LIMIT) fate = step_limit(c, p);
+                active = fate == LIVE;
+                if (fate == GONE) fate = LIVE;       // nothing left to do
+            }
+        } else if (active) {
             if (mode) {
-                if constexpr (XV) fate = charged_step_cross(c, p, sec);
-                else fate = charged_step(c, p, sec);
+                if constexpr (STEPS == CROSS) fate = charged_step_cross(c, p, sec);
+                else fate = charged_step<false>(c, p, sec, nullptr);
             } else {
                 fate = photon_step(c, p, sec);
             }
-            if (fate == LIVE && ++p.steps > STEP_LIMIT) {
-                atomicOr(a.err, ERR_LIMIT);
-                count_rare(c, ST_DROPPED, 1);
-                count_rare(c, ST_E_DROPPED, fx(p.E));
-                fate = GONE;
-            }
+            if (fate == LIVE && ++p.steps > STEP_LIMIT) fate = step_limit(c, p);
             active = fate == LIVE;
             if (fate > GONE || sec.type >= 0) finish(c, p, sec, fate);
         }
@@ -935,14 +1018,18 @@ size_t transport_smem_bytes(int n_mat) { return smem_table_bytes(n_mat); }
 
 namespace {
 constexpr unsigned long long SRC_LANES = 28;
+// Histories a warp from which an electron beam's run holds its hard events: below, a run is the chain of
+// steps of its last particles, which waiting lengthens. With 4864 warps, without and with it: 5e4 histories
+// 0.71 and 0.74 ms, 1e5 1.68 and 1.73, 2e5 1.54 and 1.55, 3e5 3.17 and 3.19, 6e5 5.33 and 5.06, 1e6 8.13 and 7.70.
+constexpr unsigned long long HELD_HISTORIES = 64;
 
-template <int BL, bool PS, int R, bool XV = false>
+template <int BL, bool PS, int R, int STEPS = PLAIN>
 cudaError_t launch_variant(const TransportArgs& a, int blocks, int threads, size_t smem, cudaStream_t s)
 {
     cudaError_t e =
-        cudaFuncSetAttribute(k_transport<BL, PS, R, XV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(k_transport<BL, PS, R, STEPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_transport<BL, PS, R, XV><<<blocks, threads, smem, s>>>(a);
+    k_transport<BL, PS, R, STEPS><<<blocks, threads, smem, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -956,12 +1043,18 @@ int occupancy(int threads, size_t smem)
     return n;
 }
 
+template <int STEPS, int BL = ONE_BEAM, bool PS = false>
+cudaError_t launch_steps(const TransportArgs& a, int blocks, int threads, size_t smem, cudaStream_t s, int nreg)
+{
+    if (nreg == 56) return launch_variant<BL, PS, 56, STEPS>(a, blocks, threads, smem, s);
+    if (nreg == 64) return launch_variant<BL, PS, 64, STEPS>(a, blocks, threads, smem, s);
+    return launch_variant<BL, PS, 80, STEPS>(a, blocks, threads, smem, s);
+}
+
 template <int BL, bool PS>
 cudaError_t launch_source(const TransportArgs& a, int blocks, int threads, size_t smem, cudaStream_t s, int nreg)
 {
-    if (nreg == 56) return launch_variant<BL, PS, 56>(a, blocks, threads, smem, s);
-    if (nreg == 64) return launch_variant<BL, PS, 64>(a, blocks, threads, smem, s);
-    return launch_variant<BL, PS, 80>(a, blocks, threads, smem, s);
+    return launch_steps<PLAIN, BL, PS>(a, blocks, threads, smem, s, nreg);
 }
 }  // namespace
 
@@ -978,9 +1071,12 @@ int transport_max_blocks_per_sm(int threads, size_t smem, int nreg)
     occupancy<ONE_BEAM, true, 56>(threads, smem);
     occupancy<ONE_BEAM, true, 64>(threads, smem);
     occupancy<ONE_BEAM, true, 80>(threads, smem);
-    cudaFuncSetAttribute(k_transport<ONE_BEAM, false, 56, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(k_transport<ONE_BEAM, false, 64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(k_transport<ONE_BEAM, false, 80, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(k_transport<ONE_BEAM, false, 56, CROSS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(k_transport<ONE_BEAM, false, 56, HELD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(k_transport<ONE_BEAM, false, 64, CROSS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(k_transport<ONE_BEAM, false, 64, HELD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(k_transport<ONE_BEAM, false, 80, CROSS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(k_transport<ONE_BEAM, false, 80, HELD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (nreg == 56) return occupancy<ONE_BEAM, false, 56>(threads, smem);
     if (nreg == 64) return occupancy<ONE_BEAM, false, 64>(threads, smem);
     return occupancy<ONE_BEAM, false, 80>(threads, smem);
@@ -991,14 +1087,13 @@ static cudaError_t launch_one(const TransportArgs& a, int blocks, int threads, s
     if (a.pp.flags & FLAG_CROSS_VOXELS) {
         // voxel-crossing electron steps: analytic single-beam source only (callers check)
         if (a.beamlets || a.ps) return cudaErrorInvalidValue;
-        if (nreg == 56) return launch_variant<ONE_BEAM, false, 56, true>(a, blocks, threads, smem, s);
-        if (nreg == 64) return launch_variant<ONE_BEAM, false, 64, true>(a, blocks, threads, smem, s);
-        return launch_variant<ONE_BEAM, false, 80, true>(a, blocks, threads, smem, s);
+        return launch_steps<CROSS>(a, blocks, threads, smem, s, nreg);
     }
     if (a.beamlets)
         return a.bl_dense ? launch_source<BEAMLETS_DENSE, false>(a, blocks, threads, smem, s, nreg)
                           : launch_source<BEAMLETS_HASH, false>(a, blocks, threads, smem, s, nreg);
     if (a.ps) return launch_source<ONE_BEAM, true>(a, blocks, threads, smem, s, nreg);
+    if (a.held) return launch_steps<HELD>(a, blocks, threads, smem, s, nreg);
     return launch_source<ONE_BEAM, false>(a, blocks, threads, smem, s, nreg);
 }
 
@@ -1014,6 +1109,7 @@ cudaError_t launch_transport(const TransportArgs& args, int blocks, int threads,
     const unsigned long long busy = (per + SRC_LANES - 1) / SRC_LANES;
     a.src_warps = (int)std::min<unsigned long long>(threads / 32, (busy + 3) / 4 * 4);
     a.src_share = (int)std::min<unsigned long long>(32, (per + a.src_warps - 1) / a.src_warps);
+    a.held = a.src.particle == 1 && !a.beamlets && !a.ps && a.count >= HELD_HISTORIES * warps;
     int* left = a.left_out;                      // one count per warp; null: no room for it, every warp finishes its photons
     a.n_left_out = a.hist_counter + 1;
     cudaError_t e = launch_one(a, blocks, threads, smem, s, nreg);
