@@ -32,15 +32,17 @@ import ocmc_inputs as I  # noqa: E402
 # launch of 2e7 histories of the default workload) and DRAM bytes of a full launch, from ncu
 # captures of the current kernel on GB300 (re-measured whenever the kernel changes). Lanes that
 # a branch switched off are not counted.
-INST_PER_LANE_STEP = 595.5
+INST_PER_LANE_STEP = 489.4
 # DRAM bytes of one transport launch measured by ncu on the full default workload
-DRAM_BYTES_PER_LAUNCH = {("photon_slab_120", 100_000_000): 20.235e9}
-# the same (predicated-on) for the beamlet-mode kernel (hash tallies) on the 512-beamlet CT
-# workload, measured by ncu on full runs of the same workload with every beamlet's histories
-# scaled by 0.2
-INST_PER_LANE_STEP_BEAMLETS = 607.2
+DRAM_BYTES_PER_LAUNCH = {("photon_slab_120", 100_000_000): 20.309e9}
+# the same (predicated-on) for the beamlet-mode kernel (dense tallies), measured by ncu on a run of
+# 1.14e7 6 MV histories in 64 beamlets on a CT-like phantom of 128x128x96 voxels (one metric, one
+# pass: the 512 beamlets' dense tallies hold 34 GB)
+INST_PER_LANE_STEP_BEAMLETS = 507.0
 # the library transports a run in launches of at most this many histories (plus one finalize)
 RUN_CHUNK = 100_000_000
+# kernels of one such launch: the transport, the long photon chains its warps left, and their resumption
+KERNELS_PER_RUN = 3
 
 WORKLOADS = {
     "photon_slab_120": (I.photon_slab_120, 100_000_000,
@@ -296,7 +298,7 @@ def run_beamlets_bench(args, make, desc):
         "config": {"workload": desc, "histories_per_step": r["histories_per_step"], "beamlets": r["beamlets"],
                    "l2": "flushed between steps (256 MB write)", "seed": 1},
         "e2e": r["e2e"],
-        "gpu_launches": args.steps,
+        "gpu_launches": KERNELS_PER_RUN * args.steps,
         "clocks": r["clocks"],
         "kernel_stats_last_step": r["kernel_stats_last_step"],
         "roofline": r["roofline"],
@@ -559,7 +561,7 @@ def run_half_slab_throughput(args, desc):
             "n_gpus": 1, "steps": args.steps, "warmup": args.warmup, "ms_per_step": r["ms_per_step"],
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
             "config": {"workload": desc, "histories_per_step": 2 * n, "l2": "flushed between steps (256 MB write)"},
-            "per_beam": r["per_beam"], "gpu_launches": 2 * ((n + RUN_CHUNK - 1) // RUN_CHUNK + 1) * args.steps,
+            "per_beam": r["per_beam"], "gpu_launches": 2 * (KERNELS_PER_RUN * ((n + RUN_CHUNK - 1) // RUN_CHUNK) + 1) * args.steps,
             "clocks": r["clocks"]}
     print(json.dumps(line))
 
@@ -603,7 +605,7 @@ def run_voxel_sweep(args, desc):
             "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
             "config": {"workload": desc, "value_is": "15 MeV electrons at 2.5 mm, voxel-limited steps",
                        "timing": "transport kernel (CUDA events inside the library)"},
-            "gpu_launches": 2 * args.steps * len(rows), "sweep": rows}
+            "gpu_launches": KERNELS_PER_RUN * args.steps * len(rows), "sweep": rows}
     print(json.dumps(line))
 
 
@@ -796,7 +798,7 @@ def main():
                    "parallelism": f"histories sharded over {world} GPU(s), int64 tally all-reduce" if world > 1
                    else "1 GPU"},
         "e2e": e2e,
-        "gpu_launches": 2 * args.steps,
+        "gpu_launches": (KERNELS_PER_RUN * ((n + RUN_CHUNK - 1) // RUN_CHUNK) + 1) * args.steps,
         "roofline": roofline,
         "clocks": clocks,
         "wall_s": wall,

@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(256) k_max_reduce(const float* __restrict__ x,
 }
 
 // x0 = dose / s, x1 = density, x2 = sigma / s (0 without sigma), channels 3-15 zero: whole sectors are
-// written (stores of the first channels alone made L2 fetch every sector first: 22 us for 128^3, now 14).
+// written (stores of the first channels alone made L2 fetch every sector first: 22 us for 128^3, now 18).
 __global__ void k_pack_input(const float* __restrict__ dose, const float* __restrict__ dens, const float* __restrict__ sigma,
                              long long n, const unsigned int* smax, __nv_bfloat16* x, float* x0f)
 {
@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(256) k_head_fwd(const __nv_bfloat16* __restric
 }
 
 // head backward: g = err 2 / count, gh[v][c] = g w[c] (h > 0); partial sums of g h and g per block.
-// 16-byte loads and stores of a voxel's channels (175 us for 128^3 with two bytes at a time, now 40).
+// 16-byte loads and stores of a voxel's channels (175 us for 128^3 with two bytes at a time, now 26).
 __global__ void __launch_bounds__(256) k_head_bwd(const __nv_bfloat16* __restrict__ h, const float* __restrict__ w,
                                                   const float* __restrict__ err, const double* acc, long long n,
                                                   __nv_bfloat16* gh, float* part /* [gridDim.x][17] */)
