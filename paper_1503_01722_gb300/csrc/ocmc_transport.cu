@@ -54,13 +54,14 @@ constexpr uint32_t CHAIN_MAX_N = 4u * STEP_LIMIT;   // draws after which a photo
 
 // Block statistics in shared memory: event counts as 32-bit words (shared memory adds 32-bit
 // integers natively and a warp's lanes together; a 64-bit shared add is a compare-and-swap loop
-// per lane), the two energy sums that hot paths add to as 32-bit halves. Counts move to the
+// per lane), the energy sums that hot paths add to as 32-bit halves. Counts move to the
 // 64-bit totals in global memory before a word can wrap (flush_stats) and when a warp ends.
 struct BlockStats {
     unsigned int n[ST_E_IN];       // event counts, slots [0, ST_E_IN)
-    unsigned int e[2][2];          // energy in, energy escaped: low and high words
+    unsigned int e[3][2];          // energy sums ST_E_IN .. ST_E_MISS: low and high words
 };
-enum { BE_IN = 0, BE_ESC = 1 };
+enum { BE_IN = 0, BE_ESC, BE_MISS };
+static_assert(ST_E_ESC - ST_E_IN == BE_ESC && ST_E_MISS - ST_E_IN == BE_MISS, "the block's sums in the totals' order");
 
 // Source and tally of a launch, compile-time so that each kernel carries only its own code: one beam
 // with a dense tally per statistical batch, beamlets with a dense tally each (a particle's batch is
@@ -82,7 +83,8 @@ struct CtxT {
 template <class C>
 __device__ __forceinline__ void count(C& c, int k) { atomicAdd(&c.st->n[k], 1u); }
 
-// rare events and energies go straight to the totals
+// what hardly ever happens goes straight to the totals (not the energy of particles that miss the phantom:
+// 1.6e7 photons, two thirds of which miss, took 10.6 ms with a global atomic each, 3.5 without)
 template <class C>
 __device__ __forceinline__ void count_rare(C& c, int k, unsigned long long v) { atomicAdd(c.a.stats + k, v); }
 
@@ -685,10 +687,10 @@ __device__ __noinline__ void flush_stats(const TransportArgs& a, BlockStats& st,
     }
     // the halves one after the other: a carry that arrives between the two is added by the next flush
 #pragma unroll 1
-    for (int k = 0; k < 2; ++k) {
+    for (int k = 0; k <= BE_MISS; ++k) {
         const unsigned lo = atomicExch(&st.e[k][0], 0u), hi = atomicExch(&st.e[k][1], 0u);
         const unsigned long long q = ((unsigned long long)hi << 32) + lo;
-        if (q) atomicAdd(a.stats + (k == BE_IN ? ST_E_IN : ST_E_ESC), q);
+        if (q) atomicAdd(a.stats + ST_E_IN + k, q);
     }
 #pragma unroll 1
     for (int k = 0; k < 3; ++k) {
@@ -821,11 +823,10 @@ __global__ void __maxnreg__(NREG) k_transport(const __grid_constant__ TransportA
                         if constexpr (BL != ONE_BEAM) in = init_beamlet(a, base + r2, p);
                         else if constexpr (ps_src) in = init_phase_space(a, a.first + base + r2, p);
                         else in = init_primary(a, a.first + base + r2, p);
+                        add_energy(c, in ? BE_IN : BE_MISS, fx(p.E));
                         if (!in) {
                             count(c, ST_MISSED);
-                            count_rare(c, ST_E_MISS, fx(p.E));
                         } else {
-                            add_energy(c, BE_IN, fx(p.E));
                             const bool charged = p.type != PHOTON;
                             if (!(p.E >= (charged ? a.pp.e_abs_e : a.pp.e_abs_g)) || (charged && (a.pp.flags & 8))) fate = ABSORBED;
                             else if (ps_src && (charged ? charged_stack(a, p.E) : 0) != mode) fate = MOVED;
