@@ -763,7 +763,7 @@ __global__ void __maxnreg__(NREG) k_transport(const __grid_constant__ TransportA
     // three stacks), 2 charged particles below e_split
     bool active = false, just_switched = false;
     Lane p;
-    int left = 0;                // photons this warp leaves to fly_chains
+    int left = 0;                // photons this warp leaves to k_chains
     int fate = LIVE;
     Pend sec;
     sec.type = -1;
