@@ -224,6 +224,8 @@ ocmc_status ocmc_load_phase_space(ocmc_ctx* ctx, const char* path);
  * deposited energy to the tally (Sec. 2.2.1, Table 1 loop). Asynchronous on
  * cuda_stream (a cudaStream_t, NULL = the legacy default stream); the call
  * returns after the launch. Repeated calls accumulate; use different seeds.
+ * Calls on one context may name different streams: each call's work runs behind the
+ * work of all earlier calls on that context.
  * Errors: OCMC_ERR_STATE without phantom or source, OCMC_ERR_ARG if n is 0. */
 ocmc_status ocmc_run(ocmc_ctx* ctx, uint64_t n_histories, uint64_t seed, void* cuda_stream);
 
@@ -253,7 +255,8 @@ ocmc_status ocmc_get_raw_tally(ocmc_ctx* ctx, int64_t* out, int on_device);
 ocmc_status ocmc_add_raw_tally(ocmc_ctx* ctx, const int64_t* in, int on_device,
                                uint64_t first, uint64_t count);
 
-/* Zero the tally, the history count and the statistics. */
+/* Zero the tally, the history count and the statistics, behind the runs in flight
+ * (it does not wait for them). */
 ocmc_status ocmc_reset_tally(ocmc_ctx* ctx);
 
 /* Statistics of the runs since the last reset (synchronises); after ocmc_run_beamlets, of that

@@ -199,11 +199,11 @@ ocmc_status ensure_tables(ocmc_ctx* c, cudaStream_t s)
     return OCMC_OK;
 }
 
-ocmc_status ensure_tally(ocmc_ctx* c)
+ocmc_status ensure_tally(ocmc_ctx* c, cudaStream_t s)
 {
     if (c->d_tally && c->tally_B == c->p.n_batches) return OCMC_OK;
     CK(dalloc(&c->d_tally, (size_t)c->p.n_batches * c->nvox), "tally allocation");
-    CK(cudaMemset(c->d_tally, 0, sizeof(long long) * (size_t)c->p.n_batches * c->nvox), "tally reset");
+    CK(cudaMemsetAsync(c->d_tally, 0, sizeof(long long) * (size_t)c->p.n_batches * c->nvox, s), "tally reset");
     c->tally_zero = true;
     c->tally_B = c->p.n_batches;
     c->nb.assign(c->tally_B, 0.0);
@@ -234,6 +234,24 @@ void launch_shape(const ocmc_ctx* c, int* threads, int* blocks, int* cap, int* n
 }  // namespace
 
 namespace ocmc {
+CallOrder::CallOrder(ocmc_ctx* c, cudaStream_t s) : c_(c), s_(s)
+{
+    if (s) {
+        cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+        if ((err_ = cudaStreamIsCapturing(s, &st)) != cudaSuccess) return;
+        if ((capturing_ = st != cudaStreamCaptureStatusNone)) return;
+        if (c->order_default && (err_ = cudaEventRecord(c->order, nullptr)) != cudaSuccess) return;
+    }
+    if (s || !c->order_default) err_ = cudaStreamWaitEvent(s, c->order, 0);
+}
+
+CallOrder::~CallOrder()
+{
+    if (capturing_ || err_ != cudaSuccess) return;
+    c_->order_default = !s_;
+    if (s_) cudaEventRecord(c_->order, s_);
+}
+
 ocmc_status ctx_fail(ocmc_ctx* c, ocmc_status s, const std::string& msg) { return fail(c, s, msg); }
 ocmc_status ctx_cuda_fail(ocmc_ctx* c, cudaError_t e, const char* where) { return cuda_fail(c, e, where); }
 ocmc_status ctx_ensure_tables(ocmc_ctx* c, cudaStream_t s) { return ensure_tables(c, s); }
@@ -263,6 +281,8 @@ ocmc_status ctx_finalize(ocmc_ctx* c, float* dose, float* sigma, bool want_sigma
     for (double v : c->nb) n += v;
     if (!(n > 0.0)) return fail(c, OCMC_ERR_STATE, "no histories have been run");
     cudaStream_t s = c->last_stream;
+    CallOrder call(c, s);
+    CK(call.error(), "order");
     std::vector<float> inv(c->tally_B);
     for (int b = 0; b < c->tally_B; ++b) inv[b] = c->nb[b] > 0 ? (float)(n / c->nb[b]) : 0.f;
     if (c->tally_B > MAX_REG_BATCHES) {
@@ -413,6 +433,7 @@ ocmc_status ocmc_init(ocmc_ctx** out, int device, const ocmc_params* p)
     if (r == cudaSuccess) r = cudaMemset(c->d_stats, 0, (ST_COUNT + 1) * sizeof(unsigned long long));
     if (r == cudaSuccess) r = cudaEventCreate(&c->ev0);
     if (r == cudaSuccess) r = cudaEventCreate(&c->ev1);
+    if (r == cudaSuccess) r = cudaEventCreateWithFlags(&c->order, cudaEventDisableTiming);
     if (r != cudaSuccess) {
         ocmc_status s = cuda_fail(nullptr, r, "ocmc_init");
         ocmc_destroy(c);
@@ -430,7 +451,11 @@ ocmc_status ocmc_set_params(ocmc_ctx* c, const ocmc_params* p)
     bool phys = memcmp(&c->p, p, offsetof(ocmc_params, block_threads)) != 0;
     c->p = *p;
     if (phys) c->tables_valid = c->mat_tables_valid = false;
-    if (c->have_phantom && c->tally_B != p->n_batches) return ensure_tally(c);
+    if (c->have_phantom && c->tally_B != p->n_batches) {
+        CallOrder call(c, nullptr);
+        CK(call.error(), "order");
+        return ensure_tally(c, nullptr);
+    }
     return OCMC_OK;
 }
 
@@ -515,6 +540,8 @@ ocmc_status ocmc_create_phantom(ocmc_ctx* c, int nx, int ny, int nz, const float
     }
     CK(cudaSetDevice(c->device), "cudaSetDevice");
     if (c->last_stream || c->ran) cudaDeviceSynchronize();
+    CallOrder call(c, nullptr);
+    CK(call.error(), "order");
     c->bl_graph_valid = false;     // a captured beamlet launch holds the old phantom's geometry and pointers
     if (n != c->nvox) c->bl_sized = c->bl_ran = c->bl_counted = false;   // as its tallies hold the old voxels
     if (n != c->nvox) {
@@ -543,7 +570,7 @@ ocmc_status ocmc_create_phantom(ocmc_ctx* c, int nx, int ny, int nz, const float
         return OCMC_OK;
     }
     CK(cudaMemset(c->d_stats, 0, (ST_COUNT + 1) * sizeof(unsigned long long)), "stats reset");
-    return ensure_tally(c);
+    return ensure_tally(c, nullptr);
 }
 
 ocmc_status ocmc_set_source(ocmc_ctx* c, int particle, int n_bins, const float* edges, const float* weights, float fx,
@@ -597,6 +624,8 @@ ocmc_status ocmc_set_phase_space(ocmc_ctx* c, const ocmc_ps_particle* records, u
     if (!records || n == 0) return fail(c, OCMC_ERR_ARG, "need at least one record");
     static_assert(sizeof(ocmc_ps_particle) == sizeof(PsRec), "record layout");
     CK(cudaSetDevice(c->device), "cudaSetDevice");
+    CallOrder call(c, nullptr);
+    CK(call.error(), "order");
     if (n > c->ps_cap) {
         cudaDeviceSynchronize();
         CK(dalloc(&c->d_ps, (size_t)n), "phase-space allocation");
@@ -661,7 +690,9 @@ ocmc_status ocmc_run_range(ocmc_ctx* c, uint64_t first, uint64_t count, uint64_t
         return fail(c, OCMC_ERR_ARG, "voxel-crossing electron steps need the analytic source (not a phase space)");
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     CK(cudaSetDevice(c->device), "cudaSetDevice");
-    ocmc_status st = ensure_tally(c);
+    CallOrder call(c, s);
+    CK(call.error(), "order");
+    ocmc_status st = ensure_tally(c, s);
     if (st != OCMC_OK) return st;
     st = ensure_tables(c, s);
     if (st != OCMC_OK) return st;
@@ -754,7 +785,7 @@ ocmc_status ocmc_add_raw_tally(ocmc_ctx* c, const int64_t* in, int on_device, ui
     if (!c || !in) return fail(c, OCMC_ERR_ARG, "NULL argument");
     if (!c->have_phantom) return fail(c, OCMC_ERR_STATE, "no phantom");
     CK(cudaSetDevice(c->device), "cudaSetDevice");
-    ocmc_status st = ensure_tally(c);
+    ocmc_status st = ensure_tally(c, nullptr);
     if (st != OCMC_OK) return st;
     long long n = (long long)c->tally_B * c->nvox;
     const long long* src = reinterpret_cast<const long long*>(in);
@@ -787,7 +818,8 @@ ocmc_status ocmc_reset_tally(ocmc_ctx* c)
 {
     if (!c) return fail(c, OCMC_ERR_ARG, "ctx is NULL");
     CK(cudaSetDevice(c->device), "cudaSetDevice");
-    if (c->last_stream) CK(cudaStreamSynchronize(c->last_stream), "synchronize");   // the clears are on the default stream
+    CallOrder call(c, nullptr);
+    CK(call.error(), "order");
     if (c->d_tally) {
         CK(cudaMemset(c->d_tally, 0, sizeof(long long) * (size_t)c->tally_B * c->nvox), "tally reset");
         c->tally_zero = true;
@@ -844,7 +876,7 @@ ocmc_status ocmc_get_stats(ocmc_ctx* c, ocmc_stats* out)
     out->pair_mass = 2.0 * MC2 * (double)st[ST_PAIR];
     out->annih_mass = 2.0 * MC2 * (double)st[ST_ANNIH];
     if (c->d_tally) {
-        CK(launch_sum_tally(c->d_tally, (long long)c->tally_B * c->nvox, c->d_sum, c->last_stream), "tally sum");
+        CK(launch_sum_tally(c->d_tally, (long long)c->tally_B * c->nvox, c->d_sum, nullptr), "tally sum");
         unsigned long long sum = 0;
         CK(cudaMemcpy(&sum, c->d_sum, sizeof(sum), cudaMemcpyDeviceToHost), "tally sum");
         out->e_dep = (double)(long long)sum * S;
@@ -883,6 +915,7 @@ void ocmc_destroy(ocmc_ctx* c)
     if (c->bl_capture) cudaStreamDestroy(c->bl_capture);
     if (c->ev0) cudaEventDestroy(c->ev0);
     if (c->ev1) cudaEventDestroy(c->ev1);
+    if (c->order) cudaEventDestroy(c->order);
     delete c;
 }
 
@@ -925,6 +958,8 @@ ocmc_status ocmc_test_source(ocmc_ctx* c, uint64_t n_total, uint64_t first, uint
     if (!c || !out || count == 0 || first + count > n_total) return fail(c, OCMC_ERR_ARG, "bad arguments");
     if (!c->have_phantom || !c->have_source) return fail(c, OCMC_ERR_STATE, "need phantom and source");
     CK(cudaSetDevice(c->device), "cudaSetDevice");
+    CallOrder call(c, nullptr);
+    CK(call.error(), "order");
     TransportArgs a;
     fill_args(c, a);
     if (c->src_kind == 0) stratify(c, n_total, a.src);
@@ -947,6 +982,8 @@ ocmc_status ocmc_test_sample(ocmc_ctx* c, int kind, int m, float E, float aux, u
     m = c->slot_of[m];
     if (!c->have_phantom) return fail(c, OCMC_ERR_STATE, "need a phantom");
     CK(cudaSetDevice(c->device), "cudaSetDevice");
+    CallOrder call(c, nullptr);
+    CK(call.error(), "order");
     ocmc_status st = ensure_tables(c, nullptr);
     if (st != OCMC_OK) return st;
     TransportArgs a;
@@ -969,6 +1006,8 @@ ocmc_status ocmc_test_tables(ocmc_ctx* c, int m, const float* E, int n, float* o
     m = c->slot_of[m];
     if (!c->have_phantom) return fail(c, OCMC_ERR_STATE, "need a phantom");
     CK(cudaSetDevice(c->device), "cudaSetDevice");
+    CallOrder call(c, nullptr);
+    CK(call.error(), "order");
     ocmc_status st = ensure_tables(c, nullptr);
     if (st != OCMC_OK) return st;
     TransportArgs a;
@@ -992,6 +1031,8 @@ ocmc_status ocmc_test_csda(ocmc_ctx* c, int m, const float* T, const float* X, i
     m = c->slot_of[m];
     if (!c->have_phantom) return fail(c, OCMC_ERR_STATE, "need a phantom");
     CK(cudaSetDevice(c->device), "cudaSetDevice");
+    CallOrder call(c, nullptr);
+    CK(call.error(), "order");
     ocmc_status st = ensure_tables(c, nullptr);
     if (st != OCMC_OK) return st;
     TransportArgs a;

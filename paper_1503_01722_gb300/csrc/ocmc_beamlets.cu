@@ -31,10 +31,10 @@ cudaError_t realloc_dev(T** p, size_t n)
     return cudaMalloc(reinterpret_cast<void**>(p), std::max<size_t>(n, 1) * sizeof(T));
 }
 
-// Per-beamlet device records for the given history counts and table capacities.
+// Per-beamlet device records for the given history counts and table capacities, there once it returns.
 ocmc_status upload_beamlets(ocmc_ctx* c, const std::vector<unsigned long long>& counts,
                             const std::vector<unsigned long long>& caps, unsigned long long* total_hist,
-                            size_t* total_slots)
+                            size_t* total_slots, cudaStream_t s)
 {
     const int n = c->bl_n;
     std::vector<BeamletDev> dev(n);
@@ -62,11 +62,15 @@ ocmc_status upload_beamlets(ocmc_ctx* c, const std::vector<unsigned long long>& 
         off += caps[b];
     }
     prefix[n] = pre;
-    BCK(cudaMemcpy(c->d_bl, dev.data(), sizeof(BeamletDev) * n, cudaMemcpyHostToDevice), "beamlet upload");
-    BCK(cudaMemcpy(c->d_bl_prefix, prefix.data(), sizeof(unsigned long long) * (n + 1), cudaMemcpyHostToDevice),
-        "beamlet upload");
-    BCK(cudaMemcpy(c->d_bl_offs, offs.data(), sizeof(unsigned long long) * n, cudaMemcpyHostToDevice), "upload");
-    BCK(cudaMemcpy(c->d_bl_caps, capv.data(), sizeof(unsigned int) * n, cudaMemcpyHostToDevice), "upload");
+    cudaError_t e = cudaMemcpyAsync(c->d_bl, dev.data(), sizeof(BeamletDev) * n, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(c->d_bl_prefix, prefix.data(), sizeof(unsigned long long) * (n + 1), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(c->d_bl_offs, offs.data(), sizeof(unsigned long long) * n, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(c->d_bl_caps, capv.data(), sizeof(unsigned int) * n, cudaMemcpyHostToDevice, s);
+    const cudaError_t e2 = cudaStreamSynchronize(s);       // the vectors live until here
+    BCK(e != cudaSuccess ? e : e2, "beamlet upload");
     if (!c->bl_dense && off > c->bl_slots) {
         BCK(realloc_dev(&c->d_bl_keys, off), "beamlet table allocation");
         BCK(realloc_dev(&c->d_bl_vals, off), "beamlet table allocation");
@@ -189,6 +193,7 @@ ocmc_status size_tables(ocmc_ctx* c, uint64_t seed, cudaStream_t s)
         p2[b] = std::max<unsigned long long>(1, p1[b] / 4);
     }
     unsigned long long saved[ST_COUNT];
+    BCK(cudaStreamSynchronize(s), "synchronize");      // the copies of this function are on the default stream
     BCK(cudaMemcpy(saved, c->d_stats, sizeof(saved), cudaMemcpyDeviceToHost), "stats");
     for (int pass = 0; pass < 2; ++pass) {
         const std::vector<unsigned long long>& cnt = pass == 0 ? p2 : p1;
@@ -197,7 +202,7 @@ ocmc_status size_tables(ocmc_ctx* c, uint64_t seed, cudaStream_t s)
         for (int attempt = 0;; ++attempt) {
             unsigned long long total;
             size_t slots;
-            ocmc_status st = upload_beamlets(c, cnt, caps, &total, &slots);
+            ocmc_status st = upload_beamlets(c, cnt, caps, &total, &slots, s);
             if (st != OCMC_OK) return st;
             TransportArgs a;
             int threads, blocks, nreg;
@@ -215,6 +220,7 @@ ocmc_status size_tables(ocmc_ctx* c, uint64_t seed, cudaStream_t s)
             if (attempt >= 8) return ctx_fail(c, OCMC_ERR_OVERFLOW, "beamlet pilot tables keep overflowing");
         }
         BCK(launch_bl_count(c->d_bl_keys, nullptr, c->d_bl_offs, c->d_bl_caps, n, c->d_bl_nnz, s), "footprint count");
+        BCK(cudaStreamSynchronize(s), "footprint count");
         BCK(cudaMemcpy(pass == 0 ? nnz2.data() : nnz1.data(), c->d_bl_nnz, sizeof(unsigned long long) * n,
                        cudaMemcpyDeviceToHost), "footprint count");
     }
@@ -236,13 +242,13 @@ ocmc_status size_tables(ocmc_ctx* c, uint64_t seed, cudaStream_t s)
 }
 
 // Capture {clear tables, clear flags, reset counter, transport} as one CUDA graph.
-ocmc_status capture_graph(ocmc_ctx* c, uint64_t seed)
+ocmc_status capture_graph(ocmc_ctx* c, uint64_t seed, cudaStream_t s)
 {
     std::vector<unsigned long long> counts(c->bl_n);
     for (int b = 0; b < c->bl_n; ++b) counts[b] = c->bl_list[b].n_histories;
     unsigned long long total;
     size_t slots;
-    ocmc_status st = upload_beamlets(c, counts, c->bl_cap, &total, &slots);
+    ocmc_status st = upload_beamlets(c, counts, c->bl_cap, &total, &slots, s);
     if (st != OCMC_OK) return st;
     TransportArgs a;
     int threads, blocks, nreg;
@@ -331,6 +337,8 @@ ocmc_status ocmc_run_beamlets(ocmc_ctx* c, uint64_t seed, void* stream)
         return ctx_fail(c, OCMC_ERR_ARG, "voxel-crossing electron steps are not available for beamlets");
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     BCK(cudaSetDevice(c->device), "cudaSetDevice");
+    CallOrder call(c, s);
+    BCK(call.error(), "order");
     ocmc_status st = ctx_ensure_tables(c, s);
     if (st != OCMC_OK) return st;
     if (!c->bl_sized) {
@@ -347,7 +355,7 @@ ocmc_status ocmc_run_beamlets(ocmc_ctx* c, uint64_t seed, void* stream)
     c->bl_counted = false;
     for (int attempt = 0;; ++attempt) {
         if (!c->bl_graph_valid || c->bl_graph_seed != seed) {
-            st = capture_graph(c, seed);
+            st = capture_graph(c, seed, s);
             if (st != OCMC_OK) return st;
         }
         BCK(cudaEventRecord(c->ev0, s), "event");

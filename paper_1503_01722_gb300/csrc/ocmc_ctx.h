@@ -65,6 +65,9 @@ struct ocmc_ctx {
     bool timed = false;
     cudaStream_t last_stream = nullptr;
     bool ran = false;
+    // order of the calls (CallOrder): behind the last call's work, unless that was on the default stream
+    cudaEvent_t order = nullptr;
+    bool order_default = true;
     // batched beamlets
     int bl_n = 0, bl_particle = 0, bl_bins = 0;
     std::vector<float> bl_edges, bl_weights;
@@ -105,6 +108,26 @@ struct ocmc_ctx {
 };
 
 namespace ocmc {
+// Lives while a call enqueues its work on stream s, and puts that work behind all that earlier calls enqueued
+// on any stream: every call uses the same tally, counters, stacks and tables, and a stream made without
+// cudaStreamNonBlocking is the only kind that waits for the default one by itself. The event is recorded at the
+// end of a call, so no handle of a caller's stream is needed later; calls on the default stream alone need no
+// event at all. A stream that is being captured is left alone (its order is that of the graph it becomes part of).
+class CallOrder {
+public:
+    CallOrder(ocmc_ctx* c, cudaStream_t s);
+    ~CallOrder();
+    CallOrder(const CallOrder&) = delete;
+    CallOrder& operator=(const CallOrder&) = delete;
+    cudaError_t error() const { return err_; }
+
+private:
+    ocmc_ctx* c_;
+    cudaStream_t s_;
+    bool capturing_ = false;
+    cudaError_t err_ = cudaSuccess;
+};
+
 // shared host helpers (ocmc_api.cu)
 ocmc_status ctx_fail(ocmc_ctx* c, ocmc_status s, const std::string& msg);
 ocmc_status ctx_cuda_fail(ocmc_ctx* c, cudaError_t e, const char* where);
