@@ -785,11 +785,13 @@ ocmc_status ocmc_add_raw_tally(ocmc_ctx* c, const int64_t* in, int on_device, ui
     if (!c || !in) return fail(c, OCMC_ERR_ARG, "NULL argument");
     if (!c->have_phantom) return fail(c, OCMC_ERR_STATE, "no phantom");
     CK(cudaSetDevice(c->device), "cudaSetDevice");
-    ocmc_status st = ensure_tally(c, nullptr);
+    cudaStream_t s = c->last_stream;
+    CallOrder call(c, s);                 // behind the clear, which may be on another stream
+    CK(call.error(), "order");
+    ocmc_status st = ensure_tally(c, s);
     if (st != OCMC_OK) return st;
     long long n = (long long)c->tally_B * c->nvox;
     const long long* src = reinterpret_cast<const long long*>(in);
-    cudaStream_t s = c->last_stream;
     if (c->tally_zero) {
         // onto a tally that nothing was added to since it was cleared: a copy, a third of the traffic
         CK(cudaMemcpyAsync(c->d_tally, in, sizeof(long long) * n, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s),
@@ -800,7 +802,7 @@ ocmc_status ocmc_add_raw_tally(ocmc_ctx* c, const int64_t* in, int on_device, ui
         long long* tmp = nullptr;
         if (!on_device) {
             CK(cudaMalloc(&tmp, sizeof(long long) * n), "allocation");
-            cudaError_t e = cudaMemcpy(tmp, in, sizeof(long long) * n, cudaMemcpyHostToDevice);
+            cudaError_t e = cudaMemcpyAsync(tmp, in, sizeof(long long) * n, cudaMemcpyHostToDevice, s);
             if (e != cudaSuccess) { cudaFree(tmp); return cuda_fail(c, e, "tally upload"); }
             src = tmp;
         }

@@ -134,3 +134,26 @@ def test_a_captured_run(ocmc, ph, ref):
         assert np.array_equal(e.raw_tally(), 2 * ref[1][0])
         e.run(SHORT, seed=12)                              # plain calls go on as before
         assert np.array_equal(e.raw_tally(), 3 * ref[1][0])
+
+
+@pytest.mark.parametrize("device", [False, True])
+@pytest.mark.parametrize("a,b", [(1, 1), (1, 0), (0, 1), (1, 2)])
+def test_tally_added_behind_a_clear(ocmc, ph, ref, streams, a, b, device):
+    """run, reset, add, run, add: the clear runs before the first addition, the runs before the additions."""
+    import torch
+    t = np.random.default_rng(5).integers(1, 1 << 40, (20,) + ph.density.shape, dtype=np.int64)
+    put = torch.from_numpy(t).cuda() if device else t
+    torch.cuda.synchronize()
+    with engine(ocmc, ph) as e:
+        for k in range(3):
+            e.run(LONG, seed=11, stream=streams[a])
+            if k == 1:
+                e.create_phantom(ph)                       # clears as well
+            else:
+                e.reset()
+            e.add_raw_tally(put, 0, 1000)
+            if k == 2:
+                assert np.array_equal(e.raw_tally(), t)
+            e.run(SHORT, seed=12, stream=streams[b])
+            e.add_raw_tally(put, 0, 1000)
+            assert np.array_equal(e.raw_tally(), 2 * t + ref[1][0])
