@@ -61,7 +61,7 @@ const char* check_params(const ocmc_params* p)
     if (!(p->d_maxs > 0.f && p->d_maxs <= 1e3f)) return "d_maxs must be in (0, 1000] cm";
     if (!(p->f_maxe > 0.f && p->f_maxe <= 0.5f)) return "f_maxe must be in (0, 0.5]";
     if (!(p->s_min >= 0.f && p->s_min <= 0.01f)) return "s_min must be in [0, 0.01] cm";
-    if (p->n_batches < 1 || p->n_batches > 1000) return "n_batches must be in [1, 1000]";
+    if (p->n_batches < 1 || p->n_batches > MAX_BATCHES) return "n_batches must be in [1, 1000]";
     if (p->flags < 0 || p->flags > 31) return "unknown flags";
     if (p->block_threads != 0 && (p->block_threads < 32 || p->block_threads > 1024 || p->block_threads % 32))
         return "block_threads must be 0 or a multiple of 32 in [32, 1024]";
@@ -285,15 +285,8 @@ ocmc_status ctx_finalize(ocmc_ctx* c, float* dose, float* sigma, bool want_sigma
     CK(call.error(), "order");
     std::vector<float> inv(c->tally_B);
     for (int b = 0; b < c->tally_B; ++b) inv[b] = c->nb[b] > 0 ? (float)(n / c->nb[b]) : 0.f;
-    if (c->tally_B > MAX_REG_BATCHES) {
-        if (c->invnb_cap < c->tally_B) {
-            CK(dalloc(&c->d_invnb, c->tally_B), "allocation");
-            c->invnb_cap = c->tally_B;
-        }
-        CK(cudaMemcpyAsync(c->d_invnb, inv.data(), sizeof(float) * c->tally_B, cudaMemcpyHostToDevice, s), "upload");
-    }
-    CK(launch_finalize(c->d_tally, c->d_density, c->tally_B, c->nvox, (double)c->dx * c->dy * c->dz, inv.data(), c->d_invnb,
-                       1.0 / n, dose ? dose : c->d_dose, want_sigma ? (sigma ? sigma : c->d_sigma) : nullptr, s),
+    CK(launch_finalize(c->d_tally, c->d_density, c->tally_B, c->nvox, (double)c->dx * c->dy * c->dz, inv.data(), 1.0 / n,
+                       dose ? dose : c->d_dose, want_sigma ? (sigma ? sigma : c->d_sigma) : nullptr, s),
        "finalize launch");
     return OCMC_OK;
 }
@@ -906,7 +899,7 @@ void ocmc_destroy(ocmc_ctx* c)
     cudaSetDevice(c->device);
     cudaDeviceSynchronize();
     dfree(&c->d_density); dfree(&c->d_material); dfree(&c->d_tally); dfree(&c->d_pool);
-    dfree(&c->d_stacks); dfree(&c->d_left); dfree(&c->d_dose); dfree(&c->d_sigma); dfree(&c->d_invnb);
+    dfree(&c->d_stacks); dfree(&c->d_left); dfree(&c->d_dose); dfree(&c->d_sigma);
     if (c->h_flags) cudaFreeHost(c->h_flags);
     dfree(&c->d_bl); dfree(&c->d_bl_prefix); dfree(&c->d_bl_offs); dfree(&c->d_bl_caps); dfree(&c->d_bl_nnz);
     dfree(&c->d_bl_over); dfree(&c->d_bl_keys); dfree(&c->d_bl_vals); dfree(&c->d_dense); dfree(&c->d_chunks);

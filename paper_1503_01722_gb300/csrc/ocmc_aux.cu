@@ -23,14 +23,15 @@ __device__ __forceinline__ float i64_to_f32(long long x)
 // outputs (FP64 here made this kernel 13x slower than its memory traffic on GB300's narrow FP64 pipe).
 // Bound by HBM: 8 B + 12 bytes a voxel. With NB > 0 a voxel's batches (B <= NB) are all loaded before
 // the first is used and stay in registers for the second sum; NB = 0 reads them twice, for any B.
+template <int N>
 struct BatchWeights {
-    float w[MAX_REG_BATCHES];
+    float w[N];
 };
 
 template <int NB>
 __global__ void __launch_bounds__(256) k_finalize(const long long* __restrict__ tally, const float* __restrict__ density, int B,
-                                                  long long nvox, float voxel_volume, const BatchWeights wk,
-                                                  const float* __restrict__ w_nb, float inv_n, float* dose, float* sigma)
+                                                  long long nvox, float voxel_volume,
+                                                  const __grid_constant__ BatchWeights<NB ? NB : MAX_BATCHES> wk, float inv_n, float* dose, float* sigma)
 {
     for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < nvox;
          v += (long long)gridDim.x * blockDim.x) {
@@ -69,7 +70,7 @@ __global__ void __launch_bounds__(256) k_finalize(const long long* __restrict__ 
                     for (int b = 0; b < NB; ++b)
                         if (b < B) add(q[b], wk.w[b]);
                 } else {
-                    for (int b = 0; b < B; ++b) add(tally[(long long)b * nvox + v], w_nb[b]);
+                    for (int b = 0; b < B; ++b) add(tally[(long long)b * nvox + v], wk.w[b]);
                 }
                 ss /= (float)B * (float)(B - 1);
             }
@@ -474,18 +475,25 @@ cudaError_t launch_sum_tally(const long long* tally, long long n, unsigned long 
     return cudaGetLastError();
 }
 
-cudaError_t launch_finalize(const long long* tally, const float* density, int B, long long nvox, double voxel_volume,
-                            const float* w_host, const float* w_nb, double inv_n, float* dose, float* sigma, cudaStream_t s)
+template <int NB>
+static void finalize_form(const long long* tally, const float* density, int B, long long nvox, float V, const float* w, float inv_n,
+                          float* dose, float* sigma, cudaStream_t s)
 {
     const unsigned blocks = (unsigned)std::max<long long>(1, std::min<long long>((nvox + 255) / 256, 152 * 16));
-    BatchWeights wk{};
-    for (int b = 0; b < B && b < MAX_REG_BATCHES; ++b) wk.w[b] = w_host[b];
+    BatchWeights<NB ? NB : MAX_BATCHES> wk{};
+    std::copy(w, w + B, wk.w);
+    k_finalize<NB><<<blocks, 256, 0, s>>>(tally, density, B, nvox, V, wk, inv_n, dose, sigma);
+}
+
+cudaError_t launch_finalize(const long long* tally, const float* density, int B, long long nvox, double voxel_volume,
+                            const float* w, double inv_n, float* dose, float* sigma, cudaStream_t s)
+{
+    if (B > MAX_BATCHES) return cudaErrorInvalidValue;
     const float V = (float)voxel_volume, in = (float)inv_n;
-    if (B <= 4) k_finalize<4><<<blocks, 256, 0, s>>>(tally, density, B, nvox, V, wk, w_nb, in, dose, sigma);
-    else if (B <= 12) k_finalize<12><<<blocks, 256, 0, s>>>(tally, density, B, nvox, V, wk, w_nb, in, dose, sigma);
-    else if (B <= MAX_REG_BATCHES)
-        k_finalize<MAX_REG_BATCHES><<<blocks, 256, 0, s>>>(tally, density, B, nvox, V, wk, w_nb, in, dose, sigma);
-    else k_finalize<0><<<blocks, 256, 0, s>>>(tally, density, B, nvox, V, wk, w_nb, in, dose, sigma);
+    if (B <= 4) finalize_form<4>(tally, density, B, nvox, V, w, in, dose, sigma, s);
+    else if (B <= 12) finalize_form<12>(tally, density, B, nvox, V, w, in, dose, sigma, s);
+    else if (B <= MAX_REG_BATCHES) finalize_form<MAX_REG_BATCHES>(tally, density, B, nvox, V, w, in, dose, sigma, s);
+    else finalize_form<0>(tally, density, B, nvox, V, w, in, dose, sigma, s);
     return cudaGetLastError();
 }
 

@@ -122,7 +122,7 @@ extern "C" ocmc_status ocmc_run_noalloc(int device, int nx, int ny, int nz, cons
     if (!(p.e_abs_e >= 1e-3f && p.e_abs_e <= 10.f && p.e_abs_g >= 1e-3f && p.e_abs_g <= 10.f &&
           p.w_cc >= 1e-3f && p.w_cc <= 10.f && p.w_cb >= 1e-3f && p.w_cb <= 10.f && p.d_maxs > 0.f &&
           p.f_maxe > 0.f && p.f_maxe <= 0.5f && p.s_min >= 0.f && p.s_min <= 0.01f && p.n_batches >= 1 &&
-          p.n_batches <= 1000 && p.flags >= 0 && p.flags <= 15))
+          p.n_batches <= MAX_BATCHES && p.flags >= 0 && p.flags <= 15))
         return M.fail(OCMC_ERR_ARG, "invalid transport parameters");
     if ((p.block_threads != 0 && (p.block_threads < 32 || p.block_threads > 1024 || p.block_threads % 32)) ||
         p.blocks_per_sm < 0 || p.blocks_per_sm > 32 ||
