@@ -1126,6 +1126,8 @@ ocmc_status ocmc_unet_test_layer(int device, int mode, int nx, int ny, int nz, i
         k_weights_bf16<<<grid_for(nw), 256>>>(w32, taps, cin, cout, m == CONV3, wf, wt);
         if (tcf) e = pack_tc(m, wf, cin, cout, pf, nullptr);
         if (tct && e == cudaSuccess) e = pack_tc(dgrad_mode(m), wt, cout, cin, pt, nullptr);
+        // the layers below are chained launches (ocmc_chain.cuh), which read their weights before they wait
+        if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
         ConvArgs a;
         std::memset(&a, 0, sizeof(a));
         a.mode = m; a.gin = gi; a.gout = go; a.in = Slice{dX, cin, 0}; a.out = Slice{dY, cout, 0};
