@@ -2,6 +2,11 @@
 // (training) kernels of 5 to 100 us, each waiting for the one before it. Launched as programmatic
 // dependents, a kernel's blocks are set up (barriers, tensor memory, weights) while the last blocks of the
 // kernel before it still run, and the launch itself costs the chain nothing.
+//
+// What a kernel of a chain writes is thus still being written while the next ones are resident. They read it
+// with ordinary loads, behind chain_wait: no __ldg and no const __restrict__ argument, which stand for data that
+// does not change while the kernel lives (and which the compiler may load ahead of the wait). Those are for the
+// caller's maps and the weights, which are complete before the chain starts.
 #pragma once
 #include <cuda_runtime.h>
 #include <utility>

@@ -97,8 +97,8 @@ __device__ __forceinline__ void unpack16(const Bf16x16& h, float f[16])
 // Head: o = x0 + sum_c h[v][c] w[c] + b. Inference (target null): out = o s. Training: out = the masked
 // error o - target / s over voxels of density >= 0.1, with the sum of its squares to acc[0] and the mask's
 // count to acc[1] (their derivative's factor 2 / count is applied by k_head_bwd).
-__global__ void __launch_bounds__(256) k_head_fwd(const __nv_bfloat16* __restrict__ h, const float* __restrict__ w,
-                                                  const float* __restrict__ b, const float* __restrict__ x0, long long n,
+__global__ void __launch_bounds__(256) k_head_fwd(const __nv_bfloat16* h, const float* __restrict__ w,
+                                                  const float* __restrict__ b, const float* x0, long long n,
                                                   const unsigned int* smax, const float* __restrict__ target,
                                                   const float* __restrict__ dens, float* __restrict__ out, double* acc)
 {
@@ -151,8 +151,8 @@ __global__ void __launch_bounds__(256) k_head_fwd(const __nv_bfloat16* __restric
 
 // head backward: g = err 2 / count, gh[v][c] = g w[c] (h > 0); partial sums of g h and g per block.
 // 16-byte loads and stores of a voxel's channels (175 us for 128^3 with two bytes at a time, now 26).
-__global__ void __launch_bounds__(256) k_head_bwd(const __nv_bfloat16* __restrict__ h, const float* __restrict__ w,
-                                                  const float* __restrict__ err, const double* acc, long long n,
+__global__ void __launch_bounds__(256) k_head_bwd(const __nv_bfloat16* h, const float* __restrict__ w,
+                                                  const float* err, const double* acc, long long n,
                                                   __nv_bfloat16* gh, float* part /* [gridDim.x][17] */)
 {
     chain_next();
@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(1024) k_sum_rows(const float* part, int parts,
 // columns, so that every load is a 128-byte segment and a block's reads are independent; identical order of
 // additions. Bound by reading the partials (33.6 MB of a 64 -> 64 layer: 28 us in the form above).
 // dst(j): where column j goes (the UP layers' gradients come out transposed).
-__global__ void __launch_bounds__(256) k_sum_rows4(const float4* __restrict__ part, int parts, long long m4,
+__global__ void __launch_bounds__(256) k_sum_rows4(const float4* part, int parts, long long m4,
                                                    float* __restrict__ out, int tn, int tc)
 {
     chain_next();
@@ -281,7 +281,7 @@ struct BiasSums {
     long long src[NBIAS], dst[NBIAS];      // offsets of the partials and of the sums
 };
 
-__global__ void __launch_bounds__(1024) k_sum_biases(const float* __restrict__ part, const BiasSums b, float* __restrict__ out)
+__global__ void __launch_bounds__(1024) k_sum_biases(const float* part, const BiasSums b, float* __restrict__ out)
 {
     chain_next();
     chain_wait();

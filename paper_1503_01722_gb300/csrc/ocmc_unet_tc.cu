@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_conv3_tc(const __grid_constan
                 if (s < TZ && inside && z0 + s < a.g.nz) {
                     const uint4* mk = reinterpret_cast<const uint4*>(a.mask + (vox0 + s * plane) * a.mask_stride + a.mask_c0 + n0);
 #pragma unroll
-                    for (int j = 0; j < MQ; ++j) m[j] = __ldg(mk + j);
+                    for (int j = 0; j < MQ; ++j) m[j] = mk[j];
                 }
             };
             if (a.mask) {
@@ -556,7 +556,7 @@ __global__ void __launch_bounds__(UP_THREADS, 1) k_up_tc(const __grid_constant__
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         if (a.mask && ok[k])
-                            mv[k][h] = __ldg(reinterpret_cast<const uint4*>(a.mask + vox[k] * a.mask_stride + a.mask_c0 + 16 * j) + h);
+                            mv[k][h] = reinterpret_cast<const uint4*>(a.mask + vox[k] * a.mask_stride + a.mask_c0 + 16 * j)[h];
                         if (a.accumulate && ok[k])
                             ov[k][h] = reinterpret_cast<const uint4*>(a.out.ptr + vox[k] * a.out.stride + a.out.c0 + 16 * j)[h];
                     }
@@ -666,7 +666,7 @@ struct DownCfg {
 };
 
 template <int CIN, int COUT>
-__global__ void __launch_bounds__(DOWN_THREADS, 1) k_down_tc(const TcArgs a, const __nv_bfloat16* __restrict__ in,
+__global__ void __launch_bounds__(DOWN_THREADS, 1) k_down_tc(const TcArgs a, const __nv_bfloat16* in,
                                                              int in_stride)
 {
     using C = DownCfg<CIN, COUT>;
@@ -775,7 +775,7 @@ __global__ void __launch_bounds__(DOWN_THREADS, 1) k_down_tc(const TcArgs a, con
                     const long long vox = ok ? ix + (long long)a.gfine.nx * (iy + (long long)a.gfine.ny * iz) : 0;
                     const uint4* src = reinterpret_cast<const uint4*>(in + vox * in_stride);
 #pragma unroll
-                    for (int g = 0; g < G; ++g) v[q][g] = ok ? __ldg(src + g) : make_uint4(0u, 0u, 0u, 0u);
+                    for (int g = 0; g < G; ++g) v[q][g] = ok ? src[g] : make_uint4(0u, 0u, 0u, 0u);
                 }
 #pragma unroll
                 for (int q = 0; q < PB; ++q)
