@@ -442,6 +442,9 @@ ocmc_status ocmc_set_params(ocmc_ctx* c, const ocmc_params* p)
     if (const char* m = check_params(p)) return fail(c, OCMC_ERR_ARG, m);
     CK(cudaSetDevice(c->device), "cudaSetDevice");
     bool phys = memcmp(&c->p, p, offsetof(ocmc_params, block_threads)) != 0;
+    // a captured beamlet launch holds the old parameters, and its tallies are of the kind the old scale chose
+    if (memcmp(&c->p, p, sizeof(*p)) != 0) c->bl_graph_valid = false;
+    if (c->p.beamlet_capacity_scale != p->beamlet_capacity_scale) c->bl_sized = false;
     c->p = *p;
     if (phys) c->tables_valid = c->mat_tables_valid = false;
     if (c->have_phantom && c->tally_B != p->n_batches) {

@@ -1,0 +1,57 @@
+"""A beamlet plan that stays while the context changes around it: parameters, phantoms, kinds of tally."""
+import numpy as np
+import pytest
+
+import ocmc_inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ocmc():
+    from paper_1503_01722_gb300 import build
+    build.build()
+    from paper_1503_01722_gb300 import ocmc as m
+    return m
+
+
+def phantom(seed=4, n=(32, 30, 28)):
+    return I.ct_like(n=n, voxel=tuple(24.0 / k for k in n), seed=seed)
+
+
+def plan(ph, count=6):
+    return I.beamlets(ph, n_beamlets=count, seed=5, log10_mean=3.3, log10_sd=0.3, lo=100, hi=20_000, offset=2.0)
+
+
+def lists(e):
+    return [a for item in e.beamlet_doses(raw=True) for a in item]
+
+
+def same(a, b):
+    return len(a) == len(b) and all(np.array_equal(x, y) for x, y in zip(a, b))
+
+
+@pytest.mark.parametrize("scale", [0.0, 1.0])             # dense tallies, hash tables
+@pytest.mark.parametrize("change", [{"e_abs_g": 0.05}, {"e_abs_e": 0.5}, {"w_cb": 0.05}, {"w_cc": 0.4}, {"d_maxs": 0.05},
+                                    {"f_maxe": 0.2}, {"flags": 8}, {"beamlet_capacity_scale": 2.0},
+                                    {"beamlet_capacity_scale": 0.0}, {"block_threads": 256, "refill_min": 20}])
+def test_changed_parameters_hold_for_the_next_run(ocmc, scale, change):
+    ph = phantom()
+    bl = plan(ph)
+    with ocmc.Engine(0, beamlet_capacity_scale=scale) as e:
+        e.create_phantom(ph)
+        e.set_beamlets(0, *I.spectrum_6mv(), bl)
+        e.run_beamlets(seed=3)
+        before = lists(e)
+        e.set_params(**change)
+        assert same(lists(e), before)                      # the last run's results stay
+        e.run_beamlets(seed=3)
+        got = lists(e)
+        now = e.params
+    with ocmc.Engine(0, params=now) as f:
+        f.create_phantom(ph)
+        f.set_beamlets(0, *I.spectrum_6mv(), bl)
+        f.run_beamlets(seed=3)
+        assert same(got, lists(f))
+    physics = not set(change) & {"beamlet_capacity_scale", "block_threads"}
+    assert same(got, before) != physics
