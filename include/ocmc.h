@@ -170,8 +170,9 @@ ocmc_status ocmc_set_materials(ocmc_ctx* ctx, int n, const ocmc_material* defs);
  * material_host: nx*ny*nz uint8, an index into the defined materials (by default 0 water,
  *   1 cortical bone (ICRP), 2 lung (ICRP); see ocmc_set_materials);
  * dx, dy, dz: voxel size in cm. The phantom occupies [0,nx*dx] x [0,ny*dy] x
- * [0,nz*dz]. 1 <= nx, ny, nz <= 1024. Copies the data (host pointers) and
- * resets the tally. Errors: OCMC_ERR_ARG for bad sizes or values. */
+ * [0,nz*dz]. 1 <= nx, ny, nz <= 1024. Copies the data (host pointers),
+ * resets the tally and drops the lists of a beamlet run (the beamlets stay).
+ * Errors: OCMC_ERR_ARG for bad sizes or values (nothing changes). */
 ocmc_status ocmc_create_phantom(ocmc_ctx* ctx, int nx, int ny, int nz,
                                 const float* density_host, const uint8_t* material_host,
                                 float dx, float dy, float dz);

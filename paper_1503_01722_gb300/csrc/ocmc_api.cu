@@ -539,7 +539,8 @@ ocmc_status ocmc_create_phantom(ocmc_ctx* c, int nx, int ny, int nz, const float
     CallOrder call(c, nullptr);
     CK(call.error(), "order");
     c->bl_graph_valid = false;     // a captured beamlet launch holds the old phantom's geometry and pointers
-    if (n != c->nvox) c->bl_sized = c->bl_ran = c->bl_counted = false;   // as its tallies hold the old voxels
+    c->bl_ran = c->bl_counted = false;     // as its tallies hold the old voxels' energies
+    if (n != c->nvox) c->bl_sized = false;
     if (n != c->nvox) {
         CK(dalloc(&c->d_density, n), "phantom allocation");
         CK(dalloc(&c->d_material, n), "phantom allocation");

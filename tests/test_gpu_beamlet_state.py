@@ -55,3 +55,32 @@ def test_changed_parameters_hold_for_the_next_run(ocmc, scale, change):
         assert same(got, lists(f))
     physics = not set(change) & {"beamlet_capacity_scale", "block_threads"}
     assert same(got, before) != physics
+
+
+@pytest.mark.parametrize("scale", [0.0, 1.0])
+@pytest.mark.parametrize("n", [(32, 30, 28), (30, 28, 32), (20, 21, 22)])    # the same grid, as many voxels, another number
+def test_a_new_phantom_drops_the_old_lists(ocmc, scale, n):
+    first, second = phantom(), phantom(seed=9, n=n)
+    bl = plan(first)
+    spec = I.spectrum_6mv()
+    with ocmc.Engine(0, beamlet_capacity_scale=scale) as e:
+        e.create_phantom(first)
+        e.set_beamlets(0, *spec, bl)
+        e.run_beamlets(seed=3)
+        before = lists(e)
+        with pytest.raises(ocmc.OcmcError):                # refused: nothing changes
+            e.create_phantom(density=second.density - 40.0, material=second.material, voxel=second.voxel)
+        assert same(lists(e), before)
+        e.create_phantom(second)
+        for call in (lambda: e.beamlet_doses(), lambda: e.beamlet_doses(raw=True), lambda: e.beamlet_dose(0)):
+            with pytest.raises(ocmc.OcmcError) as x:
+                call()
+            assert x.value.status == ocmc.ERR_STATE
+        assert ocmc.lib.ocmc_get_beamlet_entries(e._c, None, None, None, 1 << 40) == ocmc.ERR_STATE
+        e.run_beamlets(seed=3)
+        got = lists(e)
+    with ocmc.Engine(0, beamlet_capacity_scale=scale) as f:
+        f.create_phantom(second)
+        f.set_beamlets(0, *spec, bl)
+        f.run_beamlets(seed=3)
+        assert same(got, lists(f))
