@@ -409,7 +409,7 @@ ocmc_status ocmc_init(ocmc_ctx** out, int device, const ocmc_params* p)
         place(&c->t.mats, MAX_STAGED);
         place(&c->t.mc, MAX_STAGED);
         place(&c->t.elem, MAX_STAGED * MAX_ELEM);
-        place(&c->d_stats, ST_COUNT + 1);                          // the error flag behind them: one clear
+        place(&c->d_stats, ST_COUNT + 1);                          // the two error words behind them: one clear
         place(&c->d_counter, RUN_COUNTERS);
         place(&c->d_sum, 1);
     }
@@ -422,7 +422,8 @@ ocmc_status ocmc_init(ocmc_ctx** out, int device, const ocmc_params* p)
         c->t.n_mat = NMAT_DEFAULT;
     }
     if (r == cudaSuccess) r = cudaHostAlloc(reinterpret_cast<void**>(&c->h_flags), 2 * sizeof(int), cudaHostAllocDefault);
-    if (r == cudaSuccess) c->d_err = reinterpret_cast<int*>(c->d_stats + ST_COUNT);
+    if (r == cudaSuccess) c->d_bl_err = reinterpret_cast<int*>(c->d_stats + ST_COUNT);
+    if (r == cudaSuccess) c->d_err = c->d_bl_err + 1;
     if (r == cudaSuccess) r = cudaMemset(c->d_stats, 0, (ST_COUNT + 1) * sizeof(unsigned long long));
     if (r == cudaSuccess) r = cudaEventCreate(&c->ev0);
     if (r == cudaSuccess) r = cudaEventCreate(&c->ev1);

@@ -105,6 +105,7 @@ ocmc_status beamlet_args(ocmc_ctx* c, unsigned long long total, uint64_t seed, T
     a.n_beamlets = c->bl_n;
     a.bl_dense = c->bl_dense;
     if (c->bl_dense) a.tally = c->d_bl_tally;
+    a.err = c->d_bl_err;
     a.bl_keys = c->d_bl_keys;
     a.bl_vals = c->d_bl_vals;
     a.bl_overflow = c->d_bl_over;
@@ -138,8 +139,8 @@ cudaError_t enqueue_beamlets(ocmc_ctx* c, const TransportArgs& a, size_t slots, 
     }
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_bl_over, 0, sizeof(unsigned int) * c->bl_n, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_counter, 0, RUN_COUNTERS * sizeof(unsigned long long), s);
-    // a beamlet run replaces its tallies, so its statistics describe that run alone
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->d_stats, 0, sizeof(unsigned long long) * ST_COUNT, s);
+    // a beamlet run replaces its tallies, so its statistics and the error bits behind them describe that run alone
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->d_stats, 0, sizeof(unsigned long long) * ST_COUNT + sizeof(int), s);
     if (e == cudaSuccess) e = launch_transport(a, blocks, threads, transport_smem_bytes(c->t.n_mat), s, nreg);
     return e;
 }
@@ -225,7 +226,6 @@ ocmc_status size_tables(ocmc_ctx* c, uint64_t seed, cudaStream_t s)
                        cudaMemcpyDeviceToHost), "footprint count");
     }
     BCK(cudaMemcpy(c->d_stats, saved, sizeof(saved), cudaMemcpyHostToDevice), "stats");
-    BCK(cudaMemset(c->d_err, 0, sizeof(int)), "flags");
     const double scale = c->p.beamlet_capacity_scale > 0.f ? c->p.beamlet_capacity_scale : 1.0;
     c->bl_cap.resize(n);
     for (int b = 0; b < n; ++b) {
@@ -381,7 +381,7 @@ ocmc_status ocmc_run_beamlets(ocmc_ctx* c, uint64_t seed, void* stream)
     }
     c->bl_ran = true;
     int e = 0;
-    BCK(cudaMemcpy(&e, c->d_err, sizeof(int), cudaMemcpyDeviceToHost), "error flag");
+    BCK(cudaMemcpy(&e, c->d_bl_err, sizeof(int), cudaMemcpyDeviceToHost), "error flag");
     if (e & ERR_BOUNDS) return ctx_fail(c, OCMC_ERR_BOUNDS, "a bounds check failed (checks build)");
     if (e & ERR_OVERFLOW) return ctx_fail(c, OCMC_ERR_OVERFLOW, "a secondary stack overflowed");
     if (e & ERR_LIMIT) return ctx_fail(c, OCMC_ERR_TIMEOUT, "a particle hit the step or sampling limit");

@@ -50,7 +50,8 @@ struct ocmc_ctx {
     unsigned long long* d_stats = nullptr;
     unsigned long long* d_counter = nullptr;
     unsigned long long* d_sum = nullptr;
-    int* d_err = nullptr;           // behind d_stats
+    int* d_err = nullptr;           // error bits of the dose runs, behind d_bl_err
+    int* d_bl_err = nullptr;        // those of the last beamlet run, behind d_stats
     int* h_flags = nullptr;         // pinned: error bits on their way to the host (the run's, a network's)
     ocmc::PRec* d_stacks = nullptr;
     size_t stack_records = 0;

@@ -84,3 +84,36 @@ def test_a_new_phantom_drops_the_old_lists(ocmc, scale, n):
         f.set_beamlets(0, *spec, bl)
         f.run_beamlets(seed=3)
         assert same(got, lists(f))
+
+
+@pytest.mark.parametrize("scale", [0.0, 1.0])
+def test_errors_belong_to_the_run_that_made_them(ocmc, scale):
+    """Stacks of 64 records that are not switched on size overflow: reported by the dose of a dose run, or by a
+    beamlet run, and by nothing after it."""
+    ph = I.homogeneous((24, 24, 24), (0.5, 0.5, 0.5))
+    bl = plan(ph, 40)
+    narrow, wide = {"stack_capacity": 64, "switch_high": 1 << 20}, {"stack_capacity": 0, "switch_high": 0}
+
+    def overflows(call):
+        with pytest.raises(ocmc.OcmcError) as x:
+            call()
+        assert x.value.status == ocmc.ERR_OVERFLOW
+
+    with ocmc.Engine(0, beamlet_capacity_scale=scale, e_abs_e=0.02, e_abs_g=0.01) as e:
+        e.create_phantom(ph)
+        e.set_source(I.beam_on(ph, 0, I.mono(18.0), (4.0, 4.0), 100.0))
+        e.set_beamlets(0, *I.mono(18.0), bl)
+        e.set_params(**narrow)
+        e.run(400_000, seed=1)
+        overflows(e.dose)
+        e.set_params(**wide)
+        for seed in (3, 3, 4):                             # sized, replayed, another seed
+            e.run_beamlets(seed=seed)
+            assert e.stats()["dropped"] == 0
+        overflows(e.dose)                                  # the dose's error is still there
+        e.reset()
+        e.run(400_000, seed=1)
+        e.set_params(**narrow)
+        e.set_beamlets(0, *I.mono(18.0), [dict(b, n_histories=10_000) for b in bl])
+        overflows(lambda: e.run_beamlets(seed=3))
+        e.dose()
