@@ -791,8 +791,9 @@ ocmc_status ocmc_add_raw_tally(ocmc_ctx* c, const int64_t* in, int on_device, ui
     long long n = (long long)c->tally_B * c->nvox;
     const long long* src = reinterpret_cast<const long long*>(in);
     if (c->tally_zero) {
-        // onto a tally that nothing was added to since it was cleared: a copy, a third of the traffic
-        CK(cudaMemcpyAsync(c->d_tally, in, sizeof(long long) * n, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s),
+        // onto a tally that nothing was added to since it was cleared: a copy, a third of the traffic (from
+        // wherever `in` is: with on_device that is any memory that the adding kernel below could read)
+        CK(cudaMemcpyAsync(c->d_tally, in, sizeof(long long) * n, on_device ? cudaMemcpyDefault : cudaMemcpyHostToDevice, s),
            "tally upload");
         c->tally_zero = false;
         CK(cudaStreamSynchronize(s), "tally add");
