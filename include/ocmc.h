@@ -298,7 +298,8 @@ ocmc_status ocmc_set_beamlets(ocmc_ctx* ctx, int particle, int n_bins, const flo
 
 /* Transport every beamlet's histories with Philox key `seed` (replacing the
  * previous beamlet tallies). Each beamlet has a dense tally where all of them take
- * at most a quarter of the free device memory; otherwise, or when the parameters set
+ * at most a quarter of the free device memory (the context keeps that memory for
+ * later plans until one of them uses tables, or until it is destroyed); otherwise, or when the parameters set
  * beamlet_capacity_scale, the first call after ocmc_set_beamlets sizes a hash table
  * per beamlet from two pilot runs (distinct-voxel footprint at two history counts,
  * extrapolated as a power law). The first call captures the launch in a CUDA graph;

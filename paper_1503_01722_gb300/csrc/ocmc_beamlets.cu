@@ -183,6 +183,31 @@ bool dense_fits(ocmc_ctx* c)
     return true;
 }
 
+template <class T>
+void release(T** p, size_t* n)
+{
+    if (*p) cudaFree(*p);
+    *p = nullptr;
+    *n = 0;
+}
+
+// Chooses the kind of tally and gives back the memory of the other kind: both may be tens of GB, and a context
+// that has changed over would hold the larger share of a GPU that others allocate on too.
+void choose_tallies(ocmc_ctx* c)
+{
+    c->bl_dense = dense_fits(c);
+    c->bl_graph_valid = false;
+    size_t slots = 0;
+    if (c->bl_dense) {
+        release(&c->d_bl_keys, &slots);
+        release(&c->d_bl_vals, &c->bl_slots);
+    } else {
+        release(&c->d_bl_tally, &c->bl_tally_n);
+        release(&c->d_bl_offsets, &c->bl_offsets_n);
+        release(&c->d_bl_out, &c->bl_out_bytes);
+    }
+}
+
 ocmc_status size_tables(ocmc_ctx* c, uint64_t seed, cudaStream_t s)
 {
     const int n = c->bl_n;
@@ -341,9 +366,9 @@ ocmc_status ocmc_run_beamlets(ocmc_ctx* c, uint64_t seed, void* stream)
     BCK(call.error(), "order");
     ocmc_status st = ctx_ensure_tables(c, s);
     if (st != OCMC_OK) return st;
+    c->bl_ran = c->bl_counted = false;          // from here on the old tallies may be gone, also if this run fails
     if (!c->bl_sized) {
-        c->bl_dense = dense_fits(c);
-        c->bl_graph_valid = false;
+        choose_tallies(c);
         if (c->bl_dense) {
             c->bl_cap.assign(c->bl_n, 1);       // no tables
             c->bl_sized = true;
@@ -352,7 +377,6 @@ ocmc_status ocmc_run_beamlets(ocmc_ctx* c, uint64_t seed, void* stream)
             if (st != OCMC_OK) return st;
         }
     }
-    c->bl_counted = false;
     for (int attempt = 0;; ++attempt) {
         if (!c->bl_graph_valid || c->bl_graph_seed != seed) {
             st = capture_graph(c, seed, s);

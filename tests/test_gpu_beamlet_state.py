@@ -117,3 +117,27 @@ def test_errors_belong_to_the_run_that_made_them(ocmc, scale):
         e.set_beamlets(0, *I.mono(18.0), [dict(b, n_histories=10_000) for b in bl])
         overflows(lambda: e.run_beamlets(seed=3))
         e.dose()
+
+
+def test_memory_of_the_other_kind_is_given_back(ocmc):
+    import torch
+    ph = phantom(n=(128, 128, 96))
+    bl = I.beamlets(ph, n_beamlets=64, seed=5, log10_mean=3.3, log10_sd=0.3, lo=100, hi=20_000, offset=2.0)
+    dense = 8 * 64 * ph.density.size                       # 805 MB
+    spec = I.spectrum_6mv()
+
+    def used(e, scale):
+        e.set_params(beamlet_capacity_scale=scale)
+        e.set_beamlets(0, *spec, bl)
+        e.run_beamlets(seed=1)
+        r = lists(e)
+        return torch.cuda.mem_get_info()[0], r
+
+    with ocmc.Engine(0) as e:
+        e.create_phantom(ph)
+        free_dense, a = used(e, 0.0)
+        free_tables, b = used(e, 1.0)                      # tables of some 50 MB
+        free_again, c = used(e, 0.0)
+    assert same(a, b) and same(a, c)
+    assert free_tables - free_dense > 0.6 * dense
+    assert abs(free_again - free_dense) < 0.1 * dense
