@@ -85,6 +85,14 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
     }
 }
 
+// The same for a whole warp, with one answer for all its lanes: for waits in front of code that the warp runs
+// together (tensor-memory loads, shuffles, __syncwarp). A lane that left alone, on its own timeout or its own
+// look at *abort, would leave the others waiting for it; so a loop around this wait has no other way out.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort, uint64_t limit_ns)
+{
+    return __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, abort, limit_ns));
+}
+
 // ---- TMA ----
 __device__ __forceinline__ void tma_load_5d(void* dst, const void* tmap, int c0, int c1, int c2, int c3, int c4,
                                             uint64_t* bar)

@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_conv3_tc(const __grid_constan
         const int q = warp & 3;                       // the tensor-memory lane quarter of this warp
         const int row = 32 * q + lane;
         int lt = 0;
-        for (int tile = blockIdx.x; tile < a.ntiles && !*abort; tile += gridDim.x, ++lt) {
+        for (int tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x, ++lt) {
             const int acc = lt & 1, ua = lt >> 1;
             const int tx = tile % a.tiles_x, r = tile / a.tiles_x;
             const int x = tx * TX + (row & 7), y = (r % a.tiles_y) * TY + (row >> 3), z0 = (r / a.tiles_y) * TZ;
@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_conv3_tc(const __grid_constan
                 load_mask(m0, 0);
                 load_mask(m1, 1);
             }
-            if (!mbar_wait(&t_full[acc], ua & 1, abort, WAIT_NS)) break;
+            if (!mbar_wait_warp(&t_full[acc], ua & 1, abort, WAIT_NS)) break;
             fence_after_sync();
             // (with z-stacked taps output slice s is accumulator slice s + 2)
             const uint32_t tbase = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(acc * C::ASLICES * NSL) +
@@ -532,7 +532,7 @@ __global__ void __launch_bounds__(UP_THREADS, 1) k_up_tc(const __grid_constant__
         const int p0 = ((warp - 2) >> 2) * 4;
         const int row = 32 * q + lane;
         int it = 0;
-        for (int tile = blockIdx.x; tile < a.ntiles && !*abort; tile += gridDim.x, ++it) {
+        for (int tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x, ++it) {
             const int acc = it % C::NACC, ua = it / C::NACC;
             const int tx = tile % a.tiles_x, r = tile / a.tiles_x;
             const int x = tx * TX + (row & 7), y = (r % a.tiles_y) * TY + (row >> 3), z = r / a.tiles_y;
@@ -562,7 +562,7 @@ __global__ void __launch_bounds__(UP_THREADS, 1) k_up_tc(const __grid_constant__
                     }
             };
             load_extra(0);
-            if (!mbar_wait(&t_full[acc], ua & 1, abort, WAIT_NS)) break;
+            if (!mbar_wait_warp(&t_full[acc], ua & 1, abort, WAIT_NS)) break;
             fence_after_sync();
 #pragma unroll
             for (int j = 0; j < J; ++j) {
@@ -791,9 +791,9 @@ __global__ void __launch_bounds__(DOWN_THREADS, 1) k_down_tc(const TcArgs a, con
         const int q = warp & 3;                       // the tensor-memory lane quarter of this warp
         const int row = 32 * q + lane;
         int it = 0;
-        for (int tile = blockIdx.x; tile < a.ntiles && !*abort; tile += gridDim.x, ++it) {
+        for (int tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x, ++it) {
             const int acc = it & 1, ua = it >> 1;
-            if (!mbar_wait(&t_full[acc], ua & 1, abort, WAIT_NS)) break;
+            if (!mbar_wait_warp(&t_full[acc], ua & 1, abort, WAIT_NS)) break;
             fence_after_sync();
             const int tx = tile % a.tiles_x, r = tile / a.tiles_x;
             const int x = tx * TX + (row & 7), y = (r % a.tiles_y) * TY + (row >> 3), z = r / a.tiles_y;

@@ -215,9 +215,9 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
             float acc[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) acc[e] = 0.f;
-            for (long long i = 0; i < nrows && !*abort; ++i) {
+            for (long long i = 0; i < nrows; ++i) {
                 const int st = (int)(i % NS), u = (int)(i / NS);
-                if (!mbar_wait(&full[st], u & 1, abort, WG_WAIT_NS)) break;
+                if (!mbar_wait_warp(&full[st], u & 1, abort, WG_WAIT_NS)) break;
                 const uint8_t* sb = smem + (size_t)st * a.stage + in_bytes;
                 for (int p = row0; p < a.P; p += 128 / GN) {
                     const int piece = g ^ (((p * C::SPAN_B) >> 7) & (GN - 1));
@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
                 for (int e = 0; e < 8; ++e) o[e] = acc[e];
             }
         }
-        if (mbar_wait(done, 0, abort, WG_WAIT_NS)) {
+        if (mbar_wait_warp(done, 0, abort, WG_WAIT_NS)) {
             fence_after_sync();
             float* P = a.partial + (size_t)blockIdx.x * 27 * CIN * a.cout;
 #pragma unroll 1
