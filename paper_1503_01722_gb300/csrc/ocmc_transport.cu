@@ -1060,12 +1060,6 @@ cudaError_t launch_steps(const TransportArgs& a, int blocks, int threads, size_t
     if (nreg == 64) return launch_variant<BL, PS, 64, STEPS>(a, blocks, threads, smem, s);
     return launch_variant<BL, PS, 80, STEPS>(a, blocks, threads, smem, s);
 }
-
-template <int BL, bool PS>
-cudaError_t launch_source(const TransportArgs& a, int blocks, int threads, size_t smem, cudaStream_t s, int nreg)
-{
-    return launch_steps<PLAIN, BL, PS>(a, blocks, threads, smem, s, nreg);
-}
 }  // namespace
 
 bool transport_nreg_supported(int nreg) { return nreg == 56 || nreg == 64 || nreg == 80; }
@@ -1100,11 +1094,11 @@ static cudaError_t launch_one(const TransportArgs& a, int blocks, int threads, s
         return launch_steps<CROSS>(a, blocks, threads, smem, s, nreg);
     }
     if (a.beamlets)
-        return a.bl_dense ? launch_source<BEAMLETS_DENSE, false>(a, blocks, threads, smem, s, nreg)
-                          : launch_source<BEAMLETS_HASH, false>(a, blocks, threads, smem, s, nreg);
-    if (a.ps) return launch_source<ONE_BEAM, true>(a, blocks, threads, smem, s, nreg);
+        return a.bl_dense ? launch_steps<PLAIN, BEAMLETS_DENSE, false>(a, blocks, threads, smem, s, nreg)
+                          : launch_steps<PLAIN, BEAMLETS_HASH, false>(a, blocks, threads, smem, s, nreg);
+    if (a.ps) return launch_steps<PLAIN, ONE_BEAM, true>(a, blocks, threads, smem, s, nreg);
     if (a.held) return launch_steps<HELD>(a, blocks, threads, smem, s, nreg);
-    return launch_source<ONE_BEAM, false>(a, blocks, threads, smem, s, nreg);
+    return launch_steps<PLAIN, ONE_BEAM, false>(a, blocks, threads, smem, s, nreg);
 }
 
 cudaError_t launch_transport(const TransportArgs& args, int blocks, int threads, size_t smem, cudaStream_t s, int nreg)

@@ -196,33 +196,11 @@ __global__ void __launch_bounds__(256) k_head_bwd(const __nv_bfloat16* h, const 
     }
 }
 
-// Sum of `parts` rows of length m in a fixed order: thread (x, y) of a 32 x 32 block adds rows
-// [y L, (y + 1) L) of column j in order (loads unrolled, so many are in flight), then the 32
-// partial sums of the column are added in order of y.
-__global__ void __launch_bounds__(1024) k_sum_rows(const float* part, int parts, int m, float* out)
-{
-    __shared__ float sh[32][33];
-    const int j = blockIdx.x * 32 + threadIdx.x;
-    const int L = (parts + 31) / 32;
-    const int i0 = threadIdx.y * L, i1 = min(parts, i0 + L);
-    float s = 0.f;
-    if (j < m) {
-#pragma unroll 8
-        for (int i = i0; i < i1; ++i) s += part[(long long)i * m + j];
-    }
-    sh[threadIdx.y][threadIdx.x] = s;
-    __syncthreads();
-    if (threadIdx.y == 0 && j < m) {
-        float t = 0.f;
-        for (int y = 0; y < 32; ++y) t += sh[y][threadIdx.x];
-        out[j] = t;
-    }
-}
-
-// The same sums for rows of a multiple of four columns: 32 groups of consecutive parts by 8 threads of four
-// columns, so that every load is a 128-byte segment and a block's reads are independent; identical order of
-// additions. Bound by reading the partials (33.6 MB of a 64 -> 64 layer: 28 us in the form above).
-// dst(j): where column j goes (the UP layers' gradients come out transposed).
+// Sum of `parts` rows of 4 m4 columns in a fixed order: thread group y of 32 adds rows [y L, (y + 1) L) of its
+// columns in order, then a column's 32 partial sums are added in order of y. Eight threads of four columns a
+// group, so that every load is a 128-byte segment and a block's reads are independent. Bound by reading the
+// partials (33.6 MB of a 64 -> 64 layer: 28 us with 32 threads of one column a group).
+// With tc > 0, column (tap, n, c) of [taps][tn][tc] goes to (tap, c, n): the UP layers' gradients come out transposed.
 __global__ void __launch_bounds__(256) k_sum_rows4(const float4* part, int parts, long long m4,
                                                    float* __restrict__ out, int tn, int tc)
 {
@@ -252,7 +230,7 @@ __global__ void __launch_bounds__(256) k_sum_rows4(const float4* part, int parts
 #pragma unroll
             for (int k = 0; k < 32; ++k) t += reinterpret_cast<const float*>(&sh[k][c4])[e];
             long long o = col;
-            if (tc) {                      // column (tap, n, c) of [taps][tn][tc] goes to (tap, c, n)
+            if (tc) {
                 const int c = (int)(col % tc), n = (int)(col / tc % tn);
                 o = (col / ((long long)tn * tc) * tc + c) * tn + n;
             }
@@ -265,16 +243,13 @@ int sm_count();
 
 cudaError_t sum_rows(const float* part, int parts, long long m, float* out, cudaStream_t s, int tn = 0, int tc = 0)
 {
-    if (m % 4 == 0) {
-        return launch_chained(k_sum_rows4, dim3((unsigned)((m / 4 + 7) / 8)), dim3(256), 0, s,
-                              reinterpret_cast<const float4*>(part), parts, m / 4, out, tn, tc);
-    }
-    k_sum_rows<<<(unsigned)((m + 31) / 32), dim3(32, 32), 0, s>>>(part, parts, (int)m, out);
-    return cudaGetLastError();
+    if (m % 4) return cudaErrorInvalidValue;           // channels come in sixteens
+    return launch_chained(k_sum_rows4, dim3((unsigned)((m / 4 + 7) / 8)), dim3(256), 0, s,
+                          reinterpret_cast<const float4*>(part), parts, m / 4, out, tn, tc);
 }
 
 // Bias gradients of all layers (and the head's sums) from their partials in one launch: blockIdx.y is the
-// layer, its columns by blockIdx.x, summed as in k_sum_rows.
+// layer, its columns by blockIdx.x, summed as in k_sum_rows4 with one column a thread.
 constexpr int NBIAS = NLAYERS + 1;
 struct BiasSums {
     int parts[NBIAS], m[NBIAS];
