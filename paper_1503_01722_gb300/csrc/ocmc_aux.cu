@@ -22,7 +22,10 @@ __device__ __forceinline__ float i64_to_f32(long long x)
 // means D_b = tally_b / (2^28 rho_v V n_b). The integer sum is exact; the rest is FP32, like the
 // outputs (FP64 here made this kernel 13x slower than its memory traffic on GB300's narrow FP64 pipe).
 // Bound by HBM: 8 B + 12 bytes a voxel. With NB > 0 a voxel's batches (B <= NB) are all loaded before
-// the first is used and stay in registers for the second sum; NB = 0 reads them twice, for any B.
+// the first is used and stay in registers for the second sum; NB = 0 reads them twice, for any B. A form has room
+// for NB batches whatever B is, so the lines between them lie at what NB holds: a whole ocmc_get_dose on 120^3
+// (cold L2) takes 33 us with 4 batches in the form of 4 and 42 in that of 12, 55 with 12 in that of 12 and 66
+// in that of 24, 80 with 24 in that of 24 and 92 in the form that reads twice.
 template <int N>
 struct BatchWeights {
     float w[N];

@@ -161,11 +161,17 @@ ocmc_status read_overflow(ocmc_ctx* c, std::vector<unsigned int>& over)
 constexpr double BL_LOAD = 0.35;
 
 // Dense tallies for the current beamlets and phantom? A pencil beam's voxels lie together, so its dense
-// tally needs no probing and stays in L2 while it is hit (64 beamlets on a 128x128x96 grid: 11.8 ms a run
-// against 13.5 with hash tables and 4 ms of pilot runs to size them; 192 beamlets on 256x256x128: 46.5
-// against 61 ms), and its sparse list is a plain stream over it. It costs 8 bytes a voxel and beamlet to
-// clear and to read back, 2 ms each for 13 GB, so the tallies may take a quarter of the free memory;
-// beyond that, or when the caller scales the tables, hash tables.
+// tally needs no probing and stays in L2 while it is hit, and its sparse list is a plain stream over it. It
+// costs 8 bytes a voxel and beamlet to clear and to read back, so the tallies may take a quarter of the free
+// memory; beyond that, or when the caller scales the tables, hash tables. The line looks at memory alone: with
+// few histories a beamlet the clear makes a run longer, but the lists of tables, one scatter and two passes
+// over the grid a beamlet, cost more than that. Define, run and read all lists / run again, in ms, dense against
+// tables, 500 beamlets on 256x256x128 (34 GB):
+//   histories a beamlet     300          1000         1e4          1e5
+//   plan                    12.7, 57     14.5, 62     25, 77       89, 203
+//   run                     5.5, 1.5     6.3, 2.4     11.7, 9.7    67, 78
+// on 128x128x96: 5.0 and 35 for the plan, 2.2 and 1.6 for the run at 1000; 64 beamlets of 1000 on 256x256x128:
+// 2.9 and 10.7, 1.6 and 1.2.
 bool dense_fits(ocmc_ctx* c)
 {
     if (c->p.beamlet_capacity_scale > 0.f) return false;

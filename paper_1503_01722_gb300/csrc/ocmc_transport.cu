@@ -27,10 +27,9 @@
 // emits a particle (finish), 32-bit event counters (a 64-bit shared add is a loop per lane), the first
 // draws of a step taken straight from its random block, geometric crossings and post-hinge crossings
 // through one piece of code, no branches in the face distances and the rotation, and a scheduler that
-// is skipped while no lane and no stack needs it. Against the version before (88 KB of code, now 65):
-// 1e8 6 MV photons on the 120^3 slab 123.8 -> 102 ms, 5e6 electrons of 15 MeV on the half-slab
-// 50.3 -> 35.4 ms, 1.3e6 photons on a CT-like 128^3 phantom 3.7 -> 2.3 ms (k_chains, below), the same
-// tallies bit for bit.
+// is skipped while no lane and no stack needs it. 1e8 6 MV photons on the 120^3 slab take 96 ms, 1e7
+// electrons of 15 MeV on the half-slab 62.7; one copy of each kind of code, the refill thresholds
+// (REFILL_G), the held events (HELD) and k_chains each say below what they gave of that.
 //
 // Dose tally (Sec. 2.2.2): 64-bit fixed-point integer atomics (2^-28 MeV
 // units) into the tally of batch (history id mod B). Integer addition is
@@ -1029,8 +1028,12 @@ size_t transport_smem_bytes(int n_mat) { return smem_table_bytes(n_mat); }
 namespace {
 constexpr unsigned long long SRC_LANES = 28;
 // Histories a warp from which an electron beam's run holds its hard events: below, a run is the chain of
-// steps of its last particles, which waiting lengthens. With 4864 warps, without and with it: 5e4 histories
-// 0.71 and 0.74 ms, 1e5 1.68 and 1.73, 2e5 1.54 and 1.55, 3e5 3.17 and 3.19, 6e5 5.33 and 5.06, 1e6 8.13 and 7.70.
+// steps of its last particles, which waiting lengthens. 15 MeV with 4864 warps, without and with it, in ms:
+//   histories                          5e4   1e5   2e5   3e5   4e5   6e5   1e6    2e6
+//   water 61 x 61 x 60 at 0.5 cm       0.72  0.92  1.54  2.02  2.58  3.69  5.80  11.05
+//                                      0.74  0.95  1.50  1.96  2.42  3.38  5.24   9.85
+//   half-slab 120^3 at 0.25 cm         1.37  1.68  2.52  3.20  3.95  5.29  8.05  14.79
+//                                      1.41  1.74  2.56  3.14  3.77  5.05  7.50  13.64
 constexpr unsigned long long HELD_HISTORIES = 64;
 
 template <int BL, bool PS, int R, int STEPS = PLAIN>

@@ -339,7 +339,8 @@ class Engine:
 
     def beamlet_doses(self, raw=False):
         """Every beamlet's sparse dose, [(voxel indices int32, dose float32 MeV/g per history
-        [, raw int64])] in beamlet order: views of one block of host memory that all lists share."""
+        [, raw int64])] in beamlet order: views of one block of host memory that all lists share, pinned up
+        to PINNED_LISTS bytes. The block lives while any list does; copy the ones to keep for long."""
         import torch
         if self.shape is None:
             raise OcmcError(ERR_STATE, "no phantom")
