@@ -497,7 +497,23 @@ ocmc_status ocmc_get_beamlet_entries(ocmc_ctx* c, int32_t* idx, float* dose, int
     if (capacity < 0 || (size_t)capacity < total) return ctx_fail(c, OCMC_ERR_ARG, "capacity is below the number of entries");
     if (total == 0) return OCMC_OK;
     BCK(cudaSetDevice(c->device), "cudaSetDevice");
-    if (!c->bl_dense) {
+    cudaStream_t s = c->last_stream;
+    const size_t bytes = total * ((raw ? 8 : 0) + (idx ? 4 : 0) + (dose ? 4 : 0));
+    bool one_by_one = !c->bl_dense;
+    if (c->bl_dense && bytes > c->bl_out_bytes) {
+        release(&c->d_bl_out, &c->bl_out_bytes);
+        const cudaError_t e = cudaMalloc(&c->d_bl_out, bytes);
+        if (e == cudaSuccess) {
+            c->bl_out_bytes = bytes;
+        } else if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();                 // no room for all lists at once: one beamlet's after the other
+            c->d_bl_out = nullptr;
+            one_by_one = true;
+        } else {
+            return ctx_cuda_fail(c, e, "allocation");
+        }
+    }
+    if (one_by_one) {
         for (int b = 0; b < n; ++b) {
             int64_t k = 0;
             const unsigned long long o = c->bl_base[b];
@@ -506,15 +522,6 @@ ocmc_status ocmc_get_beamlet_entries(ocmc_ctx* c, int32_t* idx, float* dose, int
             if (st != OCMC_OK) return st;
         }
         return OCMC_OK;
-    }
-    cudaStream_t s = c->last_stream;
-    const size_t bytes = total * ((raw ? 8 : 0) + (idx ? 4 : 0) + (dose ? 4 : 0));
-    if (bytes > c->bl_out_bytes) {
-        if (c->d_bl_out) cudaFree(c->d_bl_out);
-        c->d_bl_out = nullptr;
-        c->bl_out_bytes = 0;
-        BCK(cudaMalloc(&c->d_bl_out, bytes), "allocation");
-        c->bl_out_bytes = bytes;
     }
     unsigned char* o = static_cast<unsigned char*>(c->d_bl_out);
     long long* o_raw = raw ? reinterpret_cast<long long*>(o) : nullptr;

@@ -349,9 +349,16 @@ class Engine:
         n = int(ptr[-1])
         size = n * (16 if raw else 8)
         # pinned, so that the copy runs at the link's rate and into memory that is already mapped (torch
-        # keeps and reuses the block once the lists are gone); pageable beyond PINNED_LISTS
-        mem = (torch.empty(max(size, 1), dtype=torch.uint8, pin_memory=True).numpy() if size <= PINNED_LISTS
-               else np.empty(size, np.uint8))
+        # keeps and reuses the block once the lists are gone); pageable beyond PINNED_LISTS and where the
+        # host does not pin that much
+        mem = None
+        if size <= PINNED_LISTS:
+            try:
+                mem = torch.empty(max(size, 1), dtype=torch.uint8, pin_memory=True).numpy()
+            except RuntimeError:
+                pass
+        if mem is None:
+            mem = np.empty(max(size, 1), np.uint8)
         r = mem[:8 * n].view(np.int64) if raw else None
         o = 8 * n if raw else 0
         idx, dose = mem[o:o + 4 * n].view(np.int32), mem[o + 4 * n:o + 8 * n].view(np.float32)

@@ -141,3 +141,23 @@ def test_memory_of_the_other_kind_is_given_back(ocmc):
     assert same(a, b) and same(a, c)
     assert free_tables - free_dense > 0.6 * dense
     assert abs(free_again - free_dense) < 0.1 * dense
+
+
+@pytest.mark.parametrize("raw", [False, True])
+def test_lists_where_the_host_does_not_pin(ocmc, monkeypatch, raw):
+    import torch
+    ph = phantom()
+    with ocmc.Engine(0) as e:
+        e.create_phantom(ph)
+        e.set_beamlets(0, *I.spectrum_6mv(), plan(ph))
+        e.run_beamlets(seed=1)
+        ref = [a for item in e.beamlet_doses(raw=raw) for a in item]
+        empty = torch.empty
+
+        def refuse(*a, **k):
+            if k.get("pin_memory"):
+                raise RuntimeError("CUDA error: out of memory")
+            return empty(*a, **k)
+
+        monkeypatch.setattr(torch, "empty", refuse)
+        assert same([a for item in e.beamlet_doses(raw=raw) for a in item], ref)
