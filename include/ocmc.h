@@ -172,7 +172,8 @@ ocmc_status ocmc_set_materials(ocmc_ctx* ctx, int n, const ocmc_material* defs);
  * dx, dy, dz: voxel size in cm. The phantom occupies [0,nx*dx] x [0,ny*dy] x
  * [0,nz*dz]. 1 <= nx, ny, nz <= 1024. Copies the data (host pointers),
  * resets the tally and drops the lists of a beamlet run (the beamlets stay).
- * Errors: OCMC_ERR_ARG for bad sizes or values (nothing changes). */
+ * Errors: OCMC_ERR_ARG for bad sizes or values (nothing changes), OCMC_ERR_OOM
+ * (there is no phantom then). */
 ocmc_status ocmc_create_phantom(ocmc_ctx* ctx, int nx, int ny, int nz,
                                 const float* density_host, const uint8_t* material_host,
                                 float dx, float dy, float dz);

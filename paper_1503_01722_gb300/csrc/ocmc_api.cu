@@ -26,8 +26,10 @@ ocmc_status fail(ocmc_ctx* c, ocmc_status s, const std::string& msg)
     return s;
 }
 
+// (the error is this call's alone: the next launch's check must not find it again)
 ocmc_status cuda_fail(ocmc_ctx* c, cudaError_t e, const char* where)
 {
+    cudaGetLastError();
     std::string m = std::string(where) + ": " + cudaGetErrorString(e);
     return fail(c, e == cudaErrorMemoryAllocation ? OCMC_ERR_OOM : OCMC_ERR_CUDA, m);
 }
@@ -541,13 +543,15 @@ ocmc_status ocmc_create_phantom(ocmc_ctx* c, int nx, int ny, int nz, const float
     CK(call.error(), "order");
     c->bl_graph_valid = false;     // a captured beamlet launch holds the old phantom's geometry and pointers
     c->bl_ran = c->bl_counted = false;     // as its tallies hold the old voxels' energies
-    if (n != c->nvox) c->bl_sized = false;
     if (n != c->nvox) {
+        c->bl_sized = false;
+        c->have_phantom = false;           // none, until every buffer has its size
+        c->nvox = 0;
+        dfree(&c->d_tally);
         CK(dalloc(&c->d_density, n), "phantom allocation");
         CK(dalloc(&c->d_material, n), "phantom allocation");
         CK(dalloc(&c->d_dose, n), "dose allocation");
         CK(dalloc(&c->d_sigma, n), "dose allocation");
-        dfree(&c->d_tally);
     }
     c->nx = nx; c->ny = ny; c->nz = nz; c->nvox = n;
     c->dx = dx; c->dy = dy; c->dz = dz;
@@ -568,7 +572,9 @@ ocmc_status ocmc_create_phantom(ocmc_ctx* c, int nx, int ny, int nz, const float
         return OCMC_OK;
     }
     CK(cudaMemset(c->d_stats, 0, (ST_COUNT + 1) * sizeof(unsigned long long)), "stats reset");
-    return ensure_tally(c, nullptr);
+    const ocmc_status st = ensure_tally(c, nullptr);
+    c->have_phantom = st == OCMC_OK;
+    return st;
 }
 
 ocmc_status ocmc_set_source(ocmc_ctx* c, int particle, int n_bins, const float* edges, const float* weights, float fx,
@@ -626,6 +632,8 @@ ocmc_status ocmc_set_phase_space(ocmc_ctx* c, const ocmc_ps_particle* records, u
     CK(call.error(), "order");
     if (n > c->ps_cap) {
         cudaDeviceSynchronize();
+        c->ps_cap = 0;
+        if (c->src_kind == 1) c->have_source = false;      // none, until the new records are there
         CK(dalloc(&c->d_ps, (size_t)n), "phase-space allocation");
         c->ps_cap = n;
     }

@@ -72,6 +72,7 @@ ocmc_status upload_beamlets(ocmc_ctx* c, const std::vector<unsigned long long>& 
     const cudaError_t e2 = cudaStreamSynchronize(s);       // the vectors live until here
     BCK(e != cudaSuccess ? e : e2, "beamlet upload");
     if (!c->bl_dense && off > c->bl_slots) {
+        c->bl_slots = 0;
         BCK(realloc_dev(&c->d_bl_keys, off), "beamlet table allocation");
         BCK(realloc_dev(&c->d_bl_vals, off), "beamlet table allocation");
         c->bl_slots = off;
@@ -337,7 +338,9 @@ ocmc_status ocmc_set_beamlets(ocmc_ctx* c, int particle, int n_bins, const float
     }
     BCK(cudaSetDevice(c->device), "cudaSetDevice");
     if (c->ran || c->bl_ran) cudaDeviceSynchronize();
+    c->bl_sized = c->bl_graph_valid = c->bl_ran = false;
     if (n_beamlets != c->bl_n) {
+        c->bl_n = 0;                       // none, until every buffer has its size
         BCK(realloc_dev(&c->d_bl, n_beamlets), "allocation");
         BCK(realloc_dev(&c->d_bl_prefix, n_beamlets + 1), "allocation");
         BCK(realloc_dev(&c->d_bl_offs, n_beamlets), "allocation");
@@ -353,9 +356,6 @@ ocmc_status ocmc_set_beamlets(ocmc_ctx* c, int particle, int n_bins, const float
     c->bl_edges.assign(edges, edges + n_bins + 1);
     c->bl_weights.assign(weights, weights + n_bins);
     c->bl_list.assign(list, list + n_beamlets);
-    c->bl_sized = false;
-    c->bl_graph_valid = false;
-    c->bl_ran = false;
     return OCMC_OK;
 }
 

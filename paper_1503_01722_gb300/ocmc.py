@@ -223,9 +223,11 @@ class Engine:
         d = np.ascontiguousarray(density, np.float32)
         m = np.ascontiguousarray(material, np.uint8)
         nz, ny, nx = d.shape
-        self._check(lib.ocmc_create_phantom(self._c, nx, ny, nz, C.c_void_p(d.ctypes.data),
-                                            C.c_void_p(m.ctypes.data), *map(float, voxel)))
-        self.shape = (nz, ny, nx)
+        status = lib.ocmc_create_phantom(self._c, nx, ny, nz, C.c_void_p(d.ctypes.data),
+                                         C.c_void_p(m.ctypes.data), *map(float, voxel))
+        if status != ERR_ARG:              # refused values leave the phantom that was there
+            self.shape = (nz, ny, nx) if status == OK else None
+        self._check(status)
 
     def set_source(self, beam=None, *, particle=None, edges=None, weights=None, field=None, ssd=None,
                    iso=None, direction=None):
@@ -275,6 +277,8 @@ class Engine:
             ps = _ptr(s)[0] if s is not None else None
             self._check(lib.ocmc_get_dose(self._c, pd, ps, dev))
             return d, s
+        if self.shape is None:
+            raise OcmcError(ERR_STATE, "no phantom")
         d = np.empty(self.shape, np.float32)
         s = np.empty(self.shape, np.float32) if sigma else None
         self._check(lib.ocmc_get_dose(self._c, C.c_void_p(d.ctypes.data),
@@ -288,6 +292,8 @@ class Engine:
             p, dev = _ptr(out)
             self._check(lib.ocmc_get_raw_tally(self._c, p, dev))
             return out
+        if self.shape is None:
+            raise OcmcError(ERR_STATE, "no phantom")
         t = np.empty((B.value,) + self.shape, np.int64)
         self._check(lib.ocmc_get_raw_tally(self._c, C.c_void_p(t.ctypes.data), 0))
         return t
