@@ -257,7 +257,8 @@ ocmc_status size_tables(ocmc_ctx* c, uint64_t seed, cudaStream_t s)
         BCK(cudaMemcpy(pass == 0 ? nnz2.data() : nnz1.data(), c->d_bl_nnz, sizeof(unsigned long long) * n,
                        cudaMemcpyDeviceToHost), "footprint count");
     }
-    BCK(cudaMemcpy(c->d_stats, saved, sizeof(saved), cudaMemcpyHostToDevice), "stats");
+    BCK(cudaMemcpyAsync(c->d_stats, saved, sizeof(saved), cudaMemcpyHostToDevice, s), "stats");
+    BCK(cudaStreamSynchronize(s), "stats");
     const double scale = c->p.beamlet_capacity_scale > 0.f ? c->p.beamlet_capacity_scale : 1.0;
     c->bl_cap.resize(n);
     for (int b = 0; b < n; ++b) {
